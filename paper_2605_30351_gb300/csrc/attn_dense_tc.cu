@@ -6,11 +6,15 @@
 // head (one TMEM lane each) and walks that head's keys in blocks of 128;
 // CTA pairs (consecutive token tiles of the same head) share each key/value
 // tile through TMA multicast.
-//   warp 0     TMA producer: K_h and V_h tiles [128 keys x d_h] (SW128)
-//   warp 1     TMEM allocation; one lane issues S = Q K^T (Q read from TMEM)
-//   warp 6     one lane issues O += P V (P read from TMEM, V MN-major)
+//   warp 0     TMA producer: K_h and V_h tiles [128 keys x d_h] (SW128) in turn
+//   warp 1     TMEM allocation; issues S = Q K^T (Q read from TMEM)
+//   warp 6     issues O += P V (P read from TMEM, V MN-major)
 //   warps 2-5  load Q into TMEM, online softmax, O / l as bf16
 // TMEM columns: S [0,128) P [128,192) O [192,192+d_h) Q [192+d_h, +d_h/2).
+// A block's softmax (~1200 cycles) outlasts its MMAs (1024 at d_h = 128) and
+// bounds the kernel once its keys arrive in time: Wan shape, 630 -> 550 us
+// (1495 -> 1710 TFLOP/s) with warp-uniform issue, the early rescale vote and
+// K and V as separate ring entries.
 #include <cmath>
 
 #include "internal.h"
@@ -26,11 +30,14 @@ constexpr float kRescaleLog2 = 8.0f;
 
 template <int DH>
 struct DenseShape {
-  static constexpr int kHalf = kBN * DH * 2;        // one K or V tile
-  static constexpr int kTileBytes = 2 * kHalf;      // K then V
+  // K and V tiles are ring entries of their own, K(j) and V(j) in turn: K is
+  // released when the scores are done, a softmax and a PV before V, and its
+  // place is loaded ahead (with [K | V] stages of 64 KB the score issuer waited
+  // 372 of a block's 1475 cycles for its keys)
+  static constexpr int kTileBytes = kBN * DH * 2;
   static constexpr int kBarBytes = 256;
   static constexpr int kFit = (232448 - 1024 - kBarBytes) / kTileBytes;
-  static constexpr int kStages = kFit > 4 ? 4 : kFit;
+  static constexpr int kStages = kFit > 8 ? 8 : kFit;
   static constexpr int kSmemBytes = 1024 + kTileBytes * kStages + kBarBytes;
   static constexpr int kTmemS = 0, kTmemP = kBN, kTmemO = kBN + kBN / 2, kTmemQ = kTmemO + DH;
   static constexpr uint32_t kTmemCols = 512;
@@ -38,7 +45,7 @@ struct DenseShape {
   static constexpr uint32_t kIdescPV = idesc_bf16_f32(kBM, DH, false, true);
   static_assert(DH % 64 == 0 && DH <= 256, "head_dim: multiple of 64 up to 256");
   static_assert(kTmemQ + DH / 2 <= 512, "TMEM budget");
-  static_assert(kStages >= 2, "smem");
+  static_assert(kStages >= 4, "smem");
 };
 
 struct DenseKParams {
@@ -79,14 +86,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   const WaitCtx wc{abort_flag, p.status};
 
   if (threadIdx.x == 0) {
-    mbar_init(q_ready, kBM);
+    mbar_init(q_ready, 4);  // one arrival per softmax warp, and so below
     for (int s = 0; s < NST; ++s) {
       mbar_init(&kv_full[s], 1);
       mbar_init(&kv_empty[s], 2);  // both CTAs of the pair read every tile
     }
     mbar_init(s_full, 1);
-    mbar_init(s_free, kBM);
-    mbar_init(p_full, kBM);
+    mbar_init(s_free, 4);
+    mbar_init(p_full, 4);
     mbar_init(pv_done, 1);
     mbar_init(&mma_drain[0], 1);
     mbar_init(&mma_drain[1], 1);
@@ -109,84 +116,75 @@ __global__ void __launch_bounds__(kThreads, 1)
       tma_prefetch_desc(&tm_k);
       tma_prefetch_desc(&tm_v);
       int issued = 0;
-      for (int j = 0; j < nblk; ++j) {
-        const int st = j % NST;
-        if (j >= NST && !mbar_wait(&kv_empty[st], ((j / NST) - 1) & 1, wc)) break;
+      for (int e = 0; e < 2 * nblk; ++e) {
+        const int st = e % NST;
+        if (e >= NST && !mbar_wait(&kv_empty[st], ((e / NST) - 1) & 1, wc)) break;
         uint8_t* kv = smem + st * S::kTileBytes;
         mbar_arrive_expect_tx(&kv_full[st], S::kTileBytes);
-        // 2*DH/64 boxes of [128 keys x 64]: K boxes then V boxes, alternated across the pair
-        for (int bx = crank; bx < 2 * (DH / 64); bx += 2) {
-          if (bx < DH / 64)
-            tma_load_3d_mc(kv + bx * 16384, &tm_k, &kv_full[st], bx * 64, j * kBN, bh, kPair);
-          else
-            tma_load_3d_mc(kv + S::kHalf + (bx - DH / 64) * 16384, &tm_v, &kv_full[st],
-                           (bx - DH / 64) * 64, j * kBN, bh, kPair);
-        }
-        issued = j + 1;
+        // DH/64 boxes of [128 keys x 64], alternated across the pair
+        for (int bx = crank; bx < DH / 64; bx += 2)
+          tma_load_3d_mc(kv + bx * 16384, (e & 1) ? &tm_v : &tm_k, &kv_full[st], bx * 64,
+                         (e >> 1) * kBN, bh, kPair);
+        issued = e + 1;
       }
-      for (int st = 0; st < NST && st < nblk && !*abort_flag; ++st)
-        mbar_wait(&kv_empty[st], (((nblk - st + NST - 1) / NST) - 1) & 1, wc);
+      for (int u = 2 * nblk > NST ? 2 * nblk - NST : 0; u < 2 * nblk && !*abort_flag; ++u)
+        mbar_wait(&kv_empty[u % NST], (u / NST) & 1, wc);
       if (*abort_flag)
         for (int u = issued > NST ? issued - NST : 0; u < issued; ++u)
           mbar_wait_drain(&kv_full[u % NST], (u / NST) & 1, p.status);
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      bool ok = mbar_wait(q_ready, 0, wc);
+    // the whole warp walks the loop; one lane issues (see elect_one)
+    bool ok = mbar_wait_warp(q_ready, 0, wc);
+    const uint64_t kd = sdesc(smem_u32(smem), 16, 1024, kSw128);
+    for (int j = 0; ok && j < nblk; ++j) {
+      const int e = 2 * j, st = e % NST;
+      ok = (j == 0 || mbar_wait_warp(s_free, (j - 1) & 1, wc)) &&
+           mbar_wait_warp(&kv_full[st], (e / NST) & 1, wc);
+      if (!ok) break;
       tc_fence_after();
-      for (int j = 0; ok && j < nblk; ++j) {
-        if (j >= 1 && !mbar_wait(s_free, (j - 1) & 1, wc)) {
-          ok = false;
-          break;
-        }
-        const int st = j % NST;
-        if (!mbar_wait(&kv_full[st], (j / NST) & 1, wc)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t ka = smem_u32(smem) + st * S::kTileBytes;
+      if (elect_one()) {
+        const uint64_t ko = static_cast<uint64_t>(st * (S::kTileBytes >> 4));
 #pragma unroll
-        for (int cb = 0; cb < DH / 64; ++cb)
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            umma_ts(tmem + S::kTmemS, tmem + S::kTmemQ + (cb * 4 + k) * 8,
-                    sdesc(ka + cb * 16384 + k * 32, 16, 1024, kSw128), S::kIdescQK,
-                    (cb | k) != 0 ? 1u : 0u);
+        for (int k = 0; k < DH / 16; ++k)
+          umma_ts(tmem + S::kTmemS, tmem + S::kTmemQ + k * 8,
+                  kd + ko + (((k >> 2) * 16384 + (k & 3) * 32) >> 4), S::kIdescQK,
+                  k != 0 ? 1u : 0u);
         umma_commit(s_full);
+        umma_commit_mc(&kv_empty[st], kPair);
       }
-      if (!ok) {
-        umma_commit(&mma_drain[0]);
-        mbar_wait_drain(&mma_drain[0], 0, p.status);
-      }
+      __syncwarp();
     }
-    __syncwarp();
+    if (!ok) {
+      if (elect_one()) umma_commit(&mma_drain[0]);
+      __syncwarp();
+      mbar_wait_drain(&mma_drain[0], 0, p.status);
+    }
   } else if (warp == 6) {
-    if (lane == 0) {
-      bool ok = true;
-      for (int i = 0; ok && i < nblk; ++i) {
-        if (!mbar_wait(p_full, i & 1, wc)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const int st = i % NST;
-        const uint32_t va = smem_u32(smem) + st * S::kTileBytes + S::kHalf;
+    bool ok = true;
+    const uint64_t vd = sdesc(smem_u32(smem), 16384, 1024, kSw128);
+    for (int i = 0; ok && i < nblk; ++i) {
+      const int e = 2 * i + 1, st = e % NST;
+      ok = mbar_wait_warp(&kv_full[st], (e / NST) & 1, wc) && mbar_wait_warp(p_full, i & 1, wc);
+      if (!ok) break;
+      tc_fence_after();
+      if (elect_one()) {
+        const uint64_t vo = static_cast<uint64_t>(st * (S::kTileBytes >> 4));
 #pragma unroll
         for (int s = 0; s < kBN / 16; ++s)
-          umma_ts(tmem + S::kTmemO, tmem + S::kTmemP + s * 8,
-                  sdesc(va + s * 2048, 16384, 1024, kSw128), S::kIdescPV,
-                  (i > 0 || s > 0) ? 1u : 0u);
+          umma_ts(tmem + S::kTmemO, tmem + S::kTmemP + s * 8, vd + vo + s * (2048 >> 4),
+                  S::kIdescPV, (i > 0 || s > 0) ? 1u : 0u);
         umma_commit_mc(&kv_empty[st], kPair);
         umma_commit(pv_done);
       }
-      if (!ok) {
-        umma_commit(&mma_drain[1]);
-        mbar_wait_drain(&mma_drain[1], 0, p.status);
-      }
+      __syncwarp();
     }
-    __syncwarp();
+    if (!ok) {
+      if (elect_one()) umma_commit(&mma_drain[1]);
+      __syncwarp();
+      mbar_wait_drain(&mma_drain[1], 0, p.status);
+    }
   } else {
     const int quarter = warp & 3;
     const int r = quarter * 32 + lane;
@@ -211,12 +209,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       tmem_wait_st();
       tc_fence_before();
-      mbar_arrive(q_ready);
+      mbar_arrive_warp(q_ready);
     }
     float m_run = -INFINITY, l_run = 0.f;
     bool ok = true;
+    bool s_now = false;  // a poll has seen the next block's scores
     for (int j = 0; j < nblk; ++j) {
-      if (!mbar_wait(s_full, j & 1, wc)) {
+      if (!s_now && !mbar_wait(s_full, j & 1, wc)) {
         ok = false;
         break;
       }
@@ -227,8 +226,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_ld32(tmem + t_lane + S::kTmemS + c * 32,
                   *reinterpret_cast<uint32_t(*)[32]>(&sr[c * 32]));
       tmem_wait_ld();
-      tc_fence_before();
-      mbar_arrive(s_free);
       float sv[kBN];
 #pragma unroll
       for (int c = 0; c < kBN; ++c) sv[c] = __uint_as_float(sr[c]);
@@ -253,17 +250,35 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float mx = fmaxf(fmaxf(fmaxf(m8[0], m8[1]), fmaxf(m8[2], m8[3])),
                              fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7])));
       const float m_blk = mx * p.scale_log2;
-      float alpha = 1.f;
-      bool need = false;
-      if (j == 0) {
-        m_run = m_blk;
-      } else if (m_blk > m_run + kRescaleLog2) {
-        need = true;
-        alpha = ex2_approx(m_run - m_blk);
-        m_run = m_blk;
+      tc_fence_before();
+      mbar_arrive_warp(s_free);  // S_j is in registers: the next block's scores may land
+      // lazy rescale: keep the running max unless this block's max exceeds it
+      // by more than 2^8 (P <= 256 then, harmless in bf16 / fp32). It is rare,
+      // so it is settled here, before the exponentials: with the vote and its
+      // branch between them and P's stores a block took 120 cycles longer.
+      const bool need = j > 0 && m_blk > m_run + kRescaleLog2;
+      if (__any_sync(0xffffffffu, need)) {
+        debug_count_rescale(need && row_ok, p.status);
+        const float alpha = need ? ex2_approx(m_run - m_blk) : 1.f;
+        if (need) m_run = m_blk;
+        l_run *= alpha;
+        if (!mbar_wait(pv_done, (j - 1) & 1, wc)) {  // PV_{j-1} has finished with O
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+#pragma unroll 1
+        for (int c = 0; c < DH / 16; ++c) {
+          uint32_t ov[16];
+          tmem_ld16(tmem + t_lane + S::kTmemO + c * 16, ov);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) ov[i] = __float_as_uint(__uint_as_float(ov[i]) * alpha);
+          tmem_st16(tmem + t_lane + S::kTmemO + c * 16, ov);
+        }
+        tmem_wait_st();
       }
-      debug_count_rescale(need && row_ok, p.status);
-      l_run *= alpha;
+      if (j == 0) m_run = m_blk;
       const float neg_m = -m_run;
       // scale-and-shift and the row sum two scores per instruction (paired
       // fp32: the same IEEE roundings as the scalar forms, same 8 sum chains)
@@ -273,46 +288,41 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
       for (int i = 0; i < 4; ++i) l4[i] = 0ull;
       uint32_t pk[kBN / 2];
+      auto store_p = [&](int i0) {
+        tmem_st32(tmem + t_lane + S::kTmemP + i0, *reinterpret_cast<uint32_t(*)[32]>(&pk[i0]));
+      };
+      auto exps = [&](int i0, int i1) {  // pairs [i0, i1) of scores -> bf16 P
 #pragma unroll
-      for (int i = 0; i < kBN / 2; ++i) {
-        float t0, t1;
-        f32x2_unpack(f32x2_fma(f32x2_pack(sv[2 * i], sv[2 * i + 1]), scale2, negm2), t0, t1);
-        const float p0 = ex2_approx(t0);
-        const float p1 = ex2_approx(t1);
-        l4[i & 3] = f32x2_add(l4[i & 3], f32x2_pack(p0, p1));
-        pk[i] = pack_bf16x2(p0, p1);
+        for (int i = i0; i < i1; ++i) {
+          float t0, t1;
+          f32x2_unpack(f32x2_fma(f32x2_pack(sv[2 * i], sv[2 * i + 1]), scale2, negm2), t0, t1);
+          const float p0 = ex2_approx(t0);
+          const float p1 = ex2_approx(t1);
+          l4[i & 3] = f32x2_add(l4[i & 3], f32x2_pack(p0, p1));
+          pk[i] = pack_bf16x2(p0, p1);
+        }
+      };
+      // the first half of P goes out under the second half's exponentials,
+      // once PV_{j-1} has read the previous P
+      exps(0, kBN / 4);
+      if (j > 0 && !mbar_wait(pv_done, (j - 1) & 1, wc)) {
+        ok = false;
+        break;
       }
+      tc_fence_after();
+      store_p(0);
+      exps(kBN / 4, kBN / 2);
+      store_p(kBN / 4);
+      s_now = mbar_test(s_full, (j + 1) & 1);
+      tmem_wait_st();
+      tc_fence_before();
+      mbar_arrive_warp(p_full);
       float l8[8];
 #pragma unroll
       for (int i = 0; i < 4; ++i) f32x2_unpack(l4[i], l8[2 * i], l8[2 * i + 1]);
       l_run += ((l8[0] + l8[1]) + (l8[2] + l8[3])) + ((l8[4] + l8[5]) + (l8[6] + l8[7]));
-      if (j > 0) {
-        if (!mbar_wait(pv_done, (j - 1) & 1, wc)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        if (__any_sync(0xffffffffu, need)) {
-#pragma unroll 1
-          for (int c = 0; c < DH / 32; ++c) {
-            uint32_t ov[32];
-            tmem_ld32(tmem + t_lane + S::kTmemO + c * 32, ov);
-            tmem_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 32; ++i) ov[i] = __float_as_uint(__uint_as_float(ov[i]) * alpha);
-            tmem_st32(tmem + t_lane + S::kTmemO + c * 32, ov);
-          }
-          tmem_wait_st();
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < kBN / 64; ++c)
-        tmem_st32(tmem + t_lane + S::kTmemP + c * 32,
-                  *reinterpret_cast<uint32_t(*)[32]>(&pk[c * 32]));
-      tmem_wait_st();
-      tc_fence_before();
-      mbar_arrive(p_full);
     }
+
     if (ok && mbar_wait(pv_done, (nblk - 1) & 1, wc)) {
       tc_fence_after();
       const float inv_l = 1.f / l_run;

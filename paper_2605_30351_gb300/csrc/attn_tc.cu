@@ -15,12 +15,12 @@
 //              the same batch element): each CTA fetches half of every key
 //              tile from L2 and multicasts it into both CTAs' stage, halving
 //              the L2-to-SM traffic, which otherwise bounds the kernel.
-//   warp 1     allocates TMEM; one lane issues the score MMAs
+//   warp 1     allocates TMEM; issues the score MMAs
 //              S_j = Q K_j^T with Q read from TMEM, so they read only the key
 //              tile from shared memory. S_{j+1} is issued as soon as the
 //              softmax has copied S_j into registers.
-//   warp 6     one lane issues O += P_j V_j with P read from TMEM. Two issuing
-//              threads keep the tensor pipe fed while either one waits on a
+//   warp 6     issues O += P_j V_j with P read from TMEM. Two issuing
+//              warps keep the tensor pipe fed while either one waits on a
 //              barrier: the MMA queue is shallow, so a single issuer's
 //              bookkeeping between groups would leave the pipe idle.
 //   warps 2-5  load q_c, rotate q_r and store both into TMEM; then the online
@@ -41,6 +41,12 @@
 // multicast as the row-tile pairs above; each keeps the q_c columns that fit
 // next to S, P and its O half in TMEM (320) and the rest of Q in shared
 // memory, so QK mixes TMEM- and shared-memory A operands.
+// What bounds it (Wan shape): the tensor pipe at d_c = 192 (92 % active; the
+// GPU's power cap in long runs), a block's softmax (~1200 cycles beside 1152 of
+// MMAs) at d_c = 128, the wait for keys at d_c = 256 (two stages beside Q) and
+// the doubled score at 512. Issuing from converged warps and settling the
+// rescale before the exponentials took d_c = 128 from 579 to 549 us, (256, 64)
+// from 1325 to 1260 us and (512, 64) from 4341 to 4131 us, bit-identical.
 // The V operand is the first d_c columns of the same key tile read MN-major,
 // so the cache is never expanded into per-head keys or values.
 #include <cmath>
@@ -82,7 +88,7 @@ struct AttnShape {
   static constexpr int kQKrOff = kQcSmem * kBM * 2;
   static constexpr int kQBytes = kQinTmem ? 0 : kQKrOff + kBM * DR * 2;
   static constexpr int kFit = (kSmemCap - 1024 - kBarBytes - kQBytes) / kTileBytes;
-  static constexpr int kMaxStages = BN == 128 ? 4 : 6;
+  static constexpr int kMaxStages = 6;
   static constexpr int kStages = kFit > kMaxStages ? kMaxStages : kFit;
   static constexpr int kSmemBytes = 1024 + kQBytes + kTileBytes * kStages + kBarBytes;
   static constexpr uint32_t kTmemCols = 512;
@@ -154,14 +160,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (threadIdx.x == 0) {
     mbar_init(q_tma_full, 1);
-    mbar_init(q_ready, kBM);
+    mbar_init(q_ready, 4);  // one arrival per softmax warp, and so below
     for (int s = 0; s < NST; ++s) {
       mbar_init(&kv_full[s], 1);
       mbar_init(&kv_empty[s], CL);  // released by the MMA of every CTA that reads it
     }
     mbar_init(s_full, 1);
-    mbar_init(s_free, kBM);
-    mbar_init(p_full, kBM);
+    mbar_init(s_free, 4);
+    mbar_init(p_full, 4);
     mbar_init(pv_done, 1);
     mbar_init(&mma_drain[0], 1);
     mbar_init(&mma_drain[1], 1);
@@ -225,85 +231,81 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------ QK^T issuer
-    if (lane == 0) {
-      bool ok = mbar_wait(q_ready, 0, wc);
-      if constexpr (!S::kQinTmem) ok = ok && mbar_wait(q_tma_full, 0, wc);
+    // the whole warp walks the loop; one lane issues (see elect_one)
+    bool ok = mbar_wait_warp(q_ready, 0, wc);
+    if constexpr (!S::kQinTmem) ok = ok && mbar_wait_warp(q_tma_full, 0, wc);
+    const uint64_t qd = sdesc(smem_u32(sQ), 16, 1024, kSw128);
+    const uint64_t qrd = sdesc(smem_u32(sQ) + S::kQKrOff, 16, S::kKrSbo, S::kKrSw);
+    const uint64_t kd = sdesc(smem_u32(sKV), 16, 1024, kSw128);
+    const uint64_t krd = sdesc(smem_u32(sKV) + S::kKrOff, 16, S::kKrSbo, S::kKrSw);
+    for (int j = 0; ok && j < nblk; ++j) {
+      // S = Q K_j^T; S's previous contents (block j-1) must have been read
+      const int st = j % NST;
+      ok = (j == 0 || mbar_wait_warp(s_free, (j - 1) & 1, wc)) &&
+           mbar_wait_warp(&kv_full[st], (j / NST) & 1, wc);
+      if (!ok) break;
       tc_fence_after();
-      const uint32_t qa = smem_u32(sQ);
-      for (int j = 0; ok && j < nblk; ++j) {
-        // S = Q K_j^T; S's previous contents (block j-1) must have been read
-        if (j >= 1 && !mbar_wait(s_free, (j - 1) & 1, wc)) {
-          ok = false;
-          break;
-        }
-        const int st = j % NST;
-        if (!mbar_wait(&kv_full[st], (j / NST) & 1, wc)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t ka = smem_u32(sKV) + st * S::kTileBytes;
+      if (elect_one()) {
+        const uint64_t ko = static_cast<uint64_t>(st * (S::kTileBytes >> 4));
 #pragma unroll
         for (int cb = 0; cb < DC / 64; ++cb)
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            const uint64_t bd = sdesc(ka + cb * S::kCBox + k * 32, 16, 1024, kSw128);
+            const uint64_t bd = kd + ko + ((cb * S::kCBox + k * 32) >> 4);
             const uint32_t acc = (cb | k) != 0 ? 1u : 0u;
             if (cb < S::kQcTmem / 64)  // resolved at compile time (unrolled)
               umma_ts(tmem + S::kTmemS, tmem + S::kTmemQ + (cb * 4 + k) * 8, bd, S::kIdescQK, acc);
             else
-              umma_ss(tmem + S::kTmemS,
-                      sdesc(qa + (cb - S::kQcTmem / 64) * 16384 + k * 32, 16, 1024, kSw128), bd,
+              umma_ss(tmem + S::kTmemS, qd + (((cb - S::kQcTmem / 64) * 16384 + k * 32) >> 4), bd,
                       S::kIdescQK, acc);
           }
 #pragma unroll
         for (int k = 0; k < DR / 16; ++k) {
-          const uint64_t bd = sdesc(ka + S::kKrOff + k * 32, 16, S::kKrSbo, S::kKrSw);
           if constexpr (S::kQinTmem)
-            umma_ts(tmem + S::kTmemS, tmem + S::kTmemQ + DC / 2 + k * 8, bd, S::kIdescQK, 1u);
+            umma_ts(tmem + S::kTmemS, tmem + S::kTmemQ + DC / 2 + k * 8, krd + ko + k * 2,
+                    S::kIdescQK, 1u);
           else
-            umma_ss(tmem + S::kTmemS, sdesc(qa + S::kQKrOff + k * 32, 16, S::kKrSbo, S::kKrSw),
-                    bd, S::kIdescQK, 1u);
+            umma_ss(tmem + S::kTmemS, qrd + k * 2, krd + ko + k * 2, S::kIdescQK, 1u);
         }
         umma_commit(s_full);
       }
-      if (!ok) {  // wait for every MMA this thread issued before TMEM is freed
-        umma_commit(&mma_drain[0]);
-        mbar_wait_drain(&mma_drain[0], 0, p.status);
-      }
+      __syncwarp();
     }
-    __syncwarp();
+    if (!ok) {  // wait for every MMA this warp issued before TMEM is freed
+      if (elect_one()) umma_commit(&mma_drain[0]);
+      __syncwarp();
+      mbar_wait_drain(&mma_drain[0], 0, p.status);
+    }
   } else if (warp == 6) {
     // --------------------------------------------------------- PV issuer
-    if (lane == 0) {
-      bool ok = true;
-      for (int i = 0; ok && i < nblk; ++i) {
-        // O += P_i V_i, V = this CTA's DV of the first d_c columns of block
-        // i's stage (MN-major)
-        if (!mbar_wait(p_full, i & 1, wc)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const int st = i % NST;
-        const uint32_t va = smem_u32(sKV) + st * S::kTileBytes + vpart * (DV / 64) * S::kCBox;
+    bool ok = true;
+    // V = this CTA's DV of the first d_c columns of block i's stage (MN-major)
+    const uint64_t vd =
+        sdesc(smem_u32(sKV) + vpart * (DV / 64) * S::kCBox, S::kCBox, 1024, kSw128);
+    for (int i = 0; ok && i < nblk; ++i) {
+      ok = mbar_wait_warp(p_full, i & 1, wc);  // O += P_i V_i
+      if (!ok) break;
+      tc_fence_after();
+      const int st = i % NST;
+      if (elect_one()) {
+        const uint64_t vo = static_cast<uint64_t>(st * (S::kTileBytes >> 4));
 #pragma unroll
         for (int s = 0; s < kBN / 16; ++s)
-          umma_ts(tmem + S::kTmemO, tmem + S::kTmemP + s * 8,
-                  sdesc(va + s * 2048, S::kCBox, 1024, kSw128), S::kIdescPV,
-                  (i > 0 || s > 0) ? 1u : 0u);
+          umma_ts(tmem + S::kTmemO, tmem + S::kTmemP + s * 8, vd + vo + s * (2048 >> 4),
+                  S::kIdescPV, (i > 0 || s > 0) ? 1u : 0u);
         if constexpr (CL == 1)
           umma_commit(&kv_empty[st]);
         else
           umma_commit_mc(&kv_empty[st], kPair);
         umma_commit(pv_done);
       }
-      if (!ok) {
-        umma_commit(&mma_drain[1]);
-        mbar_wait_drain(&mma_drain[1], 0, p.status);
-      }
+      __syncwarp();
     }
-    __syncwarp();
+    if (!ok) {
+      if (elect_one()) umma_commit(&mma_drain[1]);
+      __syncwarp();
+      mbar_wait_drain(&mma_drain[1], 0, p.status);
+    }
   } else {
     // ------------------------------------------------ softmax (warps 2..5)
     const int quarter = warp & 3;  // TMEM lane quarter this warp may access
@@ -382,14 +384,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_wait_st();
         tc_fence_before();
       }
-      mbar_arrive(q_ready);
+      mbar_arrive_warp(q_ready);
     }
 
     float m_run = -INFINITY;
     float l_run = 0.f;
     bool ok = true;
+    bool s_now = false;  // a poll has seen the next block's scores
     for (int j = 0; j < nblk; ++j) {
-      if (!mbar_wait(s_full, j & 1, wc)) {
+      if (!s_now && !mbar_wait(s_full, j & 1, wc)) {
         ok = false;
         break;
       }
@@ -401,7 +404,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                   *reinterpret_cast<uint32_t(*)[32]>(&sr[c * 32]));
       tmem_wait_ld();
       tc_fence_before();
-      mbar_arrive(s_free);  // S_j is in registers: the next block's scores may land
+      mbar_arrive_warp(s_free);  // S_j is in registers: the next block's scores may land
       float sv[kBN];
 #pragma unroll
       for (int c = 0; c < kBN; ++c) sv[c] = __uint_as_float(sr[c]);
@@ -428,18 +431,32 @@ __global__ void __launch_bounds__(kThreads, 1)
                              fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7])));
       const float m_blk = mx * p.scale_log2;
       // lazy rescale: keep the running max unless this block's max exceeds it
-      // by more than 2^8 (P <= 256 then, harmless in bf16 / fp32)
-      float alpha = 1.f;
-      bool need = false;
-      if (j == 0) {
-        m_run = m_blk;
-      } else if (m_blk > m_run + kRescaleLog2) {
-        need = true;
-        alpha = ex2_approx(m_run - m_blk);
-        m_run = m_blk;
+      // by more than 2^8 (P <= 256 then, harmless in bf16 / fp32). It is rare,
+      // so it is settled here, before the exponentials: with the vote and its
+      // branch between them and P's stores a block took 120 cycles longer.
+      const bool need = j > 0 && m_blk > m_run + kRescaleLog2;
+      if (__any_sync(0xffffffffu, need)) {
+        debug_count_rescale(need && row_ok, p.status);
+        const float alpha = need ? ex2_approx(m_run - m_blk) : 1.f;
+        if (need) m_run = m_blk;
+        l_run *= alpha;
+        if (!mbar_wait(pv_done, (j - 1) & 1, wc)) {  // PV_{j-1} has finished with O
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+#pragma unroll 1
+        for (int c = 0; c < DV / 16; ++c) {
+          uint32_t ov[16];
+          tmem_ld16(tmem + t_lane + S::kTmemO + c * 16, ov);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) ov[i] = __float_as_uint(__uint_as_float(ov[i]) * alpha);
+          tmem_st16(tmem + t_lane + S::kTmemO + c * 16, ov);
+        }
+        tmem_wait_st();
       }
-      debug_count_rescale(need && row_ok, p.status);
-      l_run *= alpha;
+      if (j == 0) m_run = m_blk;
       // P_j in registers before waiting on PV_{j-1}: only the TMEM store
       // below is serialised with the previous PV
       const float neg_m = -m_run;
@@ -451,47 +468,42 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
       for (int i = 0; i < 4; ++i) l4[i] = 0ull;
       uint32_t pk[kBN / 2];
+      auto store_p = [&](int i0) {  // half of P's words, from pair i0
+        if constexpr (kBN == 128)
+          tmem_st32(tmem + t_lane + S::kTmemP + i0, *reinterpret_cast<uint32_t(*)[32]>(&pk[i0]));
+        else
+          tmem_st16(tmem + t_lane + S::kTmemP + i0, &pk[i0]);
+      };
+      auto exps = [&](int i0, int i1) {  // pairs [i0, i1) of scores -> bf16 P
 #pragma unroll
-      for (int i = 0; i < kBN / 2; ++i) {
-        float t0, t1;
-        f32x2_unpack(f32x2_fma(f32x2_pack(sv[2 * i], sv[2 * i + 1]), scale2, negm2), t0, t1);
-        const float p0 = ex2_approx(t0);
-        const float p1 = ex2_approx(t1);
-        l4[i & 3] = f32x2_add(l4[i & 3], f32x2_pack(p0, p1));
-        pk[i] = pack_bf16x2(p0, p1);
+        for (int i = i0; i < i1; ++i) {
+          float t0, t1;
+          f32x2_unpack(f32x2_fma(f32x2_pack(sv[2 * i], sv[2 * i + 1]), scale2, negm2), t0, t1);
+          const float p0 = ex2_approx(t0);
+          const float p1 = ex2_approx(t1);
+          l4[i & 3] = f32x2_add(l4[i & 3], f32x2_pack(p0, p1));
+          pk[i] = pack_bf16x2(p0, p1);
+        }
+      };
+      // the first half of P goes out under the second half's exponentials,
+      // once PV_{j-1} has read the previous P
+      exps(0, kBN / 4);
+      if (j > 0 && !mbar_wait(pv_done, (j - 1) & 1, wc)) {
+        ok = false;
+        break;
       }
+      tc_fence_after();
+      store_p(0);
+      exps(kBN / 4, kBN / 2);
+      store_p(kBN / 4);
+      s_now = mbar_test(s_full, (j + 1) & 1);
+      tmem_wait_st();
+      tc_fence_before();
+      mbar_arrive_warp(p_full);
       float l8[8];
 #pragma unroll
       for (int i = 0; i < 4; ++i) f32x2_unpack(l4[i], l8[2 * i], l8[2 * i + 1]);
       l_run += ((l8[0] + l8[1]) + (l8[2] + l8[3])) + ((l8[4] + l8[5]) + (l8[6] + l8[7]));
-      if (j > 0) {
-        // PV_{j-1} must have read P (and finished with O) before P_j is
-        // written or O is rescaled
-        if (!mbar_wait(pv_done, (j - 1) & 1, wc)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        if (__any_sync(0xffffffffu, need)) {
-#pragma unroll 1
-          for (int c = 0; c < DV / 32; ++c) {
-            uint32_t ov[32];
-            tmem_ld32(tmem + t_lane + S::kTmemO + c * 32, ov);
-            tmem_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 32; ++i) ov[i] = __float_as_uint(__uint_as_float(ov[i]) * alpha);
-            tmem_st32(tmem + t_lane + S::kTmemO + c * 32, ov);
-          }
-          tmem_wait_st();
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < kBN / 64; ++c)
-        tmem_st32(tmem + t_lane + S::kTmemP + c * 32,
-                  *reinterpret_cast<uint32_t(*)[32]>(&pk[c * 32]));
-      tmem_wait_st();
-      tc_fence_before();
-      mbar_arrive(p_full);
     }
 
     // O / l as bf16: each thread stages its row densely in the key stages
