@@ -406,7 +406,7 @@ int launch_dense(const DenseArgs& a) {
 
 int launch_dense_attention_tc(const DenseArgs& a) {
   switch (a.head_dim) {
-    case 64: return launch_dense<64>(a);
+    case 64: return launch_dense_dual_tc(a);  // two row tiles per CTA
     case 128: return launch_dense<128>(a);
     default: return MLA_ERR_UNSUPPORTED;
   }

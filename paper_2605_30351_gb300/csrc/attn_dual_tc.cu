@@ -1,0 +1,753 @@
+// Attention with two row tiles per CTA on the sm_103a tensor cores, for value
+// width 64: the absorbed-form latent attention at d_c = 64 (Eq. score; App. E)
+// and the dense per-head baseline at head_dim 64 (App. C.1).
+//     S = Q K^T,  P = exp2(S * log2(e)/sqrt(d_h) - m),  O += P V
+// Latent: a row is one (token, head) pair, K = [c | k] and V = c, both read
+// from the same key tile. Dense: a row is one token of one head, K and V are
+// that head's planes.
+//
+// At this width the MMAs of a 128 x 128 block (6 score steps of 64 cycles and
+// 8 PV steps of ~45 at d_r = 32) are shorter than its softmax, which alone
+// takes one warp per SM sub-partition 930 cycles and two warps 1400 for two
+// blocks. With one tile per CTA neither side is busy (1335 cycles a block:
+// tensor pipe 46 %, exponential unit 39 %). A CTA therefore owns two 128-row
+// tiles, each with its own four softmax warps, S, P and O, which read the same
+// key tiles; the softmax of one runs under the MMAs and the softmax of the
+// other. At the Wan shape (56,160 rows x 32,760 keys, d_c = 64, d_r = 32) the
+// launch went from 523 to 388 us (1120 -> 1520 TFLOP/s; ~920 cycles a block);
+// the two warps that share a sub-partition's exponential unit bound it now.
+//   warp 0      TMA producer: Q tiles once, then key tiles into a ring
+//   warps 1, 2  issue the MMAs of tile 0 and of tile 1: neither waits for the
+//               other tile's softmax
+//   warp 3      allocates TMEM
+//   warps 4-7   softmax of tile 0, warps 8-11 of tile 1: thread = row
+// TMEM (512 columns): S0 S1 [0,256)  P0 P1 [256,384)  O0 O1 [384,512). P has
+// its own columns, so S goes back to the issuer as soon as it has been read.
+// Q stays in shared memory (the score MMAs read both operands there). At value
+// width 128 O leaves P no columns of its own and PV and the next score must
+// follow each other: that form measured no faster than one tile per CTA.
+//
+// Tail of the grid: a tile's key blocks may be split over the CTAs of its
+// cluster. Each CTA then keeps its own running maximum m and sum l; at the end
+// every row has an owner among the CTAs, the others write (O, m, l) of the row
+// to the owner's shared memory, and the owner combines them:
+//     O = sum_s 2^(m_s - m) O_s / sum_s 2^(m_s - m) l_s
+#include <cmath>
+
+#include "internal.h"
+#include "ptx_sm103.cuh"
+
+namespace vmla {
+namespace {
+
+constexpr int kBM = 128;  // rows per tile = TMEM lanes
+constexpr int kBN = 128;  // keys per block
+constexpr int DV = 64;    // value width
+constexpr int kThreads = 384;
+constexpr int kCtlRegs = 120, kSoftRegs = 192;  // 128 * 120 + 256 * 192 <= 384 * 168
+constexpr float kRescaleLog2 = 8.0f;
+constexpr int kMaxCluster = 8;
+
+// DR > 0: latent rows, score width DV + DR. DR = 0: dense, head_dim = DV.
+template <int DR>
+struct DualShape {
+  static constexpr bool kLatent = DR > 0;
+  static constexpr int DK = DV + DR;
+  static constexpr int kQTile = kBM * DK * 2;  // one row tile of Q
+  static constexpr int kQrOff = kBM * DV * 2;  // its d_r columns
+  static constexpr int kEntry = kBN * DK * 2;  // ring entry: a [c | k] tile, or one of K, V
+  static constexpr int kKrOff = kBN * DV * 2;  // latent: the positional key's columns
+  static constexpr int kEntriesPerBlock = kLatent ? 1 : 2;
+  static constexpr int kBarBytes = 256;
+  static constexpr int kFit = (232448 - 1024 - kBarBytes - 2 * kQTile) / kEntry;
+  static constexpr int kRing = kFit > 8 ? 8 : kFit;
+  static constexpr int kSmemBytes = 1024 + 2 * kQTile + kRing * kEntry + kBarBytes;
+  static constexpr int kTmemP = 2 * kBN;           // P_t at kTmemP + 64 t, two bf16 a column
+  static constexpr int kTmemO = kTmemP + kBN;      // O_t at kTmemO + DV t
+  // one row of a split tile on its way to its owner: O, then m and l
+  static constexpr int kRecord = DV * 4 + 16;
+  static constexpr uint32_t kKrSw = DR == 32 ? kSw64 : kSw128;
+  static constexpr uint32_t kKrRow = DR * 2;
+  static constexpr uint32_t kKrSbo = 8 * kKrRow;
+  static constexpr uint32_t kIdescQK = idesc_bf16_f32(kBM, kBN, false, false);
+  static constexpr uint32_t kIdescPV = idesc_bf16_f32(kBM, DV, false, true);
+  static_assert(DR == 0 || DR == 32 || DR == 64, "d_r");
+  static_assert(kRing >= 2 * kEntriesPerBlock, "two key blocks in flight");
+  static_assert(kEntry % 1024 == 0 && kQTile % 1024 == 0, "swizzle-atom alignment");
+  static_assert(2 * kBM * kRecord / kMaxCluster * (kMaxCluster - 1) <=
+                    2 * kQTile + kRing * kEntry,
+                "records of a split tile fit where Q and the ring were");
+};
+
+struct DualKParams {
+  const __nv_bfloat16* q_r;  // latent
+  const int* q_pos;
+  const float2* rope;
+  __nv_bfloat16* o;
+  int rows;       // rows per plane (latent: a batch element; dense: a head of one)
+  int heads, n_valid, rope_len, pairs_t, pairs_h;
+  float scale_log2;
+  int* status;
+  int planes, tiles;  // tiles of 256 rows per plane
+  int cl;             // CTAs per cluster
+  int n_whole;        // per plane: clusters whose CTAs each take a whole tile
+};
+
+template <int DR>
+__global__ void __launch_bounds__(kThreads, 1)
+    mla_attn_dual_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
+                            const __grid_constant__ CUtensorMap tm_k,
+                            const __grid_constant__ CUtensorMap tm_v, const DualKParams p) {
+  using S = DualShape<DR>;
+  constexpr int NST = S::kRing;
+  constexpr bool kLatent = S::kLatent;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = align_smem_1024(smem_raw);
+  uint8_t* sQ = smem;
+  uint8_t* sKV = smem + 2 * S::kQTile;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sKV + NST * S::kEntry);
+  uint64_t* q_tma_full = bars;
+  uint64_t* q_ready = bars + 1;  // [2], one per tile
+  uint64_t* kv_full = bars + 3;
+  uint64_t* kv_empty = kv_full + NST;
+  uint64_t* s_full = kv_empty + NST;  // [2], and so below
+  uint64_t* s_free = s_full + 2;
+  uint64_t* p_full = s_free + 2;
+  uint64_t* pv_done = p_full + 2;
+  uint64_t* mma_drain = pv_done + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_drain + 2);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const WaitCtx wc{abort_flag, p.status};
+
+  // Which tile, and which of its key blocks. The clusters that hold one whole
+  // tile per CTA come first (they run longest), then the tiles whose blocks
+  // are split over a cluster.
+  const int crank = p.cl > 1 ? static_cast<int>(cluster_ctarank()) : 0;
+  const int cid = blockIdx.x / p.cl;
+  const bool whole = cid < p.n_whole * p.planes;
+  int plane, tile, n_split;
+  if (whole) {
+    plane = cid / p.n_whole;
+    tile = (cid - plane * p.n_whole) * p.cl + crank;
+    n_split = 1;
+  } else {
+    const int rest = p.tiles - p.n_whole * p.cl;  // split tiles per plane
+    const int i = cid - p.n_whole * p.planes;
+    plane = i / rest;
+    tile = p.n_whole * p.cl + (i - plane * rest);
+    n_split = p.cl;
+  }
+  const int row0 = tile * 2 * kBM;
+  const int nt = row0 + kBM < p.rows ? 2 : 1;  // row tiles with any row
+  const int nblk_all = (p.n_valid + kBN - 1) / kBN;
+  const int part = n_split > 1 ? crank : 0;
+  const int jb0 = static_cast<int>(static_cast<long long>(nblk_all) * part / n_split);
+  const int nblk =
+      static_cast<int>(static_cast<long long>(nblk_all) * (part + 1) / n_split) - jb0;
+
+  if (threadIdx.x == 0) {
+    mbar_init(q_tma_full, 1);
+        for (int s = 0; s < NST; ++s) {
+      mbar_init(&kv_full[s], 1);
+      mbar_init(&kv_empty[s], nt);  // each tile's issuer releases it
+    }
+    for (int t = 0; t < 2; ++t) {
+      mbar_init(&q_ready[t], 4);  // one arrival per softmax warp, and so below
+      mbar_init(&s_full[t], 1);
+      mbar_init(&s_free[t], 4);
+      mbar_init(&p_full[t], 4);
+      mbar_init(&pv_done[t], 1);
+      mbar_init(&mma_drain[t], 1);
+    }
+    *abort_flag = 0;
+    fence_mbar_init();
+  }
+  if (warp == 3) {
+    tmem_alloc(tmem_slot, 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  grid_dep_sync();
+
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kCtlRegs));
+    if (warp == 0) {
+      // ------------------------------------------------------------ producer
+      if (lane == 0) {
+        tma_prefetch_desc(&tm_q);
+        tma_prefetch_desc(&tm_k);
+        tma_prefetch_desc(&tm_v);
+        mbar_arrive_expect_tx(q_tma_full, nt * kBM * DV * 2);
+        const int qx = kLatent ? 0 : (plane % p.heads) * DV;
+        const int qz = kLatent ? plane : plane / p.heads;
+        for (int t = 0; t < nt; ++t)
+#pragma unroll
+          for (int cb = 0; cb < DV / 64; ++cb)
+            tma_load_3d(sQ + t * S::kQTile + cb * 16384, &tm_q, q_tma_full, qx + cb * 64,
+                        row0 + t * kBM, qz);
+        int issued = 0;
+        const int entries = nblk * S::kEntriesPerBlock;
+        for (int e = 0; e < entries; ++e) {
+          const int st = e % NST;
+          if (e >= NST && !mbar_wait(&kv_empty[st], ((e / NST) - 1) & 1, wc)) break;
+          uint8_t* kv = sKV + st * S::kEntry;
+          mbar_arrive_expect_tx(&kv_full[st], S::kEntry);
+          const int key0 = (jb0 + e / S::kEntriesPerBlock) * kBN;
+          // latent: tm_k covers c, tm_v the positional key; dense: K and V in turn
+          const CUtensorMap* tm = !kLatent && (e & 1) ? &tm_v : &tm_k;
+#pragma unroll
+          for (int cb = 0; cb < DV / 64; ++cb)
+            tma_load_3d(kv + cb * 16384, tm, &kv_full[st], cb * 64, key0, plane);
+          if constexpr (kLatent)
+            tma_load_3d(kv + S::kKrOff, &tm_v, &kv_full[st], 0, key0, plane);
+          issued = e + 1;
+        }
+        if (*abort_flag) {  // let every copy this CTA started land before exit
+          mbar_wait_drain(q_tma_full, 0, p.status);
+          for (int u = issued > NST ? issued - NST : 0; u < issued; ++u)
+            mbar_wait_drain(&kv_full[u % NST], (u / NST) & 1, p.status);
+        }
+      }
+    } else if (warp - 1 < nt) {
+      // ------------------------------------------------------- MMA issuer of one tile
+      // The whole warp walks the loop; one lane issues (see elect_one).
+      const uint64_t qd = sdesc(smem_u32(sQ), 16, 1024, kSw128);
+      const uint64_t qrd = sdesc(smem_u32(sQ) + S::kQrOff, 16, S::kKrSbo, S::kKrSw);
+      const uint64_t kd = sdesc(smem_u32(sKV), 16, 1024, kSw128);
+      const uint64_t krd = sdesc(smem_u32(sKV) + S::kKrOff, 16, S::kKrSbo, S::kKrSw);
+      const uint64_t vd = sdesc(smem_u32(sKV), 16384, 1024, kSw128);
+      auto issue_qk = [&](int t, int st) {  // S_t = Q_t K^T, K in ring stage st
+        const uint64_t qo = static_cast<uint64_t>(t * (S::kQTile >> 4));
+        const uint64_t ko = static_cast<uint64_t>(st * (S::kEntry >> 4));
+#pragma unroll
+        for (int k = 0; k < DV / 16; ++k) {
+          const uint64_t step = ((k >> 2) * 16384 + (k & 3) * 32) >> 4;
+          umma_ss(tmem + t * kBN, qd + qo + step, kd + ko + step, S::kIdescQK, k != 0 ? 1u : 0u);
+        }
+#pragma unroll
+        for (int k = 0; k < DR / 16; ++k)
+          umma_ss(tmem + t * kBN, qrd + qo + k * 2, krd + ko + k * 2, S::kIdescQK, 1u);
+        umma_commit(&s_full[t]);
+        if (!kLatent) umma_commit(&kv_empty[st]);
+      };
+      // O_t += P_t V, V in ring stage st (MN-major)
+      auto issue_pv = [&](int t, int st, bool first) {
+        const uint64_t vo = static_cast<uint64_t>(st * (S::kEntry >> 4));
+#pragma unroll
+        for (int s = 0; s < kBN / 16; ++s)
+          umma_ts(tmem + S::kTmemO + t * DV, tmem + S::kTmemP + t * (kBN / 2) + s * 8,
+                  vd + vo + s * (2048 >> 4), S::kIdescPV, (!first || s > 0) ? 1u : 0u);
+      };
+      auto wait_full = [&](int e) {
+        return mbar_wait_warp(&kv_full[e % NST], (e / NST) & 1, wc);
+      };
+      constexpr int kE = S::kEntriesPerBlock;
+      bool ok = mbar_wait_warp(q_tma_full, 0, wc) && wait_full(0);
+      const int t = warp - 1;
+      ok = ok && (!kLatent || mbar_wait_warp(&q_ready[t], 0, wc));
+      tc_fence_after();
+      if (ok && elect_one()) issue_qk(t, 0);
+      __syncwarp();
+      for (int j = 0; ok && j < nblk; ++j) {
+        const int ek = (j + 1) * kE, ev = j * kE + (kE - 1);  // entries of K(j+1) and V(j)
+        if (j + 1 < nblk) {  // S(j+1) as soon as S(j) has been read
+          ok = wait_full(ek) && mbar_wait_warp(&s_free[t], j & 1, wc);
+          if (!ok) break;
+          tc_fence_after();
+          if (elect_one()) issue_qk(t, ek % NST);
+          __syncwarp();
+        }
+        ok = (kLatent || wait_full(ev)) && mbar_wait_warp(&p_full[t], j & 1, wc);
+        if (!ok) break;
+        tc_fence_after();
+        if (elect_one()) {
+          issue_pv(t, ev % NST, j == 0);
+          umma_commit(&kv_empty[ev % NST]);
+          umma_commit(&pv_done[t]);
+        }
+        __syncwarp();
+      }
+      if (!ok) {  // every MMA this warp issued is done before TMEM is freed
+        if (elect_one()) umma_commit(&mma_drain[warp - 1]);
+        __syncwarp();
+        mbar_wait_drain(&mma_drain[warp - 1], 0, p.status);
+      }
+    }
+    __syncwarp();
+    if (n_split > 1) {  // the two barrier phases of the combination
+      cluster_arrive_release();
+      cluster_wait_acquire();
+      cluster_arrive_release();
+      cluster_wait_acquire();
+    }
+  } else {
+    // --------------------------------------------------------- softmax warps
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftRegs));
+    const int t = (warp - 4) >> 2;
+    const int quarter = warp & 3;  // TMEM lane quarter this warp may access
+    const int r = quarter * 32 + lane;
+    const uint32_t t_lane = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
+    const int grow = row0 + t * kBM + r;
+    const bool row_ok = grow < p.rows;
+    const bool active = t < nt;
+    if (kLatent && active) {
+      // q_r rotated by the query position (RoPE3D), next to the TMA-loaded q_c
+      uint32_t w[DR > 0 ? DR / 2 : 1];
+#pragma unroll
+      for (int i = 0; i < DR / 2; ++i) w[i] = 0u;
+      if (row_ok) {
+        const uint4* src = reinterpret_cast<const uint4*>(
+            p.q_r + (static_cast<size_t>(plane) * p.rows + grow) * DR);
+#pragma unroll
+        for (int i = 0; i < DR / 8; ++i) {
+          const uint4 v = __ldg(src + i);
+          w[4 * i + 0] = v.x;
+          w[4 * i + 1] = v.y;
+          w[4 * i + 2] = v.z;
+          w[4 * i + 3] = v.w;
+        }
+        const int nq = p.rows / p.heads;
+        const int* pp = p.q_pos + (static_cast<size_t>(plane) * nq + grow / p.heads) * 3;
+        int pa[3] = {__ldg(pp), __ldg(pp + 1), __ldg(pp + 2)};
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+          if (pa[a] < 0 || pa[a] >= p.rope_len) {
+            record_status(p.status, MLA_ERR_RANGE);
+            pa[a] = 0;
+          }
+#pragma unroll
+        for (int i = 0; i < DR / 2; ++i) {
+          const int pos = i < p.pairs_t ? pa[0] : (i < p.pairs_t + p.pairs_h ? pa[1] : pa[2]);
+          const float2 cs = __ldg(p.rope + static_cast<size_t>(pos) * (DR / 2) + i);
+          const float x0 = bf16_lo(w[i]), x1 = bf16_hi(w[i]);
+          w[i] = pack_bf16x2(x0 * cs.x - x1 * cs.y, x0 * cs.y + x1 * cs.x);
+        }
+      }
+      // the 16-byte-chunk swizzle of a row of the d_r block
+      uint8_t* krow = sQ + t * S::kQTile + S::kQrOff + r * S::kKrRow;
+#pragma unroll
+      for (int c = 0; c < DR / 8; ++c) {
+        const int phys = DR == 32 ? (c ^ ((r >> 1) & 3)) : (c ^ (r & 7));
+        *reinterpret_cast<uint4*>(krow + phys * 16) =
+            make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+      }
+      fence_proxy_async_smem();
+      mbar_arrive_warp(&q_ready[t]);
+    }
+
+    float m_run = -INFINITY;
+    float l_run = 0.f;
+    bool ok = active;
+    const uint32_t tS = t_lane + t * kBN;
+    const uint32_t tP = t_lane + S::kTmemP + t * (kBN / 2);
+    const uint32_t tO = t_lane + S::kTmemO + t * DV;
+    bool s_now = false;  // a poll has seen the next block's scores
+    for (int j = 0; ok && j < nblk; ++j) {
+      if (!s_now && !mbar_wait(&s_full[t], j & 1, wc)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      uint32_t sr[kBN];
+#pragma unroll
+      for (int c = 0; c < kBN / 32; ++c)
+        tmem_ld32(tS + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[c * 32]));
+      tmem_wait_ld();
+      float sv[kBN];
+#pragma unroll
+      for (int c = 0; c < kBN; ++c) sv[c] = __uint_as_float(sr[c]);
+      const int valid = p.n_valid - (jb0 + j) * kBN;
+      if (valid < kBN) {
+#pragma unroll
+        for (int c = 0; c < kBN; ++c)
+          if (c >= valid) sv[c] = -INFINITY;
+      }
+      // row max: 8 chains of three-input maxima, then a tree
+      float m8[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) m8[i] = fmaxf(sv[i], sv[8 + i]);
+#pragma unroll
+      for (int c = 16; c + 16 <= kBN; c += 16)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) m8[i] = fmax3(m8[i], sv[c + i], sv[c + 8 + i]);
+      const float mx = fmaxf(fmaxf(fmaxf(m8[0], m8[1]), fmaxf(m8[2], m8[3])),
+                             fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7])));
+      const float m_blk = mx * p.scale_log2;
+      // S is in registers: the next block's scores may land (after the max: any
+      // earlier and the arrival's fence delays the reads, 416 against 427 us)
+      tc_fence_before();
+      mbar_arrive_warp(&s_free[t]);
+      // lazy rescale: keep the running max unless this block's max exceeds it
+      // by more than 2^8 (P <= 256 then, harmless in bf16 / fp32). Rare, so it
+      // is settled here, off the path between the exponentials and P (the vote
+      // and its branch cost a block 120 cycles there).
+      const bool need = j > 0 && m_blk > m_run + kRescaleLog2;
+      if (__any_sync(0xffffffffu, need)) {
+        debug_count_rescale(need && row_ok, p.status);
+        const float alpha = need ? ex2_approx(m_run - m_blk) : 1.f;
+        if (need) m_run = m_blk;
+        l_run *= alpha;
+        if (!mbar_wait(&pv_done[t], (j - 1) & 1, wc)) {  // PV(j-1) is done with O
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+#pragma unroll 1
+        for (int c = 0; c < DV / 16; ++c) {
+          uint32_t ov[16];
+          tmem_ld16(tO + c * 16, ov);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) ov[i] = __float_as_uint(__uint_as_float(ov[i]) * alpha);
+          tmem_st16(tO + c * 16, ov);
+        }
+        tmem_wait_st();
+      }
+      if (j == 0) m_run = m_blk;
+      const uint64_t scale2 = f32x2_pack(p.scale_log2, p.scale_log2);
+      const uint64_t negm2 = f32x2_pack(-m_run, -m_run);
+      uint64_t l4[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) l4[i] = 0ull;
+      uint32_t pk[kBN / 2];
+      auto exps = [&](int i0, int i1) {  // pairs [i0, i1) of scores -> bf16 P
+#pragma unroll
+        for (int i = i0; i < i1; ++i) {
+          float t0, t1;
+          f32x2_unpack(f32x2_fma(f32x2_pack(sv[2 * i], sv[2 * i + 1]), scale2, negm2), t0, t1);
+          const float p0 = ex2_approx(t0);
+          const float p1 = ex2_approx(t1);
+          l4[i & 3] = f32x2_add(l4[i & 3], f32x2_pack(p0, p1));
+          pk[i] = pack_bf16x2(p0, p1);
+        }
+      };
+      // the first half of P goes out under the second half's exponentials,
+      // once PV(j-1) has read the previous P
+      exps(0, kBN / 4);
+      if (j > 0 && !mbar_wait(&pv_done[t], (j - 1) & 1, wc)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      tmem_st32(tP, *reinterpret_cast<uint32_t(*)[32]>(&pk[0]));
+      exps(kBN / 4, kBN / 2);
+      tmem_st32(tP + 32, *reinterpret_cast<uint32_t(*)[32]>(&pk[32]));
+      s_now = mbar_test(&s_full[t], (j + 1) & 1);
+      tmem_wait_st();
+      tc_fence_before();
+      mbar_arrive_warp(&p_full[t]);
+      float l8[8];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) f32x2_unpack(l4[i], l8[2 * i], l8[2 * i + 1]);
+      l_run += ((l8[0] + l8[1]) + (l8[2] + l8[3])) + ((l8[4] + l8[5]) + (l8[6] + l8[7]));
+    }
+    bool have_o =
+        ok && mbar_wait(&pv_done[t], (nblk - 1) & 1, wc) && !*abort_flag;
+    have_o = __all_sync(0xffffffffu, have_o);
+    tc_fence_after();
+
+    const size_t orow =
+        kLatent ? static_cast<size_t>(plane) * p.rows + grow
+                : (static_cast<size_t>(plane / p.heads) * p.rows + grow) * p.heads +
+                      plane % p.heads;
+    uint4* dst = reinterpret_cast<uint4*>(p.o + orow * DV);
+    // 32 columns of O, scaled, as bf16
+    auto store32 = [&](int c, const float (&v)[32], float inv) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        dst[c * 4 + i] = make_uint4(pack_bf16x2(v[8 * i] * inv, v[8 * i + 1] * inv),
+                                    pack_bf16x2(v[8 * i + 2] * inv, v[8 * i + 3] * inv),
+                                    pack_bf16x2(v[8 * i + 4] * inv, v[8 * i + 5] * inv),
+                                    pack_bf16x2(v[8 * i + 6] * inv, v[8 * i + 7] * inv));
+    };
+    auto load32 = [&](int c, float (&v)[32]) {
+      uint32_t ov[32];
+      tmem_ld32(tO + c * 32, ov);
+      tmem_wait_ld();
+#pragma unroll
+      for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(ov[i]);
+    };
+    if (n_split == 1) {
+      if (have_o) {
+        const float inv_l = 1.f / l_run;
+#pragma unroll 1
+        for (int c = 0; c < DV / 32; ++c) {
+          float v[32];
+          load32(c, v);
+          if (row_ok) store32(c, v, inv_l);
+        }
+      }
+    } else {
+      // phase 1: every CTA of the cluster is done with its shared memory
+      cluster_arrive_release();
+      cluster_wait_acquire();
+      const int per = nt * kBM / n_split;  // rows each CTA owns
+      const int lrow = t * kBM + r;
+      const int owner = lrow / per;
+      const int in_owner = lrow - owner * per;
+      if (have_o) {
+        const int slot = crank < owner ? crank : crank - 1;  // among the owner's n_split - 1
+        const uint32_t rec = dsmem_addr(
+            smem_u32(smem) + (slot * per + in_owner) * S::kRecord,
+            static_cast<uint32_t>(active ? owner : crank));
+        const bool send = owner != crank;
+#pragma unroll 1
+        for (int c = 0; c < DV / 32; ++c) {
+          float v[32];
+          load32(c, v);
+          if (send) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              dsmem_st_v4(rec + c * 128 + i * 16, v[4 * i], v[4 * i + 1], v[4 * i + 2],
+                          v[4 * i + 3]);
+          }
+        }
+        if (send) dsmem_st_v4(rec + DV * 4, m_run, l_run, 0.f, 0.f);
+      }
+      // phase 2: the records have arrived
+      cluster_arrive_release();
+      cluster_wait_acquire();
+      if (have_o) {
+        const bool mine = owner == crank;
+        const uint8_t* rec = smem + (mine ? in_owner : 0) * S::kRecord;
+        const int step = per * S::kRecord;
+        float m_all = m_run;
+        for (int s = 0; s < n_split - 1; ++s)
+          m_all = fmaxf(m_all, *reinterpret_cast<const float*>(rec + s * step + DV * 4));
+        const float w_own = ex2_approx(m_run - m_all);
+        float l_all = l_run * w_own;
+        for (int s = 0; s < n_split - 1; ++s) {
+          const float2 ml = *reinterpret_cast<const float2*>(rec + s * step + DV * 4);
+          l_all = fmaf(ml.y, ex2_approx(ml.x - m_all), l_all);
+        }
+        const float inv_l = 1.f / l_all;
+#pragma unroll 1
+        for (int c = 0; c < DV / 32; ++c) {
+          float v[32];
+          load32(c, v);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) v[i] *= w_own;
+          for (int s = 0; s < n_split - 1; ++s) {
+            const float w = ex2_approx(
+                *reinterpret_cast<const float*>(rec + s * step + DV * 4) - m_all);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const float4 x =
+                  *reinterpret_cast<const float4*>(rec + s * step + c * 128 + i * 16);
+              v[4 * i] = fmaf(x.x, w, v[4 * i]);
+              v[4 * i + 1] = fmaf(x.y, w, v[4 * i + 1]);
+              v[4 * i + 2] = fmaf(x.z, w, v[4 * i + 2]);
+              v[4 * i + 3] = fmaf(x.w, w, v[4 * i + 3]);
+            }
+          }
+          if (mine && row_ok) store32(c, v, inv_l);
+        }
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 3) {
+    tc_fence_after();
+    tmem_dealloc(tmem, 512);
+  }
+}
+
+// How a launch spreads its 256-row tiles over clusters: `whole` clusters per
+// plane hold one tile per CTA, the remaining tiles are split over the CTAs of
+// a cluster each.
+struct DualPlan {
+  int cl, whole;
+};
+
+// Clusters of 2, 4 and 8 CTAs that are resident at once.
+struct Resident {
+  int n[4];
+};
+
+template <int DR>
+cudaLaunchConfig_t dual_config(int cl, long long clusters, cudaStream_t stream,
+                               cudaLaunchAttribute (&attr)[2]) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(clusters * cl), 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = DualShape<DR>::kSmemBytes;
+  cfg.stream = stream;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cl;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see grid_dep_sync
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cfg;
+}
+
+template <int DR>
+Resident query_resident() {
+  Resident r = {};
+  for (int i = 1; i < 4; ++i) {
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = dual_config<DR>(1 << i, 1, nullptr, attr);
+    if (cudaOccupancyMaxActiveClusters(&r.n[i], mla_attn_dual_tc_kernel<DR>, &cfg) !=
+        cudaSuccess) {
+      cudaGetLastError();  // a failed query only disables that cluster size
+      r.n[i] = 0;
+    }
+  }
+  return r;
+}
+
+// The plan with the shortest estimated time. A CTA's time in key blocks: its
+// blocks, kFixed for its start and end, and kCombine when its tile is split.
+DualPlan plan_dual(int tiles, int planes, int nblk, const Resident& res) {
+  constexpr double kFixed = 4, kCombine = 3;
+  DualPlan best = {1, tiles};
+  double best_t = 1e300;
+  // pairs: whole clusters first, then split tiles on whichever pair is free
+  const long long slots = res.n[1];
+  if (slots > 0) {
+    const double ta = nblk + kFixed;
+    const double tb = (nblk + 1) / 2 + kFixed + kCombine;
+    const int pairs = tiles / 2;
+    for (int w = nblk >= 2 ? 0 : pairs; w <= pairs; ++w) {
+      const long long na = static_cast<long long>(w) * planes;
+      const long long nb = static_cast<long long>(tiles - 2 * w) * planes;
+      if (nblk < 2 && nb > 0) break;  // a single block cannot be split
+      // after the whole tiles, `late` pairs are free at t0 + ta, the others at t0
+      const double t0 = static_cast<double>(na / slots) * ta;
+      const long long late = na % slots;
+      double t = late > 0 ? t0 + ta : t0;
+      if (nb > 0) {
+        auto done_by = [&](double end) {  // split tiles finished by `end`
+          const double e = (end - t0) / tb + 1e-9, l = (end - t0 - ta) / tb + 1e-9;
+          return (slots - late) * static_cast<long long>(e) +
+                 (l > 0 ? late * static_cast<long long>(l) : 0);
+        };
+        double end = 1e300;
+        for (int c = 0; c < 2; ++c) {
+          long long k = nb / (2 * slots) + 1;
+          const double from = c == 0 ? t0 : t0 + ta;
+          while (done_by(from + static_cast<double>(k) * tb) < nb) ++k;
+          end = std::fmin(end, from + static_cast<double>(k) * tb);
+        }
+        t = std::fmax(t, end);
+      }
+      if (t < best_t) {
+        best_t = t;
+        best = {2, w};
+      }
+    }
+  }
+  for (int i = 2; i < 4; ++i) {
+    const int cl = 1 << i;
+    if (res.n[i] < 1 || nblk < cl) continue;
+    const long long n = static_cast<long long>(tiles) * planes;
+    const double t = static_cast<double>((n + res.n[i] - 1) / res.n[i]) *
+                     ((nblk + cl - 1) / cl + kFixed + kCombine);
+    if (t < best_t) {
+      best_t = t;
+      best = {cl, 0};
+    }
+  }
+  return best;
+}
+
+template <int DR>
+int launch_dual(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
+                DualKParams kp, cudaStream_t stream) {
+  using S = DualShape<DR>;
+  auto kern = mla_attn_dual_tc_kernel<DR>;
+  cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmemBytes);
+  if (e != cudaSuccess) {
+    set_last_cuda_error(e);
+    return MLA_ERR_CUDA;
+  }
+  static const Resident res = query_resident<DR>();
+  kp.tiles = (kp.rows + 2 * kBM - 1) / (2 * kBM);
+  const DualPlan plan =
+      plan_dual(kp.tiles, kp.planes, (kp.n_valid + kBN - 1) / kBN, res);
+  kp.cl = plan.cl;
+  kp.n_whole = plan.whole;
+  const long long clusters =
+      static_cast<long long>(kp.planes) * (plan.whole + kp.tiles - plan.whole * plan.cl);
+  if (clusters * plan.cl > 0x7fffffffll) return MLA_ERR_UNSUPPORTED;
+  cudaLaunchAttribute attr[2];
+  const cudaLaunchConfig_t cfg = dual_config<DR>(plan.cl, clusters, stream, attr);
+  e = cudaLaunchKernelEx(&cfg, kern, tm_q, tm_k, tm_v, kp);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    set_last_cuda_error(e);
+    return MLA_ERR_CUDA;
+  }
+  return MLA_OK;
+}
+
+template <int DR>
+int launch_latent(const AttnArgs& a) {
+  constexpr int DC = DV;
+  CUtensorMap tm_q, tm_c, tm_kr;
+  const unsigned long long rows = a.rows, slots = a.slots;
+  if (!encode_map_3d_bf16(&tm_q, a.q_c, DC, rows, a.batch, DC * 2ull, rows * DC * 2ull, 64, kBM,
+                          CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_map_3d_bf16(&tm_c, a.c, DC, a.n_valid, a.batch, DC * 2ull, slots * DC * 2ull, 64,
+                          kBN, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_map_3d_bf16(&tm_kr, a.kr, DR, a.n_valid, a.batch, DR * 2ull, slots * DR * 2ull, DR,
+                          kBN, DR == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B))
+    return MLA_ERR_CUDA;
+  DualKParams kp = {};
+  kp.q_r = static_cast<const __nv_bfloat16*>(a.q_r);
+  kp.q_pos = a.q_pos;
+  kp.rope = reinterpret_cast<const float2*>(a.rope);
+  kp.o = static_cast<__nv_bfloat16*>(a.o);
+  kp.rows = a.rows;
+  kp.heads = a.heads;
+  kp.n_valid = a.n_valid;
+  kp.rope_len = a.rope_len;
+  kp.pairs_t = a.pairs_t;
+  kp.pairs_h = a.pairs_h;
+  kp.scale_log2 = a.scale_log2;
+  kp.status = a.status;
+  kp.planes = a.batch;
+  return launch_dual<DR>(tm_q, tm_c, tm_kr, kp, a.stream);
+}
+
+}  // namespace
+
+int launch_attention_dual_tc(const AttnArgs& a) {
+  return a.d_r == 32 ? launch_latent<32>(a) : launch_latent<64>(a);
+}
+
+int launch_dense_dual_tc(const DenseArgs& a) {
+  constexpr int DH = DV;
+  CUtensorMap tm_q, tm_k, tm_v;
+  const unsigned long long slots = a.slots, nq = a.nq, wide = static_cast<unsigned long long>(a.heads) * DH,
+                           planes = static_cast<unsigned long long>(a.batch) * a.heads;
+  if (!encode_map_3d_bf16(&tm_q, a.q, wide, nq, a.batch, wide * 2, nq * wide * 2, 64, kBM,
+                          CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_map_3d_bf16(&tm_k, a.k, DH, a.n_valid, planes, DH * 2ull, slots * DH * 2ull, 64, kBN,
+                          CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_map_3d_bf16(&tm_v, a.v, DH, a.n_valid, planes, DH * 2ull, slots * DH * 2ull, 64, kBN,
+                          CU_TENSOR_MAP_SWIZZLE_128B))
+    return MLA_ERR_CUDA;
+  DualKParams kp = {};
+  kp.o = static_cast<__nv_bfloat16*>(a.o);
+  kp.rows = a.nq;
+  kp.heads = a.heads;
+  kp.n_valid = a.n_valid;
+  kp.scale_log2 = a.scale_log2;
+  kp.status = a.status;
+  kp.planes = a.batch * a.heads;
+  return launch_dual<0>(tm_q, tm_k, tm_v, kp, a.stream);
+}
+
+}  // namespace vmla

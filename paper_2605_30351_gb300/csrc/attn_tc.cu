@@ -632,7 +632,7 @@ int launch_tc_pick(const AttnArgs& a) {
 int launch_attention_tc(const AttnArgs& a) {
   if (a.d_r == 32) {
     switch (a.d_c) {
-      case 64: return launch_tc_pick<64, 32>(a);
+      case 64: return launch_attention_dual_tc(a);  // two row tiles per CTA
       case 128: return launch_tc_pick<128, 32>(a);
       case 192: return launch_tc_pick<192, 32>(a);
       case 256: return launch_tc_pick<256, 32>(a);  // Q in shared memory (faster than 64-key blocks)
@@ -641,7 +641,7 @@ int launch_attention_tc(const AttnArgs& a) {
     }
   } else if (a.d_r == 64) {
     switch (a.d_c) {
-      case 64: return launch_tc_pick<64, 64>(a);
+      case 64: return launch_attention_dual_tc(a);
       case 128: return launch_tc_pick<128, 64>(a);
       case 192: return launch_tc_pick<192, 64>(a);
       case 256: return launch_tc_pick<256, 64>(a);  // Q split between TMEM and shared memory

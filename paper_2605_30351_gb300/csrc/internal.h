@@ -139,6 +139,7 @@ struct DecompressArgs {
 
 // Each launcher returns MLA_OK, MLA_ERR_UNSUPPORTED or MLA_ERR_CUDA.
 int launch_attention_tc(const AttnArgs& a);
+int launch_attention_dual_tc(const AttnArgs& a);  // d_c 64, d_r 32 or 64
 int launch_attention_simt(const AttnArgs& a);
 int launch_append_tc(const AppendArgs& a);
 int launch_append_simt(const AppendArgs& a);
@@ -146,6 +147,7 @@ int launch_absorb(const AbsorbArgs& a);
 int launch_query_prologue(const QueryArgs& a);
 int launch_output_projection(const OutProjArgs& a);
 int launch_dense_attention_tc(const DenseArgs& a);
+int launch_dense_dual_tc(const DenseArgs& a);  // head_dim 64
 int launch_window_assemble(const WindowArgs& a);
 int launch_decompress(const DecompressArgs& a);
 int launch_wait_selftest(unsigned long long limit_ns, int* status, cudaStream_t stream);

@@ -1,0 +1,79 @@
+"""Attention with two row tiles per CTA (value width 64) where its launch plan
+changes: one or two row tiles, a single key block, blocks split over clusters
+of two, four and eight CTAs, whole and split tiles in one launch."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import mla_oracle as O
+from paper_2605_30351_gb300 import synth
+from paper_2605_30351_gb300 import videomla as V
+
+from test_gpu_dense import draw_dense
+from test_gpu_parity import assert_rows_close, f64, oracle_latent, small, upload_cache
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    V.load()
+    V.mla_device_status(clear=True)
+    yield
+    assert V.mla_device_status(clear=True) == V.MLA_OK
+
+
+@pytest.mark.parametrize("grid,frames,nq,batch,d_r", [
+    ((1, 1), 1, 1, 1, 32),      # 12 rows, one key: one row tile, one block, no cluster
+    ((8, 16), 1, 11, 1, 64),    # 132 rows: the second row tile has four; one full block
+    ((8, 16), 2, 22, 2, 32),    # two blocks: a pair splits one tile
+    ((10, 13), 4, 21, 1, 32),   # 252 rows, 520 keys: five blocks over a cluster of four
+    ((10, 13), 13, 21, 2, 64),  # 1690 keys: fourteen blocks over a cluster of eight
+    ((10, 13), 12, 150, 3, 32), # 1800 rows x 3: eight tiles per element
+])
+def test_split_key_blocks(grid, frames, nq, batch, d_r):
+    w = small(d_c=64, d_r=d_r, rope_pairs=(6, 5, 5) if d_r == 32 else (12, 10, 10),
+              rope_axis_dims=(44, 42, 42) if d_r == 32 else (64, 64, 64), grid_h=grid[0],
+              grid_w=grid[1], window_frames=frames, batch=batch)
+    cache, c, k = upload_cache(w, 21, frames)
+    q_c, q_r = synth.draw_queries(w, nq, 22, qc_std=2.0)  # scores that differ between splits
+    q_pos = synth.grid_positions(w, 0, frames)[:, -nq:].contiguous()
+    if q_pos.shape[1] < nq:
+        q_pos = q_pos[:, :1].repeat(1, nq, 1).contiguous()
+    o = torch.empty(batch, nq, w.heads, 64, dtype=torch.bfloat16, device="cuda")
+    V.mla_attention_forward(cache, q_c.cuda(), q_r.cuda(), q_pos.cuda(), o)
+    torch.cuda.synchronize()
+    ref = oracle_latent(w, q_c, q_r, q_pos, c, k, cache.n_valid())
+    assert_rows_close(f64(o), ref, "split key blocks")
+
+
+def test_whole_and_split_tiles_agree_across_the_grid():
+    """More tiles than pairs of SMs: whole tiles first, split ones after; rows
+    of the first and the last tile and of the border between them."""
+    w = synth.workload("wan", d_c=64, window_frames=3, last_frame=3)
+    cache, c, k = upload_cache(w, 23, 3)
+    nq = w.chunk_tokens
+    q_c, q_r = synth.draw_queries(w, nq, 24)
+    q_pos = synth.grid_positions(w, 0, 3)
+    o = torch.empty(1, nq, w.heads, 64, dtype=torch.bfloat16, device="cuda")
+    V.mla_attention_forward(cache, q_c.cuda(), q_r.cuda(), q_pos.cuda(), o)
+    torch.cuda.synchronize()
+    tok = np.unique(np.concatenate([np.arange(0, nq, 307), np.arange(nq - 12, nq)]))
+    ref = oracle_latent(w, q_c[:, tok], q_r[:, tok], q_pos[:, tok], c, k, cache.n_valid())
+    assert_rows_close(f64(o[:, tok]), ref, "whole and split tiles")
+
+
+@pytest.mark.parametrize("nq,slots,n_valid,batch", [
+    (1, 128, 128, 1), (257, 300, 300, 1), (130, 2000, 1921, 2)])
+def test_dense_width_64(nq, slots, n_valid, batch):
+    w = synth.workload("tiny", batch=batch, head_dim=64)
+    q, k, v = draw_dense(w, nq, slots, 25)
+    o = torch.empty_like(q, device="cuda")
+    V.mla_dense_attention_forward(V.make_config(w), q.cuda(), k.cuda(), v.cuda(), n_valid, o)
+    torch.cuda.synchronize()
+    ref = np.stack([O.dense_attention(f64(q[b]), f64(k[b, :, :n_valid]), f64(v[b, :, :n_valid]),
+                                      w.head_dim) for b in range(batch)])
+    assert_rows_close(f64(o), ref, "dense width 64")
