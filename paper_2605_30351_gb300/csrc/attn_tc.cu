@@ -8,7 +8,8 @@
 //     P   = exp2(S * log2(e)/sqrt(d_h) - m)        online, fp32
 //     O  += P . c                                  N = d_c (192), latent output
 // One CTA owns 128 rows (one TMEM lane each) and walks the window in blocks
-// of BN keys (128; 64 for d_c = 512):
+// of 128 keys; this file holds the widths whose Q fits in TMEM beside S, P and
+// O (d_c = 128 and 192; other kernels serve the narrower and wider ones):
 //   warp 0     TMA producer: [c | k] tiles into a ring of shared-memory
 //              stages (c with 128-byte swizzle, k with 64-byte swizzle).
 //              CTAs run in pairs (a cluster of two consecutive row tiles of
@@ -28,25 +29,11 @@
 //              it), writes P_j (bf16) once PV_{j-1} has read the previous P,
 //              rescales O in TMEM only when its running max grows by more
 //              than 2^8, and finally writes O / l as bf16.
-// TMEM columns: S [0,BN) P [BN,3BN/2) O [3BN/2,3BN/2+d_c) Q [3BN/2+d_c, +(d_c+d_r)/2).
-// When Q does not fit there (d_c = 256) it stays in shared memory (TMA-loaded
-// q_c plus the rotated q_r stored by the softmax warps) and QK reads it there;
-// where that leaves room for fewer than two key stages ((256, 64)), the first
-// q_c columns go to the TMEM left after O and QK mixes TMEM and shared-memory
-// A operands.
-// d_c = 512: a 512-column fp32 O alone fills TMEM, so each 128-row tile runs
-// on a cluster of two CTAs, each owning 256 output columns (DV). Both score
-// the full [c | k] tile (QK is computed twice, PV once: 2112 useful of 3200
-// issued FLOP per row-key pair) and share every key tile through the same
-// multicast as the row-tile pairs above; each keeps the q_c columns that fit
-// next to S, P and its O half in TMEM (320) and the rest of Q in shared
-// memory, so QK mixes TMEM- and shared-memory A operands.
+// TMEM columns: S [0,128) P [128,192) O [192,192+d_c) Q [192+d_c, +(d_c+d_r)/2).
 // What bounds it (Wan shape): the tensor pipe at d_c = 192 (92 % active; the
 // GPU's power cap in long runs), a block's softmax (~1200 cycles beside 1152 of
-// MMAs) at d_c = 128, the wait for keys at d_c = 256 (two stages beside Q) and
-// the doubled score at 512. Issuing from converged warps and settling the
-// rescale before the exponentials took d_c = 128 from 579 to 549 us, (256, 64)
-// from 1325 to 1260 us and (512, 64) from 4341 to 4131 us, bit-identical.
+// MMAs) at d_c = 128. Issuing from converged warps and settling the rescale
+// before the exponentials took d_c = 128 from 579 to 549 us, bit-identical.
 // The V operand is the first d_c columns of the same key tile read MN-major,
 // so the cache is never expanded into per-head keys or values.
 #include <cmath>
@@ -58,55 +45,35 @@ namespace vmla {
 namespace {
 
 constexpr int kBM = 128;       // rows per CTA = TMEM lanes
+constexpr int kBN = 128;       // keys per block
 constexpr int kThreads = 224;  // 7 warps
 constexpr float kRescaleLog2 = 8.0f;
 
-template <int DC, int DR, int BN, int DV = DC>
+template <int DC, int DR>
 struct AttnShape {
-  static constexpr int kBN = BN;                   // keys per block
   static constexpr int DK = DC + DR;
-  static constexpr int kSplit = DC / DV;           // CTAs per row tile, DV output columns each
   static constexpr int kTileBytes = kBN * DK * 2;  // one key stage
-  static constexpr int kCBox = kBN * 128;          // one [BN keys x 64 columns] box of c
+  static constexpr int kCBox = kBN * 128;          // one [128 keys x 64 columns] box of c
   static constexpr int kKrOff = DC * kBN * 2;      // byte offset of the d_r columns in a tile
   static constexpr int kTmemS = 0;
   static constexpr int kTmemP = kBN;               // bf16 P: two values per column
   static constexpr int kTmemO = kBN + kBN / 2;
-  static constexpr int kTmemQ = kTmemO + DV;
+  static constexpr int kTmemQ = kTmemO + DC;
   static constexpr int kBarBytes = 256;
-  static constexpr int kSmemCap = 232448;
-  static constexpr bool kQinTmem = kTmemQ + DK / 2 <= 512;
-  // Where Q lives when it does not fit in TMEM: all of it in shared memory
-  // if two key stages still fit beside it (SS score MMAs measured faster
-  // than a TS/SS mix there), else the leading 64-column boxes of q_c that
-  // fit go to TMEM and the rest of Q to shared memory
-  static constexpr bool kQSmemFits = 1024 + kBarBytes + kBM * DK * 2 + 2 * kTileBytes <= kSmemCap;
-  static constexpr int kQcTmem =
-      kQinTmem ? DC : (kQSmemFits ? 0 : ((512 - kTmemQ) * 2 / 64) * 64);
-  static constexpr int kQcSmem = DC - kQcTmem;
-  // shared-memory Q tile: [128 rows x 64 columns] boxes of q_c, then q_r
-  static constexpr int kQKrOff = kQcSmem * kBM * 2;
-  static constexpr int kQBytes = kQinTmem ? 0 : kQKrOff + kBM * DR * 2;
-  static constexpr int kFit = (kSmemCap - 1024 - kBarBytes - kQBytes) / kTileBytes;
-  static constexpr int kMaxStages = 6;
-  static constexpr int kStages = kFit > kMaxStages ? kMaxStages : kFit;
-  static constexpr int kSmemBytes = 1024 + kQBytes + kTileBytes * kStages + kBarBytes;
+  static constexpr int kFit = (232448 - 1024 - kBarBytes) / kTileBytes;
+  static constexpr int kStages = kFit > 6 ? 6 : kFit;
+  static constexpr int kSmemBytes = 1024 + kTileBytes * kStages + kBarBytes;
   static constexpr uint32_t kTmemCols = 512;
   static constexpr uint32_t kKrSw = DR == 32 ? kSw64 : kSw128;
   static constexpr uint32_t kKrRow = DR * 2;      // bytes per row of the d_r block
   static constexpr uint32_t kKrSbo = 8 * kKrRow;  // one 8-row swizzle atom
   static constexpr uint32_t kIdescQK = idesc_bf16_f32(kBM, kBN, false, false);
-  static constexpr uint32_t kIdescPV = idesc_bf16_f32(kBM, DV, false, true);
-  static_assert(BN == 128 || BN == 64, "key block: 128 or 64");
-  static_assert(DC % 64 == 0 && DC >= 64 && DV % 64 == 0 && DV <= 256 && DC % DV == 0,
-                "d_c: multiple of 64; each CTA's output columns: multiple of 64 up to 256");
-  static_assert(kSplit == 1 || kSplit == 2, "output split over at most two CTAs");
+  static constexpr uint32_t kIdescPV = idesc_bf16_f32(kBM, DC, false, true);
+  static_assert(DC % 64 == 0 && DC >= 64 && DC <= 256, "d_c: multiple of 64");
   static_assert(DR == 32 || DR == 64, "d_r: 32 or 64");
-  static_assert(kTmemO + DV <= 512 && kTmemQ + kQcTmem / 2 <= 512,
-                "S, P, O and the TMEM part of Q must fit in 512 TMEM columns");
+  static_assert(kTmemQ + DK / 2 <= 512, "S, P, O and Q must fit in 512 TMEM columns");
   static_assert(kStages >= 2, "at least two key stages must fit in shared memory");
-  static_assert(kTileBytes % 1024 == 0 && kKrOff % 1024 == 0 && kQKrOff % 1024 == 0,
-                "swizzle-atom alignment");
+  static_assert(kTileBytes % 1024 == 0 && kKrOff % 1024 == 0, "swizzle-atom alignment");
 };
 
 struct AttnKParams {
@@ -120,26 +87,20 @@ struct AttnKParams {
   int* status;
 };
 
-template <int DC, int DR, int CL, int BN, int DV>
+template <int DC, int DR, int CL>
 __global__ void __launch_bounds__(kThreads, 1)
-    mla_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_qc,
-                       const __grid_constant__ CUtensorMap tm_c,
+    mla_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_c,
                        const __grid_constant__ CUtensorMap tm_kr, const AttnKParams p) {
-  using S = AttnShape<DC, DR, BN, DV>;
-  constexpr int kBN = S::kBN;
+  using S = AttnShape<DC, DR>;
   constexpr int NST = S::kStages;
   constexpr uint16_t kPair = static_cast<uint16_t>((1u << CL) - 1u);  // every CTA of the cluster
   static_assert(CL == 1 || CL == 2, "clusters of one or two CTAs");
-  // a split row tile's CTAs form the cluster: both read every key tile
-  static_assert(S::kSplit == 1 || CL == S::kSplit, "split CTAs share one cluster");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem_1024(smem_raw);
-  uint8_t* sQ = smem;  // only when Q stays in shared memory
-  uint8_t* sKV = smem + S::kQBytes;
+  uint8_t* sKV = smem;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sKV + NST * S::kTileBytes);
-  uint64_t* q_tma_full = bars + 0;
-  uint64_t* q_ready = bars + 1;
-  uint64_t* kv_full = bars + 2;
+  uint64_t* q_ready = bars;
+  uint64_t* kv_full = bars + 1;
   uint64_t* kv_empty = kv_full + NST;
   uint64_t* s_full = kv_empty + NST;
   uint64_t* s_free = s_full + 1;
@@ -152,14 +113,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.y;
-  const int tile = blockIdx.x / S::kSplit;
-  const int vpart = blockIdx.x - tile * S::kSplit;  // which DV output columns
-  const int row0 = tile * kBM;
+  const int row0 = blockIdx.x * kBM;
   const int nblk = (p.n_valid + kBN - 1) / kBN;
   const WaitCtx wc{abort_flag, p.status};
 
   if (threadIdx.x == 0) {
-    mbar_init(q_tma_full, 1);
     mbar_init(q_ready, 4);  // one arrival per softmax warp, and so below
     for (int s = 0; s < NST; ++s) {
       mbar_init(&kv_full[s], 1);
@@ -192,12 +150,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       tma_prefetch_desc(&tm_c);
       tma_prefetch_desc(&tm_kr);
-      if constexpr (!S::kQinTmem) {
-        tma_prefetch_desc(&tm_qc);
-        mbar_arrive_expect_tx(q_tma_full, S::kQcSmem * kBM * 2);
-        for (int cb = 0; cb < S::kQcSmem / 64; ++cb)
-          tma_load_3d(sQ + cb * 16384, &tm_qc, q_tma_full, S::kQcTmem + cb * 64, row0, b);
-      }
       int issued = 0;
       for (int j = 0; j < nblk; ++j) {
         const int st = j % NST;
@@ -223,7 +175,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int st = 0; st < NST && st < nblk && !*abort_flag; ++st)
         mbar_wait(&kv_empty[st], (((nblk - st + NST - 1) / NST) - 1) & 1, wc);
       if (*abort_flag) {  // let every copy this CTA started land before exit
-        if constexpr (!S::kQinTmem) mbar_wait_drain(q_tma_full, 0, p.status);
         for (int u = issued > NST ? issued - NST : 0; u < issued; ++u)
           mbar_wait_drain(&kv_full[u % NST], (u / NST) & 1, p.status);
       }
@@ -233,9 +184,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ------------------------------------------------------ QK^T issuer
     // the whole warp walks the loop; one lane issues (see elect_one)
     bool ok = mbar_wait_warp(q_ready, 0, wc);
-    if constexpr (!S::kQinTmem) ok = ok && mbar_wait_warp(q_tma_full, 0, wc);
-    const uint64_t qd = sdesc(smem_u32(sQ), 16, 1024, kSw128);
-    const uint64_t qrd = sdesc(smem_u32(sQ) + S::kQKrOff, 16, S::kKrSbo, S::kKrSw);
     const uint64_t kd = sdesc(smem_u32(sKV), 16, 1024, kSw128);
     const uint64_t krd = sdesc(smem_u32(sKV) + S::kKrOff, 16, S::kKrSbo, S::kKrSw);
     for (int j = 0; ok && j < nblk; ++j) {
@@ -250,23 +198,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int cb = 0; cb < DC / 64; ++cb)
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const uint64_t bd = kd + ko + ((cb * S::kCBox + k * 32) >> 4);
-            const uint32_t acc = (cb | k) != 0 ? 1u : 0u;
-            if (cb < S::kQcTmem / 64)  // resolved at compile time (unrolled)
-              umma_ts(tmem + S::kTmemS, tmem + S::kTmemQ + (cb * 4 + k) * 8, bd, S::kIdescQK, acc);
-            else
-              umma_ss(tmem + S::kTmemS, qd + (((cb - S::kQcTmem / 64) * 16384 + k * 32) >> 4), bd,
-                      S::kIdescQK, acc);
-          }
+          for (int k = 0; k < 4; ++k)
+            umma_ts(tmem + S::kTmemS, tmem + S::kTmemQ + (cb * 4 + k) * 8,
+                    kd + ko + ((cb * S::kCBox + k * 32) >> 4), S::kIdescQK,
+                    (cb | k) != 0 ? 1u : 0u);
 #pragma unroll
-        for (int k = 0; k < DR / 16; ++k) {
-          if constexpr (S::kQinTmem)
-            umma_ts(tmem + S::kTmemS, tmem + S::kTmemQ + DC / 2 + k * 8, krd + ko + k * 2,
-                    S::kIdescQK, 1u);
-          else
-            umma_ss(tmem + S::kTmemS, qrd + k * 2, krd + ko + k * 2, S::kIdescQK, 1u);
-        }
+        for (int k = 0; k < DR / 16; ++k)
+          umma_ts(tmem + S::kTmemS, tmem + S::kTmemQ + DC / 2 + k * 8, krd + ko + k * 2,
+                  S::kIdescQK, 1u);
         umma_commit(s_full);
       }
       __syncwarp();
@@ -279,9 +218,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == 6) {
     // --------------------------------------------------------- PV issuer
     bool ok = true;
-    // V = this CTA's DV of the first d_c columns of block i's stage (MN-major)
-    const uint64_t vd =
-        sdesc(smem_u32(sKV) + vpart * (DV / 64) * S::kCBox, S::kCBox, 1024, kSw128);
+    // V = the first d_c columns of block i's stage (MN-major)
+    const uint64_t vd = sdesc(smem_u32(sKV), S::kCBox, 1024, kSw128);
     for (int i = 0; ok && i < nblk; ++i) {
       ok = mbar_wait_warp(p_full, i & 1, wc);  // O += P_i V_i
       if (!ok) break;
@@ -347,43 +285,27 @@ __global__ void __launch_bounds__(kThreads, 1)
           w[i] = pack_bf16x2(x0 * cs.x - x1 * cs.y, x0 * cs.y + x1 * cs.x);
         }
       }
-      if constexpr (S::kQcTmem > 0) {
-        // TMEM holds the MMA's A operand row-major: column c = elements 2c, 2c+1
-        const uint4* qsrc = reinterpret_cast<const uint4*>(
-            p.q_c + (static_cast<size_t>(b) * p.rows + (row_ok ? grow : 0)) * DC);
+      // TMEM holds the MMA's A operand row-major: column c = elements 2c, 2c+1
+      const uint4* qsrc = reinterpret_cast<const uint4*>(
+          p.q_c + (static_cast<size_t>(b) * p.rows + (row_ok ? grow : 0)) * DC);
 #pragma unroll
-        for (int c = 0; c < S::kQcTmem / 64; ++c) {
-          uint32_t qw[32];
+      for (int c = 0; c < DC / 64; ++c) {
+        uint32_t qw[32];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const uint4 v = row_ok ? __ldg(qsrc + c * 8 + i) : make_uint4(0u, 0u, 0u, 0u);
-            qw[4 * i + 0] = v.x;
-            qw[4 * i + 1] = v.y;
-            qw[4 * i + 2] = v.z;
-            qw[4 * i + 3] = v.w;
-          }
-          tmem_st32(tmem + t_lane + S::kTmemQ + c * 32, qw);
+        for (int i = 0; i < 8; ++i) {
+          const uint4 v = row_ok ? __ldg(qsrc + c * 8 + i) : make_uint4(0u, 0u, 0u, 0u);
+          qw[4 * i + 0] = v.x;
+          qw[4 * i + 1] = v.y;
+          qw[4 * i + 2] = v.z;
+          qw[4 * i + 3] = v.w;
         }
+        tmem_st32(tmem + t_lane + S::kTmemQ + c * 32, qw);
       }
-      if constexpr (S::kQinTmem) {
 #pragma unroll
-        for (int c = 0; c < DR / 32; ++c)
-          tmem_st16(tmem + t_lane + S::kTmemQ + DC / 2 + c * 16, w + c * 16);
-      } else {
-        // the same 16-byte-chunk swizzle the TMA applies to the q_c part
-        uint8_t* krow = sQ + S::kQKrOff + r * S::kKrRow;
-#pragma unroll
-        for (int c = 0; c < DR / 8; ++c) {
-          const int phys = DR == 32 ? (c ^ ((r >> 1) & 3)) : (c ^ (r & 7));
-          *reinterpret_cast<uint4*>(krow + phys * 16) =
-              make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
-        }
-        fence_proxy_async_smem();
-      }
-      if constexpr (S::kQcTmem > 0) {
-        tmem_wait_st();
-        tc_fence_before();
-      }
+      for (int c = 0; c < DR / 32; ++c)
+        tmem_st16(tmem + t_lane + S::kTmemQ + DC / 2 + c * 16, w + c * 16);
+      tmem_wait_st();
+      tc_fence_before();
       mbar_arrive_warp(q_ready);
     }
 
@@ -423,10 +345,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int c = 8; c + 16 <= kBN; c += 16)
 #pragma unroll
         for (int i = 0; i < 8; ++i) m8[i] = fmax3(m8[i], sv[c + i], sv[c + 8 + i]);
-      if constexpr ((kBN - 8) % 16 != 0) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) m8[i] = fmaxf(m8[i], sv[kBN - 8 + i]);
-      }
+      for (int i = 0; i < 8; ++i) m8[i] = fmaxf(m8[i], sv[kBN - 8 + i]);
       const float mx = fmaxf(fmaxf(fmaxf(m8[0], m8[1]), fmaxf(m8[2], m8[3])),
                              fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7])));
       const float m_blk = mx * p.scale_log2;
@@ -446,7 +366,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         tc_fence_after();
 #pragma unroll 1
-        for (int c = 0; c < DV / 16; ++c) {
+        for (int c = 0; c < DC / 16; ++c) {
           uint32_t ov[16];
           tmem_ld16(tmem + t_lane + S::kTmemO + c * 16, ov);
           tmem_wait_ld();
@@ -469,10 +389,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int i = 0; i < 4; ++i) l4[i] = 0ull;
       uint32_t pk[kBN / 2];
       auto store_p = [&](int i0) {  // half of P's words, from pair i0
-        if constexpr (kBN == 128)
-          tmem_st32(tmem + t_lane + S::kTmemP + i0, *reinterpret_cast<uint32_t(*)[32]>(&pk[i0]));
-        else
-          tmem_st16(tmem + t_lane + S::kTmemP + i0, &pk[i0]);
+        tmem_st32(tmem + t_lane + S::kTmemP + i0, *reinterpret_cast<uint32_t(*)[32]>(&pk[i0]));
       };
       auto exps = [&](int i0, int i1) {  // pairs [i0, i1) of scores -> bf16 P
 #pragma unroll
@@ -508,16 +425,15 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     // O / l as bf16: each thread stages its row densely in the key stages
     // (free once the last PV is done: every key tile, the peer's multicast
-    // halves included, has landed and been read) and the rows leave shared
-    // memory by bulk copy, the whole tile at once when its rows are
-    // consecutive rows of o (DV = d_c).
+    // halves included, has landed and been read), and the tile leaves shared
+    // memory by one bulk copy: its rows are consecutive rows of o.
     const bool have_o = ok && mbar_wait(pv_done, (nblk - 1) & 1, wc);
-    uint8_t* srow = sKV + r * DV * 2;
+    uint8_t* srow = sKV + r * DC * 2;
     if (have_o) {
       tc_fence_after();
       const float inv_l = 1.f / l_run;
 #pragma unroll 1
-      for (int sg = 0; sg < DV / 64; ++sg) {
+      for (int sg = 0; sg < DC / 64; ++sg) {
         uint32_t va[32], vb[32];
         tmem_ld32(tmem + t_lane + S::kTmemO + sg * 64, va);
         tmem_ld32(tmem + t_lane + S::kTmemO + sg * 64 + 32, vb);
@@ -534,20 +450,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     fence_proxy_async_smem();
-    if constexpr (DV == DC) {
-      asm volatile("bar.sync 1, 128;" ::: "memory");  // the four softmax warps
-      // the tile's rows below p.rows; none in the CTA that only pads the grid
-      // to whole clusters (an odd number of row tiles)
-      const int valid = min(kBM, p.rows - row0);
-      if (r == 0 && have_o && !*abort_flag && valid > 0) {
-        bulk_store(p.o + (static_cast<size_t>(b) * p.rows + row0) * DC, sKV, valid * DC * 2);
-        bulk_commit();
-        bulk_wait_read_all();  // the staged rows must outlive the copy's reads
-      }
-    } else if (have_o && row_ok) {
-      bulk_store(p.o + (static_cast<size_t>(b) * p.rows + grow) * DC + vpart * DV, srow, DV * 2);
+    asm volatile("bar.sync 1, 128;" ::: "memory");  // the four softmax warps
+    // the tile's rows below p.rows; none in the CTA that only pads the grid
+    // to whole clusters (an odd number of row tiles)
+    const int valid = min(kBM, p.rows - row0);
+    if (r == 0 && have_o && !*abort_flag && valid > 0) {
+      bulk_store(p.o + (static_cast<size_t>(b) * p.rows + row0) * DC, sKV, valid * DC * 2);
       bulk_commit();
-      bulk_wait_read_all();
+      bulk_wait_read_all();  // the staged rows must outlive the copy's reads
     }
   }
 
@@ -561,20 +471,18 @@ __global__ void __launch_bounds__(kThreads, 1)
   if constexpr (CL > 1) cluster_sync();
 }
 
-template <int DC, int DR, int CL, int BN, int DV = DC>
+template <int DC, int DR, int CL>
 int launch_tc(const AttnArgs& a) {
-  using S = AttnShape<DC, DR, BN, DV>;
-  CUtensorMap tm_qc, tm_c, tm_kr;
-  const unsigned long long rows = a.rows, slots = a.slots;
-  if (!encode_map_3d_bf16(&tm_qc, a.q_c, DC, rows, a.batch, DC * 2ull, rows * DC * 2ull, 64,
-                          kBM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !encode_map_3d_bf16(&tm_c, a.c, DC, a.n_valid, a.batch, DC * 2ull, slots * DC * 2ull, 64,
-                          S::kBN, CU_TENSOR_MAP_SWIZZLE_128B) ||
+  using S = AttnShape<DC, DR>;
+  CUtensorMap tm_c, tm_kr;
+  const unsigned long long slots = a.slots;
+  if (!encode_map_3d_bf16(&tm_c, a.c, DC, a.n_valid, a.batch, DC * 2ull, slots * DC * 2ull, 64,
+                          kBN, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !encode_map_3d_bf16(&tm_kr, a.kr, DR, a.n_valid, a.batch, DR * 2ull, slots * DR * 2ull, DR,
-                          S::kBN,
+                          kBN,
                           DR == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B))
     return MLA_ERR_CUDA;
-  auto kern = mla_attn_tc_kernel<DC, DR, CL, BN, DV>;
+  auto kern = mla_attn_tc_kernel<DC, DR, CL>;
   cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmemBytes);
   if (e != cudaSuccess) {
@@ -597,8 +505,7 @@ int launch_tc(const AttnArgs& a) {
   kp.status = a.status;
   const int tiles = (a.rows + kBM - 1) / kBM;
   cudaLaunchConfig_t cfg = {};
-  // pairs stay within a batch row; a split tile's CTAs are adjacent
-  cfg.gridDim = dim3((tiles * S::kSplit + CL - 1) / CL * CL, a.batch, 1);
+  cfg.gridDim = dim3((tiles + CL - 1) / CL * CL, a.batch, 1);  // pairs stay within a batch row
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = S::kSmemBytes;
   cfg.stream = a.stream;
@@ -611,7 +518,7 @@ int launch_tc(const AttnArgs& a) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  e = cudaLaunchKernelEx(&cfg, kern, tm_qc, tm_c, tm_kr, kp);
+  e = cudaLaunchKernelEx(&cfg, kern, tm_c, tm_kr, kp);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_last_cuda_error(e);
@@ -622,34 +529,23 @@ int launch_tc(const AttnArgs& a) {
 
 // Pairs of CTAs share every key tile through TMA multicast; a single row tile
 // per batch element runs alone.
-template <int DC, int DR, int BN = 128>
+template <int DC, int DR>
 int launch_tc_pick(const AttnArgs& a) {
-  return (a.rows + kBM - 1) / kBM >= 2 ? launch_tc<DC, DR, 2, BN>(a) : launch_tc<DC, DR, 1, BN>(a);
+  return (a.rows + kBM - 1) / kBM >= 2 ? launch_tc<DC, DR, 2>(a) : launch_tc<DC, DR, 1>(a);
 }
 
 }  // namespace
 
 int launch_attention_tc(const AttnArgs& a) {
-  if (a.d_r == 32) {
-    switch (a.d_c) {
-      case 64: return launch_attention_dual_tc(a);  // two row tiles per CTA
-      case 128: return launch_tc_pick<128, 32>(a);
-      case 192: return launch_tc_pick<192, 32>(a);
-      case 256: return launch_tc_pick<256, 32>(a);  // Q in shared memory (faster than 64-key blocks)
-      case 512: return launch_tc<512, 32, 2, 64, 256>(a);  // output split over a CTA pair
-      default: break;
-    }
-  } else if (a.d_r == 64) {
-    switch (a.d_c) {
-      case 64: return launch_attention_dual_tc(a);
-      case 128: return launch_tc_pick<128, 64>(a);
-      case 192: return launch_tc_pick<192, 64>(a);
-      case 256: return launch_tc_pick<256, 64>(a);  // Q split between TMEM and shared memory
-      case 512: return launch_tc<512, 64, 2, 64, 256>(a);
-      default: break;
-    }
+  if (a.d_r != 32 && a.d_r != 64) return MLA_ERR_UNSUPPORTED;
+  switch (a.d_c) {
+    case 64: return launch_attention_dual_tc(a);  // two row tiles per CTA
+    case 128: return a.d_r == 32 ? launch_tc_pick<128, 32>(a) : launch_tc_pick<128, 64>(a);
+    case 192: return a.d_r == 32 ? launch_tc_pick<192, 32>(a) : launch_tc_pick<192, 64>(a);
+    case 256:
+    case 512: return launch_attention_wide_tc(a);  // paired-SM MMAs
+    default: return MLA_ERR_UNSUPPORTED;
   }
-  return MLA_ERR_UNSUPPORTED;
 }
 
 }  // namespace vmla

@@ -1,0 +1,568 @@
+// Absorbed-form MLA attention for wide latents (d_c = 256 and 512) on the
+// sm_103a tensor cores, with paired-SM MMAs (tcgen05 cta_group::2).
+//
+// Paper: Eq. (score) and App. E, as in the kernel for narrower latents: rows
+// are (token, head) pairs, every row scores the same cached latents,
+//     S = [q_c | RoPE(q_r)] . [c | k]^T,  P = exp2(S * log2(e)/sqrt(d_h) - m),
+//     O += P . c
+// A cluster of two CTAs takes 256 rows, 128 each, as M = 256 MMAs: each CTA
+// holds its rows' Q, P, S and O, and half of every key operand (64 of a block's
+// 128 keys for the score, 128 of the 256 value columns for PV). With one CTA
+// per 128 rows the wide latents left room for two key tiles beside Q, and the
+// score MMAs waited for their keys; 64-key blocks, which d_c = 512 needed to
+// fit, cost 45-48 cycles an MMA for 32 cycles of math. Halves of the operands
+// leave room for K boxes and V tiles in rings of their own and for 128-key
+// blocks at both widths, and halve the shared-memory reads of B. Wan shape,
+// same box: (256, 32) 1166 -> 938 us, (256, 64) 1325 -> 992 us, (512, 32) 4250
+// -> 3262 us, (512, 64) 4360 -> 3360 us (1190 useful, 1800 issued TFLOP/s, the
+// tensor pipe 89 % busy). In long runs both widths sit at the GPU's power cap.
+// d_c = 512: O of 512 fp32 columns would fill TMEM, so a row tile's output is
+// split over two clusters of 256 columns each (DV); both compute the full
+// score (3200 issued FLOP for 2112 useful per row-key pair at d_r = 32).
+//   warp 0     TMA producer of this CTA's halves: K boxes [64 keys x 64] (the
+//              last box of a block: the positional key), V tiles [128 x 128]
+//   warp 1     allocates TMEM; in the even CTA issues the MMAs
+//   warps 2-5  load Q's TMEM part (64 columns of q_c and the rotated q_r), then
+//              the online softmax: thread = row
+// TMEM: S [0,128) P [128,192) O [192,448) Q [448,512).
+#include <cmath>
+
+#include "internal.h"
+#include "ptx_sm103.cuh"
+
+namespace vmla {
+namespace {
+
+constexpr int kBM = 128;       // rows per CTA = TMEM lanes
+constexpr int kBN = 128;       // keys per block
+constexpr int DV = 256;        // output columns per cluster
+constexpr int kThreads = 192;  // 6 warps
+constexpr float kRescaleLog2 = 8.0f;
+
+template <int DC, int DR>
+struct WideShape {
+  static constexpr int kSplit = DC / DV;         // clusters per row tile
+  static constexpr int kCBoxes = DC / 64;        // K boxes of c per block
+  static constexpr int kBoxes = kCBoxes + 1;     // and one of k^R
+  static constexpr int kKBox = (kBN / 2) * 128;  // [64 keys x 64 columns]
+  static constexpr int kKrBytes = (kBN / 2) * DR * 2;
+  static constexpr int kVBox = kBN * 128;        // [128 keys x 64 columns]
+  static constexpr int kVTile = 2 * kVBox;       // this CTA's 128 value columns
+  static constexpr int kQBox = kBM * 128;        // [128 rows x 64 columns]
+  static constexpr int kQBytes = (kCBoxes - 1) * kQBox;  // q_c columns 64.., the rest in TMEM
+  static constexpr int kBarBytes = 512;
+  static constexpr int kFree = 232448 - 1024 - kBarBytes - kQBytes;
+  static constexpr int kVStages = kFree >= 3 * kVTile + 10 * kKBox ? 3 : 2;
+  static constexpr int kKFit = (kFree - kVStages * kVTile) / kKBox;
+  static constexpr int kKStages = kKFit > 12 ? 12 : kKFit;
+  static constexpr int kSmemBytes =
+      1024 + kQBytes + kVStages * kVTile + kKStages * kKBox + kBarBytes;
+  static constexpr int kTmemP = kBN, kTmemO = kBN + kBN / 2, kTmemQ = kTmemO + DV;
+  static constexpr uint32_t kKrSw = DR == 32 ? kSw64 : kSw128;
+  static constexpr uint32_t kKrSbo = 8 * DR * 2;
+  static constexpr uint32_t kIdescQK = idesc_bf16_f32(2 * kBM, kBN, false, false);
+  static constexpr uint32_t kIdescPV = idesc_bf16_f32(2 * kBM, DV, false, true);
+  static_assert(DC == 256 || DC == 512, "wide latents");
+  static_assert(DR == 32 || DR == 64, "d_r: 32 or 64");
+  static_assert(kTmemQ + 32 + DR / 2 <= 512, "TMEM budget");
+  static_assert(kKStages >= 5, "K boxes in flight");
+  static_assert(kBM * DV * 2 <= kVStages * kVTile, "output rows staged in the V ring");
+  static_assert(2 * (kKStages + kVStages) + 8 <= kBarBytes / 8 - 1, "barriers, slot, abort flag");
+};
+
+struct WideKParams {
+  const __nv_bfloat16* q_c;
+  const __nv_bfloat16* q_r;
+  const int* q_pos;
+  const float2* rope;
+  __nv_bfloat16* o;
+  int rows, heads, n_valid, rope_len, pairs_t, pairs_h;
+  float scale_log2;
+  int* status;
+};
+
+template <int DC, int DR>
+__global__ void __launch_bounds__(kThreads, 1)
+    mla_attn_wide_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
+                            const __grid_constant__ CUtensorMap tm_k,
+                            const __grid_constant__ CUtensorMap tm_kr,
+                            const __grid_constant__ CUtensorMap tm_v, const WideKParams p) {
+  using S = WideShape<DC, DR>;
+  constexpr int NK = S::kKStages, NV = S::kVStages;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = align_smem_1024(smem_raw);
+  uint8_t* sQ = smem;
+  uint8_t* sV = sQ + S::kQBytes;
+  uint8_t* sK = sV + NV * S::kVTile;
+  // Barriers sit at the same offsets in both CTAs. Those the MMA issuers wait
+  // on (q_full, q_ready, k_full, v_full, s_free, p_full) are used in the even
+  // CTA and count both CTAs' bytes or warps; the MMAs' commits reach the
+  // others in both CTAs.
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sK + NK * S::kKBox);
+  uint64_t* q_full = bars;
+  uint64_t* q_ready = bars + 1;
+  uint64_t* s_full = bars + 2;
+  uint64_t* s_free = bars + 3;
+  uint64_t* p_full = bars + 4;
+  uint64_t* pv_done = bars + 5;
+  uint64_t* mma_drain = bars + 6;
+  uint64_t* k_full = bars + 7;
+  uint64_t* k_empty = k_full + NK;
+  uint64_t* v_full = k_empty + NK;
+  uint64_t* v_empty = v_full + NV;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(v_empty + NV);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const int b = blockIdx.y;
+  const int item = blockIdx.x / 2;  // cluster
+  const int vpart = item % S::kSplit;
+  const int nblk = (p.n_valid + kBN - 1) / kBN;
+  const WaitCtx wc{abort_flag, p.status};
+
+  if (threadIdx.x == 0) {
+    mbar_init(q_full, 1);
+    mbar_init(q_ready, 8);  // one arrival per softmax warp of both CTAs, and so below
+    mbar_init(s_full, 1);
+    mbar_init(s_free, 8);
+    mbar_init(p_full, 8);
+    mbar_init(pv_done, 1);
+    mbar_init(mma_drain, 1);
+    for (int s = 0; s < NK; ++s) {
+      mbar_init(&k_full[s], 1);
+      mbar_init(&k_empty[s], 1);
+    }
+    for (int s = 0; s < NV; ++s) {
+      mbar_init(&v_full[s], 1);
+      mbar_init(&v_empty[s], 1);
+    }
+    *abort_flag = 0;
+    fence_mbar_init();
+  }
+  if (warp == 1) {
+    tmem_alloc_pair(tmem_slot, 512);
+    tmem_relinquish_pair();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const int crank = static_cast<int>(cluster_ctarank());
+  const int row0 = (item / S::kSplit * 2 + crank) * kBM;
+  cluster_sync();  // the peer's barriers exist before copies, commits and arrivals reach them
+  grid_dep_sync();
+
+  if (warp == 0) {
+    // ------------------------------------------------------------ producer
+    if (lane == 0) {
+      tma_prefetch_desc(&tm_q);
+      tma_prefetch_desc(&tm_k);
+      tma_prefetch_desc(&tm_kr);
+      tma_prefetch_desc(&tm_v);
+      auto even = [&](uint64_t* bar) { return dsmem_addr(smem_u32(bar), 0); };
+      if (crank == 0) mbar_arrive_expect_tx(q_full, 2 * S::kQBytes);
+      for (int cb = 1; cb < S::kCBoxes; ++cb)
+        tma_load_3d_pair(sQ + (cb - 1) * S::kQBox, &tm_q, even(q_full), cb * 64, row0, b);
+      int kt = 0, vt = 0;  // K boxes and V tiles issued so far
+      bool ok = true;
+      auto load_v = [&](int j) {
+        const int st = vt % NV;
+        if (vt >= NV && !mbar_wait(&v_empty[st], ((vt / NV) - 1) & 1, wc)) return false;
+        if (crank == 0) mbar_arrive_expect_tx(&v_full[st], 2 * S::kVTile);
+        for (int h = 0; h < 2; ++h)
+          tma_load_3d_pair(sV + st * S::kVTile + h * S::kVBox, &tm_v, even(&v_full[st]),
+                           vpart * DV + crank * 128 + h * 64, j * kBN, b);
+        ++vt;
+        return true;
+      };
+      for (int j = 0; ok && j < nblk; ++j) {
+        for (int bx = 0; bx < S::kBoxes; ++bx) {
+          const int st = kt % NK;
+          if (kt >= NK && !mbar_wait(&k_empty[st], ((kt / NK) - 1) & 1, wc)) {
+            ok = false;
+            break;
+          }
+          const bool is_c = bx < S::kCBoxes;
+          if (crank == 0)
+            mbar_arrive_expect_tx(&k_full[st], 2 * (is_c ? S::kKBox : S::kKrBytes));
+          const int key = j * kBN + crank * (kBN / 2);
+          if (is_c)
+            tma_load_3d_pair(sK + st * S::kKBox, &tm_k, even(&k_full[st]), bx * 64, key, b);
+          else
+            tma_load_3d_pair(sK + st * S::kKBox, &tm_kr, even(&k_full[st]), 0, key, b);
+          ++kt;
+        }
+        ok = ok && load_v(j);
+      }
+      // the even CTA's MMAs release this CTA's stages: the last releases must
+      // have landed before the CTA may exit
+      for (int u = kt > NK ? kt - NK : 0; u < kt && !*abort_flag; ++u)
+        mbar_wait(&k_empty[u % NK], (u / NK) & 1, wc);
+      for (int u = vt > NV ? vt - NV : 0; u < vt && !*abort_flag; ++u)
+        mbar_wait(&v_empty[u % NV], (u / NV) & 1, wc);
+      if (*abort_flag && crank == 0) {  // let every copy of the pair land before exit
+        mbar_wait_drain(q_full, 0, p.status);
+        for (int u = kt > NK ? kt - NK : 0; u < kt; ++u)
+          mbar_wait_drain(&k_full[u % NK], (u / NK) & 1, p.status);
+        for (int u = vt > NV ? vt - NV : 0; u < vt; ++u)
+          mbar_wait_drain(&v_full[u % NV], (u / NV) & 1, p.status);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // -------------------------------------------------------- MMA issuer
+    // S_0, S_1, PV_0, S_2, PV_1, ...: PV_{j-1} runs while the softmax warps read
+    // S_j out, and the softmax of block j under PV_{j-1} and S_{j+1}. The whole
+    // warp walks the loop; one lane issues (see elect_one).
+    if (crank == 0) {
+      bool ok = mbar_wait_warp(q_ready, 0, wc) && mbar_wait_warp(q_full, 0, wc);
+      const uint64_t qd = sdesc(smem_u32(sQ), 16, 1024, kSw128);
+      const uint64_t kd = sdesc(smem_u32(sK), 16, 1024, kSw128);
+      const uint64_t krd = sdesc(smem_u32(sK), 16, S::kKrSbo, S::kKrSw);
+      const uint64_t vd = sdesc(smem_u32(sV), S::kVBox, 1024, kSw128);
+      int st = 0, ph = 0;  // K ring stage and phase
+      for (int j = 0; ok && j <= nblk; ++j) {
+        if (j < nblk) {
+          ok = j == 0 || mbar_wait_warp(s_free, (j - 1) & 1, wc);
+#pragma unroll
+          for (int bx = 0; bx < S::kBoxes; ++bx) {
+            ok = ok && mbar_wait_warp(&k_full[st], ph, wc);
+            if (!ok) break;
+            tc_fence_after();
+            if (elect_one()) {
+              const uint64_t ko = static_cast<uint64_t>(st * (S::kKBox >> 4));
+              if (bx < S::kCBoxes) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                  if (bx == 0)
+                    umma_pair_ts(tmem, tmem + S::kTmemQ + k * 8, kd + ko + k * 2, S::kIdescQK,
+                                 k != 0 ? 1u : 0u);
+                  else
+                    umma_pair_ss(tmem, qd + (((bx - 1) * S::kQBox + k * 32) >> 4),
+                                 kd + ko + k * 2, S::kIdescQK, 1u);
+                }
+              } else {
+#pragma unroll
+                for (int k = 0; k < DR / 16; ++k)
+                  umma_pair_ts(tmem, tmem + S::kTmemQ + 32 + k * 8, krd + ko + k * 2,
+                               S::kIdescQK, 1u);
+              }
+              umma_pair_commit_mc(&k_empty[st], 3);
+              if (bx == S::kBoxes - 1) umma_pair_commit_mc(s_full, 3);
+            }
+            __syncwarp();
+            if (++st == NK) {
+              st = 0;
+              ph ^= 1;
+            }
+          }
+        }
+        if (ok && j > 0) {
+          const int i = j - 1, sv = i % NV;
+          ok = mbar_wait_warp(&v_full[sv], (i / NV) & 1, wc) &&
+               mbar_wait_warp(p_full, i & 1, wc);
+          if (!ok) break;
+          tc_fence_after();
+          if (elect_one()) {
+            const uint64_t vo = static_cast<uint64_t>(sv * (S::kVTile >> 4));
+#pragma unroll
+            for (int s = 0; s < kBN / 16; ++s)
+              umma_pair_ts(tmem + S::kTmemO, tmem + S::kTmemP + s * 8, vd + vo + s * (2048 >> 4),
+                           S::kIdescPV, (i > 0 || s > 0) ? 1u : 0u);
+            umma_pair_commit_mc(&v_empty[sv], 3);
+            umma_pair_commit_mc(pv_done, 3);
+          }
+          __syncwarp();
+        }
+      }
+      if (!ok) {  // every MMA this warp issued is done before TMEM is freed
+        if (elect_one()) umma_pair_commit_mc(mma_drain, 1);
+        __syncwarp();
+        mbar_wait_drain(mma_drain, 0, p.status);
+      }
+    }
+  } else {
+    // ------------------------------------------------ softmax (warps 2..5)
+    const int quarter = warp & 3;  // TMEM lane quarter this warp may access
+    const int r = quarter * 32 + lane;
+    const uint32_t t_lane = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
+    const int grow = row0 + r;
+    const bool row_ok = grow < p.rows;
+    const uint32_t q_ready_even = dsmem_addr(smem_u32(q_ready), 0);
+    const uint32_t s_free_even = dsmem_addr(smem_u32(s_free), 0);
+    const uint32_t p_full_even = dsmem_addr(smem_u32(p_full), 0);
+    {
+      // Q's TMEM part: columns [0, 64) of q_c, then q_r rotated by the query
+      // position (RoPE3D); column c of the A operand holds elements 2c, 2c + 1
+      uint32_t qw[32];
+      const uint4* qsrc = reinterpret_cast<const uint4*>(
+          p.q_c + (static_cast<size_t>(b) * p.rows + (row_ok ? grow : 0)) * DC);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const uint4 v = row_ok ? __ldg(qsrc + i) : make_uint4(0u, 0u, 0u, 0u);
+        qw[4 * i + 0] = v.x;
+        qw[4 * i + 1] = v.y;
+        qw[4 * i + 2] = v.z;
+        qw[4 * i + 3] = v.w;
+      }
+      tmem_st32(t_lane + S::kTmemQ, qw);
+      uint32_t w[DR / 2];
+#pragma unroll
+      for (int i = 0; i < DR / 2; ++i) w[i] = 0u;
+      if (row_ok) {
+        const uint4* src = reinterpret_cast<const uint4*>(
+            p.q_r + (static_cast<size_t>(b) * p.rows + grow) * DR);
+#pragma unroll
+        for (int i = 0; i < DR / 8; ++i) {
+          const uint4 v = __ldg(src + i);
+          w[4 * i + 0] = v.x;
+          w[4 * i + 1] = v.y;
+          w[4 * i + 2] = v.z;
+          w[4 * i + 3] = v.w;
+        }
+        const int nq = p.rows / p.heads;
+        const int* pp = p.q_pos + (static_cast<size_t>(b) * nq + grow / p.heads) * 3;
+        int pa[3] = {__ldg(pp), __ldg(pp + 1), __ldg(pp + 2)};
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+          if (pa[a] < 0 || pa[a] >= p.rope_len) {
+            record_status(p.status, MLA_ERR_RANGE);
+            pa[a] = 0;
+          }
+#pragma unroll
+        for (int i = 0; i < DR / 2; ++i) {
+          const int pos = i < p.pairs_t ? pa[0] : (i < p.pairs_t + p.pairs_h ? pa[1] : pa[2]);
+          const float2 cs = __ldg(p.rope + static_cast<size_t>(pos) * (DR / 2) + i);
+          const float x0 = bf16_lo(w[i]), x1 = bf16_hi(w[i]);
+          w[i] = pack_bf16x2(x0 * cs.x - x1 * cs.y, x0 * cs.y + x1 * cs.x);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < DR / 32; ++c) tmem_st16(t_lane + S::kTmemQ + 32 + c * 16, w + c * 16);
+      tmem_wait_st();
+      tc_fence_before();
+      mbar_arrive_peer_warp(q_ready_even);
+    }
+
+    float m_run = -INFINITY;
+    float l_run = 0.f;
+    bool ok = true;
+    bool s_now = false;  // a poll has seen the next block's scores
+    const uint32_t tP = t_lane + S::kTmemP, tO = t_lane + S::kTmemO;
+    for (int j = 0; j < nblk; ++j) {
+      if (!s_now && !mbar_wait(s_full, j & 1, wc)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      uint32_t sr[kBN];
+#pragma unroll
+      for (int c = 0; c < kBN / 32; ++c)
+        tmem_ld32(t_lane + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[c * 32]));
+      tmem_wait_ld();
+      tc_fence_before();
+      mbar_arrive_peer_warp(s_free_even);  // the next block's scores may land
+      float sv[kBN];
+#pragma unroll
+      for (int c = 0; c < kBN; ++c) sv[c] = __uint_as_float(sr[c]);
+      const int valid = p.n_valid - j * kBN;
+      if (valid < kBN) {
+#pragma unroll
+        for (int c = 0; c < kBN; ++c)
+          if (c >= valid) sv[c] = -INFINITY;
+      }
+      // row max: 8 chains of three-input maxima, then a tree
+      float m8[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) m8[i] = fmaxf(sv[i], sv[8 + i]);
+#pragma unroll
+      for (int c = 16; c + 16 <= kBN; c += 16)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) m8[i] = fmax3(m8[i], sv[c + i], sv[c + 8 + i]);
+      const float mx = fmaxf(fmaxf(fmaxf(m8[0], m8[1]), fmaxf(m8[2], m8[3])),
+                             fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7])));
+      const float m_blk = mx * p.scale_log2;
+      // lazy rescale, settled before the exponentials: keep the running max
+      // unless this block's max exceeds it by more than 2^8 (P <= 256 then,
+      // harmless in bf16 / fp32)
+      const bool need = j > 0 && m_blk > m_run + kRescaleLog2;
+      if (__any_sync(0xffffffffu, need)) {
+        debug_count_rescale(need && row_ok, p.status);
+        const float alpha = need ? ex2_approx(m_run - m_blk) : 1.f;
+        if (need) m_run = m_blk;
+        l_run *= alpha;
+        if (!mbar_wait(pv_done, (j - 1) & 1, wc)) {  // PV_{j-1} has finished with O
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+#pragma unroll 1
+        for (int c = 0; c < DV / 16; ++c) {
+          uint32_t ov[16];
+          tmem_ld16(tO + c * 16, ov);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) ov[i] = __float_as_uint(__uint_as_float(ov[i]) * alpha);
+          tmem_st16(tO + c * 16, ov);
+        }
+        tmem_wait_st();
+      }
+      if (j == 0) m_run = m_blk;
+      const uint64_t scale2 = f32x2_pack(p.scale_log2, p.scale_log2);
+      const uint64_t negm2 = f32x2_pack(-m_run, -m_run);
+      uint64_t l4[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) l4[i] = 0ull;
+      uint32_t pk[kBN / 2];
+      auto exps = [&](int i0, int i1) {  // pairs [i0, i1) of scores -> bf16 P
+#pragma unroll
+        for (int i = i0; i < i1; ++i) {
+          float t0, t1;
+          f32x2_unpack(f32x2_fma(f32x2_pack(sv[2 * i], sv[2 * i + 1]), scale2, negm2), t0, t1);
+          const float p0 = ex2_approx(t0);
+          const float p1 = ex2_approx(t1);
+          l4[i & 3] = f32x2_add(l4[i & 3], f32x2_pack(p0, p1));
+          pk[i] = pack_bf16x2(p0, p1);
+        }
+      };
+      // the first half of P goes out under the second half's exponentials,
+      // once PV_{j-1} has read the previous P
+      exps(0, kBN / 4);
+      if (j > 0 && !mbar_wait(pv_done, (j - 1) & 1, wc)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      tmem_st32(tP, *reinterpret_cast<uint32_t(*)[32]>(&pk[0]));
+      exps(kBN / 4, kBN / 2);
+      tmem_st32(tP + 32, *reinterpret_cast<uint32_t(*)[32]>(&pk[32]));
+      s_now = mbar_test(s_full, (j + 1) & 1);
+      tmem_wait_st();
+      tc_fence_before();
+      mbar_arrive_peer_warp(p_full_even);
+      float l8[8];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) f32x2_unpack(l4[i], l8[2 * i], l8[2 * i + 1]);
+      l_run += ((l8[0] + l8[1]) + (l8[2] + l8[3])) + ((l8[4] + l8[5]) + (l8[6] + l8[7]));
+    }
+
+    // O / l as bf16: each thread stages its row densely in the V ring (free
+    // once the last PV is done) and the rows leave by bulk copy, the whole
+    // tile at once when its rows are consecutive rows of o (DV = d_c).
+    const bool have_o = ok && mbar_wait(pv_done, (nblk - 1) & 1, wc);
+    uint8_t* srow = sV + r * DV * 2;
+    if (have_o) {
+      tc_fence_after();
+      const float inv_l = 1.f / l_run;
+#pragma unroll 1
+      for (int sg = 0; sg < DV / 64; ++sg) {
+        uint32_t va[32], vb[32];
+        tmem_ld32(tO + sg * 64, va);
+        tmem_ld32(tO + sg * 64 + 32, vb);
+        tmem_wait_ld();
+        uint32_t pk[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          const uint32_t* v = i < 16 ? va : vb;
+          const int q = i & 15;
+          pk[i] = pack_bf16x2(__uint_as_float(v[2 * q]) * inv_l,
+                              __uint_as_float(v[2 * q + 1]) * inv_l);
+        }
+        stage_row<8>(srow + sg * 128, pk, r & 7);
+      }
+    }
+    fence_proxy_async_smem();
+    if constexpr (DV == DC) {
+      asm volatile("bar.sync 1, 128;" ::: "memory");  // the four softmax warps
+      // the tile's rows below p.rows; none in a CTA past an odd last tile
+      const int valid = min(kBM, p.rows - row0);
+      if (r == 0 && have_o && !*abort_flag && valid > 0) {
+        bulk_store(p.o + (static_cast<size_t>(b) * p.rows + row0) * DC, sV, valid * DC * 2);
+        bulk_commit();
+        bulk_wait_read_all();  // the staged rows must outlive the copy's reads
+      }
+    } else if (have_o && row_ok) {
+      bulk_store(p.o + (static_cast<size_t>(b) * p.rows + grow) * DC + vpart * DV, srow, DV * 2);
+      bulk_commit();
+      bulk_wait_read_all();
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();  // both CTAs are done with the pair's TMEM, barriers and shared memory
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc_pair(tmem, 512);
+  }
+}
+
+template <int DC, int DR>
+int launch_wide(const AttnArgs& a) {
+  using S = WideShape<DC, DR>;
+  CUtensorMap tm_q, tm_k, tm_kr, tm_v;
+  const unsigned long long rows = a.rows, slots = a.slots;
+  if (!encode_map_3d_bf16(&tm_q, a.q_c, DC, rows, a.batch, DC * 2ull, rows * DC * 2ull, 64, kBM,
+                          CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_map_3d_bf16(&tm_k, a.c, DC, a.n_valid, a.batch, DC * 2ull, slots * DC * 2ull, 64,
+                          kBN / 2, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_map_3d_bf16(&tm_kr, a.kr, DR, a.n_valid, a.batch, DR * 2ull, slots * DR * 2ull, DR,
+                          kBN / 2,
+                          DR == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_map_3d_bf16(&tm_v, a.c, DC, a.n_valid, a.batch, DC * 2ull, slots * DC * 2ull, 64,
+                          kBN, CU_TENSOR_MAP_SWIZZLE_128B))
+    return MLA_ERR_CUDA;
+  auto kern = mla_attn_wide_tc_kernel<DC, DR>;
+  cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmemBytes);
+  if (e != cudaSuccess) {
+    set_last_cuda_error(e);
+    return MLA_ERR_CUDA;
+  }
+  WideKParams kp;
+  kp.q_c = static_cast<const __nv_bfloat16*>(a.q_c);
+  kp.q_r = static_cast<const __nv_bfloat16*>(a.q_r);
+  kp.q_pos = a.q_pos;
+  kp.rope = reinterpret_cast<const float2*>(a.rope);
+  kp.o = static_cast<__nv_bfloat16*>(a.o);
+  kp.rows = a.rows;
+  kp.heads = a.heads;
+  kp.n_valid = a.n_valid;
+  kp.rope_len = a.rope_len;
+  kp.pairs_t = a.pairs_t;
+  kp.pairs_h = a.pairs_h;
+  kp.scale_log2 = a.scale_log2;
+  kp.status = a.status;
+  const int pairs = (a.rows + 2 * kBM - 1) / (2 * kBM);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * pairs * S::kSplit, a.batch, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = S::kSmemBytes;
+  cfg.stream = a.stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see grid_dep_sync
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  e = cudaLaunchKernelEx(&cfg, kern, tm_q, tm_k, tm_kr, tm_v, kp);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    set_last_cuda_error(e);
+    return MLA_ERR_CUDA;
+  }
+  return MLA_OK;
+}
+
+}  // namespace
+
+int launch_attention_wide_tc(const AttnArgs& a) {
+  if (a.d_c == 256) return a.d_r == 32 ? launch_wide<256, 32>(a) : launch_wide<256, 64>(a);
+  return a.d_r == 32 ? launch_wide<512, 32>(a) : launch_wide<512, 64>(a);
+}
+
+}  // namespace vmla

@@ -1,0 +1,47 @@
+"""Attention at d_c = 256 and 512 (paired-SM MMAs over two row tiles) where a
+CTA of the pair has no rows or no keys of its own, and at the edges of tiles,
+key blocks and rings."""
+
+import pytest
+import torch
+
+from paper_2605_30351_gb300 import synth
+from paper_2605_30351_gb300 import videomla as V
+
+from test_gpu_parity import assert_rows_close, f64, oracle_latent, small, upload_cache
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    V.load()
+    V.mla_device_status(clear=True)
+    yield
+    assert V.mla_device_status(clear=True) == V.MLA_OK
+
+
+@pytest.mark.parametrize("d_c", [256, 512])
+@pytest.mark.parametrize("grid,frames,nq,batch,d_r", [
+    ((1, 1), 1, 1, 1, 32),      # one key, 12 rows: the odd CTA has neither
+    ((4, 16), 1, 10, 1, 64),    # 64 keys: the odd CTA's half is empty; 120 rows
+    ((8, 16), 3, 11, 2, 32),    # whole blocks; the odd CTA has four rows
+    ((5, 13), 3, 40, 1, 64),    # 195 keys: the last block ends inside the odd half
+    ((10, 13), 13, 22, 3, 32),  # 14 blocks, more K boxes and V tiles than ring stages
+])
+def test_wide_latent_edges(d_c, grid, frames, nq, batch, d_r):
+    w = small(d_c=d_c, d_r=d_r, rope_pairs=(6, 5, 5) if d_r == 32 else (12, 10, 10),
+              rope_axis_dims=(44, 42, 42) if d_r == 32 else (64, 64, 64), grid_h=grid[0],
+              grid_w=grid[1], window_frames=frames, batch=batch)
+    cache, c, k = upload_cache(w, 31, frames)
+    q_c, q_r = synth.draw_queries(w, nq, 32, qc_std=1.0)
+    q_pos = synth.grid_positions(w, 0, frames)[:, -nq:].contiguous()
+    if q_pos.shape[1] < nq:
+        q_pos = q_pos[:, :1].repeat(1, nq, 1).contiguous()
+    o = torch.empty(batch, nq, w.heads, d_c, dtype=torch.bfloat16, device="cuda")
+    V.mla_attention_forward(cache, q_c.cuda(), q_r.cuda(), q_pos.cuda(), o)
+    torch.cuda.synchronize()
+    ref = oracle_latent(w, q_c, q_r, q_pos, c, k, cache.n_valid())
+    assert_rows_close(f64(o), ref, f"wide latent {d_c}")
