@@ -4,7 +4,7 @@
 // k = RoPE3D(W_R^K x), FIFO ring write (App. D.4). One CTA takes 128 tokens:
 //   warp 0     TMA producer: x tile [128 x 64] and the matching 64 columns of
 //              [W_dkv ; W_kr] ([d_c + d_r] x 64) per stage, SW128.
-//   warp 1     allocates TMEM; one lane issues tcgen05.mma into one
+//   warp 1     allocates TMEM; issues tcgen05.mma into one
 //              [128 x (d_c + d_r)] fp32 accumulator (a single N = 224 MMA per
 //              K step at the paper's shape).
 //   warps 2-5  epilogue, thread i = token i: RMSNorm over the d_c columns in
@@ -210,44 +210,43 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
       cluster_wait_acquire();
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      bool ok = true;
-      for (int kb = 0; kb < p.k_blocks; ++kb) {
-        const int st = kb % NST;
-        if (!mbar_wait(&full[st], (kb / NST) & 1, wc)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t aa = smem_u32(smem + st * S::kStageBytes);
-        const uint32_t ba = aa + S::kABytes;
+    // the whole warp walks the loop; one lane issues (see elect_one)
+    bool ok = true;
+    const uint64_t a0 = sdesc(smem_u32(smem), 16, 1024, kSw128);
+    const uint64_t b0 = sdesc(smem_u32(smem) + S::kABytes, 16, 1024, kSw128);
+    for (int kb = 0; kb < p.k_blocks; ++kb) {
+      const int st = kb % NST;
+      ok = mbar_wait_warp(&full[st], (kb / NST) & 1, wc);
+      if (!ok) break;
+      tc_fence_after();
+      if (elect_one()) {
+        const uint64_t so = static_cast<uint64_t>(st * (S::kStageBytes >> 4));
 #pragma unroll
         for (int k = 0; k < kBK / 16; ++k) {
           const uint32_t acc = (kb | k) != 0 ? 1u : 0u;
-          const uint64_t ad = sdesc(aa + k * 32, 16, 1024, kSw128);
+          const uint64_t ad = a0 + so + k * 2, bd = b0 + so + k * 2;
           if constexpr (!S::kSplitN) {
             constexpr uint32_t idesc = idesc_bf16_f32(kBM, S::N, false, false);
-            umma_ss(tmem, ad, sdesc(ba + k * 32, 16, 1024, kSw128), idesc, acc);
+            umma_ss(tmem, ad, bd, idesc, acc);
           } else {
             constexpr int kHc = NC < 256 ? NC : 256;  // columns per c MMA
             constexpr uint32_t idesc_c = idesc_bf16_f32(kBM, kHc, false, false);
 #pragma unroll
             for (int h = 0; h < NC / kHc; ++h)
-              umma_ss(tmem + h * kHc, ad, sdesc(ba + h * kHc * 128 + k * 32, 16, 1024, kSw128),
-                      idesc_c, acc);
+              umma_ss(tmem + h * kHc, ad, bd + ((h * kHc * 128) >> 4), idesc_c, acc);
             if constexpr (NK > 0) {
               constexpr uint32_t idesc_k = idesc_bf16_f32(kBM, NK, false, false);
-              umma_ss(tmem + NC, ad, sdesc(ba + NC * 128 + k * 32, 16, 1024, kSw128), idesc_k,
-                      acc);
+              umma_ss(tmem + NC, ad, bd + ((NC * 128) >> 4), idesc_k, acc);
             }
           }
         }
         umma_commit(&empty[st]);
       }
-      umma_commit(acc_full);
-      if (!ok) mbar_wait_drain(acc_full, 0, p.status);
+      __syncwarp();
     }
+    if (elect_one()) umma_commit(acc_full);
     __syncwarp();
+    if (!ok) mbar_wait_drain(acc_full, 0, p.status);
     if constexpr (CL > 1) {  // the cluster's second barrier phase
       cluster_arrive_release();
       cluster_wait_acquire();

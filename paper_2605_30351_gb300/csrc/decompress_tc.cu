@@ -16,7 +16,7 @@
 // window the 201 MB of keys and values written dominate, so the kernel is
 // bound by HBM writes.
 //   warp 0     TMA producer (weights once, then c tiles)
-//   warp 1     TMEM allocation; one lane issues tcgen05.mma (M = 128, N = BN)
+//   warp 1     TMEM allocation; issues tcgen05.mma (M = 128, N = BN)
 //   warps 2-13 epilogue: warps w, w + 4, w + 8 read TMEM lane quarter w % 4
 //              (slot rows), each a third of the columns, into shared staging
 //              as bf16: one [128 slots x 32 columns] box per 32 columns, in
@@ -175,32 +175,33 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      bool ok = mbar_wait(w_full, 0, wc);
-      for (int i = 0, r = g; ok && r < p.n_row_tiles; ++i, r += G) {
-        const int s = i & 1;
-        if (!mbar_wait(&c_full[s], (i >> 1) & 1, wc) ||
-            (i >= 2 && !mbar_wait(&acc_empty[s], ((i >> 1) - 1) & 1, wc))) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t ca = smem_u32(sC + s * S::kCBytes);
-        const uint32_t wa = smem_u32(sW);
+    // the whole warp walks the loop; one lane issues (see elect_one)
+    bool ok = mbar_wait_warp(w_full, 0, wc);
+    const uint64_t cd = sdesc(smem_u32(sC), 16, 1024, kSw128);
+    const uint64_t wd = sdesc(smem_u32(sW), 16, 1024, kSw128);
+    for (int i = 0, r = g; ok && r < p.n_row_tiles; ++i, r += G) {
+      const int s = i & 1;
+      ok = mbar_wait_warp(&c_full[s], (i >> 1) & 1, wc) &&
+           (i < 2 || mbar_wait_warp(&acc_empty[s], ((i >> 1) - 1) & 1, wc));
+      if (!ok) break;
+      tc_fence_after();
+      if (elect_one()) {
+        const uint64_t co = static_cast<uint64_t>(s * (S::kCBytes >> 4));
 #pragma unroll
         for (int kc = 0; kc < KC; ++kc)
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            umma_ss(tmem + s * BN, sdesc(ca + kc * S::kChunkBytesC + k * 32, 16, 1024, kSw128),
-                    sdesc(wa + kc * S::kChunkBytesW + k * 32, 16, 1024, kSw128), S::kIdesc,
+            umma_ss(tmem + s * BN, cd + co + ((kc * S::kChunkBytesC + k * 32) >> 4),
+                    wd + ((kc * S::kChunkBytesW + k * 32) >> 4), S::kIdesc,
                     (kc | k) != 0 ? 1u : 0u);
         umma_commit(&c_empty[s]);
         umma_commit(&acc_full[s]);
       }
-      umma_commit(mma_done);
-      mbar_wait_drain(mma_done, 0, p.status);  // every MMA of this CTA has completed
+      __syncwarp();
     }
+    if (elect_one()) umma_commit(mma_done);
     __syncwarp();
+    mbar_wait_drain(mma_done, 0, p.status);  // every MMA of this CTA has completed
   } else {
     const int quarter = warp & 3;
     const int part = (warp - 2) >> 2;       // which share of the columns this warp reads

@@ -5,7 +5,7 @@
 // both operands K-major, fp32 accumulation, one 128 x BN tile per CTA:
 //   warp 0     TMA producer (A [128 x 64], B [BN x 64] per stage, SW128;
 //              B in two boxes when BN > 256)
-//   warp 1     TMEM allocation; one lane issues tcgen05.mma (N = BN, or two
+//   warp 1     TMEM allocation; issues tcgen05.mma (N = BN, or two
 //              MMAs of N = BN/2 when BN > 256)
 //   warps 2-5  epilogue, thread i = row i: TMEM -> registers -> bf16 staged
 //              in shared memory, then one bulk copy per row (two when the row
@@ -161,41 +161,46 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0 && crank == 0) {
+    // the whole warp walks the loop; one lane issues (see elect_one)
+    if (crank == 0) {
       bool ok = true;
+      const uint64_t ad = sdesc(smem_u32(smem), 16, 1024, kSw128);
+      const uint64_t bd = sdesc(smem_u32(smem) + S::kABytes, 16, 1024, kSw128);
       for (int kb = 0; kb < k_blocks; ++kb) {
         const int st = kb % NST;
-        if (!mbar_wait(&full[st], (kb / NST) & 1, wc)) {
-          ok = false;
-          break;
-        }
+        ok = mbar_wait_warp(&full[st], (kb / NST) & 1, wc);
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t aa = smem_u32(smem + st * S::kStageBytes);
-        const uint32_t ba = aa + S::kABytes;
-        if constexpr (PAIR) {
+        if (elect_one()) {
+          const uint64_t so = static_cast<uint64_t>(st * (S::kStageBytes >> 4));
+          if constexpr (PAIR) {
 #pragma unroll
-          for (int k = 0; k < kBK / 16; ++k)
-            umma_pair_ss(tmem, sdesc(aa + k * 32, 16, 1024, kSw128),
-                         sdesc(ba + k * 32, 16, 1024, kSw128), S::kIdesc, (kb | k) != 0 ? 1u : 0u);
-          umma_pair_commit_mc(&empty[st], 3);
-        } else {
+            for (int k = 0; k < kBK / 16; ++k)
+              umma_pair_ss(tmem, ad + so + k * 2, bd + so + k * 2, S::kIdesc,
+                           (kb | k) != 0 ? 1u : 0u);
+            umma_pair_commit_mc(&empty[st], 3);
+          } else {
 #pragma unroll
-          for (int k = 0; k < kBK / 16; ++k)
+            for (int k = 0; k < kBK / 16; ++k)
 #pragma unroll
-            for (int h = 0; h < S::kHalves; ++h)
-              umma_ss(tmem + h * S::kBN1, sdesc(aa + k * 32, 16, 1024, kSw128),
-                      sdesc(ba + h * S::kBN1 * 128 + k * 32, 16, 1024, kSw128), S::kIdesc,
-                      (kb | k) != 0 ? 1u : 0u);
-          umma_commit(&empty[st]);
+              for (int h = 0; h < S::kHalves; ++h)
+                umma_ss(tmem + h * S::kBN1, ad + so + k * 2,
+                        bd + so + ((h * S::kBN1 * 128) >> 4) + k * 2, S::kIdesc,
+                        (kb | k) != 0 ? 1u : 0u);
+            umma_commit(&empty[st]);
+          }
         }
+        __syncwarp();
       }
-      if constexpr (PAIR)
-        umma_pair_commit_mc(acc_full, 3);
-      else
-        umma_commit(acc_full);
+      if (elect_one()) {
+        if constexpr (PAIR)
+          umma_pair_commit_mc(acc_full, 3);
+        else
+          umma_commit(acc_full);
+      }
+      __syncwarp();
       if (!ok) mbar_wait_drain(acc_full, 0, p.status);
     }
-    __syncwarp();
   } else {
     const int quarter = warp & 3;
     const int r = quarter * 32 + lane;
@@ -340,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], 2 * 128);  // every epilogue thread of both CTAs
+      mbar_init(&acc_empty[b], 2 * 4);  // every epilogue warp of both CTAs
     }
     mbar_init(mma_drain, 1);
     *abort_flag = 0;
@@ -391,41 +396,45 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0 && crank == 0) {
-      int it = 0, tl = 0;
+    // the whole warp walks the loop; one lane issues (see elect_one)
+    if (crank == 0) {
+      int st = 0, ph = 0, tl = 0;  // ring stage and phase, tile
       bool ok = true;
+      const uint64_t ad = sdesc(smem_u32(smem), 16, 1024, kSw128);
+      const uint64_t bd = sdesc(smem_u32(smem) + S::kABytes, 16, 1024, kSw128);
       for (int t = cluster; t < total && ok; t += clusters, ++tl) {
         const int buf = tl & 1;
         // both CTAs' epilogues have drained this accumulator (two tiles ago)
-        if (tl >= 2 && !mbar_wait_cluster(&acc_empty[buf], ((tl >> 1) - 1) & 1, wc)) {
-          ok = false;
-          break;
-        }
+        ok = tl < 2 || mbar_wait_warp(&acc_empty[buf], ((tl >> 1) - 1) & 1, wc);
+        if (!ok) break;
         tc_fence_after();
         const uint32_t acc = tmem + buf * S::kAccStride;
-        for (int kb = 0; kb < k_blocks; ++kb, ++it) {
-          const int st = it % NST;
-          if (!mbar_wait(&full[st], (it / NST) & 1, wc)) {
-            ok = false;
-            break;
-          }
+        for (int kb = 0; kb < k_blocks; ++kb) {
+          ok = mbar_wait_warp(&full[st], ph, wc);
+          if (!ok) break;
           tc_fence_after();
-          const uint32_t aa = smem_u32(smem + st * S::kStageBytes);
-          const uint32_t ba = aa + S::kABytes;
+          if (elect_one()) {
+            const uint64_t so = static_cast<uint64_t>(st * (S::kStageBytes >> 4));
 #pragma unroll
-          for (int k = 0; k < kBK / 16; ++k)
-            umma_pair_ss(acc, sdesc(aa + k * 32, 16, 1024, kSw128),
-                         sdesc(ba + k * 32, 16, 1024, kSw128), S::kIdesc, (kb | k) != 0 ? 1u : 0u);
-          umma_pair_commit_mc(&empty[st], 3);
+            for (int k = 0; k < kBK / 16; ++k)
+              umma_pair_ss(acc, ad + so + k * 2, bd + so + k * 2, S::kIdesc,
+                           (kb | k) != 0 ? 1u : 0u);
+            umma_pair_commit_mc(&empty[st], 3);
+            if (kb == k_blocks - 1) umma_pair_commit_mc(&acc_full[buf], 3);
+          }
+          __syncwarp();
+          if (++st == NST) {
+            st = 0;
+            ph ^= 1;
+          }
         }
-        if (ok) umma_pair_commit_mc(&acc_full[buf], 3);
       }
       if (!ok) {  // every MMA issued must be done before the CTA moves on
-        umma_pair_commit_mc(mma_drain, 1);
+        if (elect_one()) umma_pair_commit_mc(mma_drain, 1);
+        __syncwarp();
         mbar_wait_drain(mma_drain, 0, p.status);
       }
     }
-    __syncwarp();
   } else {
     const int quarter = warp & 3;
     const int r = quarter * 32 + lane;
@@ -474,10 +483,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           pk[sg][i] = pack_bf16x2(a0 * scale, a1 * scale);
         }
       }
-      // this thread's reads of the accumulator are done: release it to the
-      // MMA issuer (in the even CTA)
+      // this warp's reads of the accumulator are done: release it to the MMA
+      // issuer (in the even CTA)
       tc_fence_before();
-      mbar_arrive_cluster(dsmem_addr(smem_u32(&acc_empty[buf]), 0));
+      mbar_arrive_peer_warp(dsmem_addr(smem_u32(&acc_empty[buf]), 0));
       bulk_wait_read_all();  // the previous tile's copy of this row has read it
 #pragma unroll
       for (int sg = 0; sg < BN / 64; ++sg) stage_row<8>(srow + sg * 128, pk[sg], r & 7);
