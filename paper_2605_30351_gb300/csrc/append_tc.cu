@@ -3,7 +3,12 @@
 // Paper: Eq. (ckv) c = W_dn^KV x, RMSNorm on c (App. D.2), Eq. (krope)
 // k = RoPE3D(W_R^K x), FIFO ring write (App. D.4). One CTA takes 128 tokens:
 //   warp 0     TMA producer: x tile [128 x 64] and the matching 64 columns of
-//              [W_dkv ; W_kr] ([d_c + d_r] x 64) per stage, SW128.
+//              [W_dkv ; W_kr] ([d_c + d_r] x 64) per K block, SW128. In the
+//              cluster form a stage holds two K blocks and warp 6 fetches the
+//              weights: one producer took ~370 cycles to issue a K block's
+//              copies and ~170 to pass the ring's barrier, which set the pace
+//              (553 cycles a K block, the same with either operand left out);
+//              now shared memory does (432: 24 KB written and read again).
 //   warp 1     allocates TMEM; issues tcgen05.mma into one
 //              [128 x (d_c + d_r)] fp32 accumulator (a single N = 224 MMA per
 //              K step at the paper's shape).
@@ -34,6 +39,7 @@ namespace {
 constexpr int kBM = 128;
 constexpr int kBK = 64;
 constexpr int kThreads = 192;
+constexpr int kClusterThreads = 224;  // the cluster form has a second producer warp
 // dynamic shared memory of a CTA that has an SM to itself, and of one of two
 // CTAs sharing an SM (228 KB per SM, 1 KB of it reserved per CTA)
 constexpr int kSmemOne = 232448;
@@ -70,8 +76,11 @@ struct AppendShape {
   // sums at the same offset in every CTA)
   static constexpr int kBRows = CL > 1 ? 64 + DR : N;
   static constexpr int kBBytes = kBRows * kBK * 2;
-  static constexpr int kTxBytes = kABytes + N * kBK * 2;  // lands in this CTA per stage
-  static constexpr int kStageBytes = kABytes + kBBytes;
+  static constexpr int kWTxBytes = N * kBK * 2;  // weight bytes of a K block in this CTA
+  static constexpr int kBlockBytes = kABytes + kBBytes;  // one K block: x, then weights
+  static constexpr int kKS = CL > 1 ? 2 : 1;             // K blocks per stage
+  static constexpr int kStageBytes = kKS * kBlockBytes;
+  static constexpr int kProducers = CL > 1 ? 2 : 1;
   static constexpr int kBarBytes = 256;
   // [CL][128] partial sums of squares at the front of shared memory: the same
   // offset in every CTA of a cluster, whichever slice it computes
@@ -136,9 +145,14 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
   const int row0 = tile * kBM;
   const WaitCtx wc{abort_flag, p.status};
 
+  if (warp == 0 && lane == 0) {  // kernel parameters: no need to wait for anyone
+    tma_prefetch_desc(tm_x);
+    if constexpr (NC > 0) tma_prefetch_desc(tm_wc);
+    if constexpr (NK > 0) tma_prefetch_desc(tm_wk);
+  }
   if (threadIdx.x == 0) {
     for (int s = 0; s < NST; ++s) {
-      mbar_init(&full[s], 1);
+      mbar_init(&full[s], S::kProducers);
       mbar_init(&empty[s], 1);
     }
     mbar_init(acc_full, 1);
@@ -180,30 +194,51 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
   if constexpr (CL > 1) cluster_sync();
   grid_dep_sync();
 
-  if (warp == 0) {
-    if (lane == 0) {
-      tma_prefetch_desc(tm_x);
-      if constexpr (NC > 0) tma_prefetch_desc(tm_wc);
-      if constexpr (NK > 0) tma_prefetch_desc(tm_wk);
-      int issued = 0;
-      for (int kb = 0; kb < p.k_blocks; ++kb) {
-        const int st = kb % NST;
-        if (kb >= NST && !mbar_wait(&empty[st], ((kb / NST) - 1) & 1, wc)) break;
-        uint8_t* a = smem + st * S::kStageBytes;
-        uint8_t* bm = a + S::kABytes;
-        mbar_arrive_expect_tx(&full[st], S::kTxBytes);
-        tma_load_3d(a, tm_x, &full[st], kb * kBK, row0, b);
-        if constexpr (NC > 0)
-          for (int h = 0; h < NC / S::kWcBox; ++h)
-            tma_load_2d(bm + h * S::kWcBox * 128, tm_wc, &full[st], kb * kBK,
-                        c0 + h * S::kWcBox);
-        if constexpr (NK > 0) tma_load_2d(bm + NC * 128, tm_wk, &full[st], kb * kBK, 0);
-        issued = kb + 1;
+  const int n_stage = (p.k_blocks + S::kKS - 1) / S::kKS;
+  if (warp == 0 || warp == 6) {
+    int issued = 0;
+    auto fill = [&](int i, int st) {  // issue stage i's copies into ring stage st
+      const int kn =  // the last stage may be short
+          S::kKS == 1 ? 1 : min(S::kKS, p.k_blocks - i * S::kKS);
+      uint8_t* blk = smem + st * S::kStageBytes;
+      const bool do_x = warp == 0, do_w = warp == 6 || S::kProducers == 1;
+      mbar_arrive_expect_tx(&full[st],
+                            kn * ((do_x ? S::kABytes : 0) + (do_w ? S::kWTxBytes : 0)));
+#pragma unroll
+      for (int k = 0; k < S::kKS; ++k) {
+        if (k >= kn) break;
+        const int kc = (i * S::kKS + k) * kBK;
+        if (do_x) tma_load_3d(blk + k * S::kBlockBytes, tm_x, &full[st], kc, row0, b);
+        if (do_w) {
+          uint8_t* bm = blk + k * S::kBlockBytes + S::kABytes;
+          if constexpr (NC > 0)
+#pragma unroll
+            for (int h = 0; h < NC / S::kWcBox; ++h)
+              tma_load_2d(bm + h * S::kWcBox * 128, tm_wc, &full[st], kc, c0 + h * S::kWcBox);
+          if constexpr (NK > 0) tma_load_2d(bm + NC * 128, tm_wk, &full[st], kc, 0);
+        }
       }
-      if (*abort_flag)
-        for (int u = issued > NST ? issued - NST : 0; u < issued; ++u)
-          mbar_wait_drain(&full[u % NST], (u / NST) & 1, p.status);
+    };
+    if constexpr (CL > 1) {
+      // the whole warp walks the loop; one lane issues (see elect_one)
+      for (int i = 0; i < n_stage; ++i) {
+        const int st = i % NST;
+        if (i >= NST && !mbar_wait_warp(&empty[st], ((i / NST) - 1) & 1, wc)) break;
+        if (elect_one()) fill(i, st);
+        __syncwarp();
+        issued = i + 1;
+      }
+    } else if (lane == 0) {
+      for (int i = 0; i < n_stage; ++i) {
+        const int st = i % NST;
+        if (i >= NST && !mbar_wait(&empty[st], ((i / NST) - 1) & 1, wc)) break;
+        fill(i, st);
+        issued = i + 1;
+      }
     }
+    if (*abort_flag && lane == 0)
+      for (int u = issued > NST ? issued - NST : 0; u < issued; ++u)
+        mbar_wait_drain(&full[u % NST], (u / NST) & 1, p.status);
     __syncwarp();
     if constexpr (CL > 1) {  // the cluster's second barrier phase (see the epilogue)
       cluster_arrive_release();
@@ -212,37 +247,49 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
   } else if (warp == 1) {
     // the whole warp walks the loop; one lane issues (see elect_one)
     bool ok = true;
+    bool now = false;  // a poll has seen the next stage
+    int st = 0, ph = 0;
     const uint64_t a0 = sdesc(smem_u32(smem), 16, 1024, kSw128);
     const uint64_t b0 = sdesc(smem_u32(smem) + S::kABytes, 16, 1024, kSw128);
-    for (int kb = 0; kb < p.k_blocks; ++kb) {
-      const int st = kb % NST;
-      ok = mbar_wait_warp(&full[st], (kb / NST) & 1, wc);
+    for (int i = 0; i < n_stage; ++i) {
+      ok = now || mbar_wait_warp(&full[st], ph, wc);
       if (!ok) break;
+      const int nst = st + 1 == NST ? 0 : st + 1, nph = st + 1 == NST ? ph ^ 1 : ph;
+      // (where the copies set the pace the poll only delays the MMAs)
+      if constexpr (CL > 1) now = __all_sync(0xffffffffu, mbar_test(&full[nst], nph));
       tc_fence_after();
+      const int kn = S::kKS == 1 ? 1 : min(S::kKS, p.k_blocks - i * S::kKS);
       if (elect_one()) {
-        const uint64_t so = static_cast<uint64_t>(st * (S::kStageBytes >> 4));
 #pragma unroll
-        for (int k = 0; k < kBK / 16; ++k) {
-          const uint32_t acc = (kb | k) != 0 ? 1u : 0u;
-          const uint64_t ad = a0 + so + k * 2, bd = b0 + so + k * 2;
-          if constexpr (!S::kSplitN) {
-            constexpr uint32_t idesc = idesc_bf16_f32(kBM, S::N, false, false);
-            umma_ss(tmem, ad, bd, idesc, acc);
-          } else {
-            constexpr int kHc = NC < 256 ? NC : 256;  // columns per c MMA
-            constexpr uint32_t idesc_c = idesc_bf16_f32(kBM, kHc, false, false);
+        for (int q = 0; q < S::kKS; ++q) {
+          if (q >= kn) break;
+          const uint64_t so =
+              static_cast<uint64_t>((st * S::kStageBytes + q * S::kBlockBytes) >> 4);
 #pragma unroll
-            for (int h = 0; h < NC / kHc; ++h)
-              umma_ss(tmem + h * kHc, ad, bd + ((h * kHc * 128) >> 4), idesc_c, acc);
-            if constexpr (NK > 0) {
-              constexpr uint32_t idesc_k = idesc_bf16_f32(kBM, NK, false, false);
-              umma_ss(tmem + NC, ad, bd + ((NC * 128) >> 4), idesc_k, acc);
+          for (int k = 0; k < kBK / 16; ++k) {
+            const uint32_t acc = (i | q | k) != 0 ? 1u : 0u;
+            const uint64_t ad = a0 + so + k * 2, bd = b0 + so + k * 2;
+            if constexpr (!S::kSplitN) {
+              constexpr uint32_t idesc = idesc_bf16_f32(kBM, S::N, false, false);
+              umma_ss(tmem, ad, bd, idesc, acc);
+            } else {
+              constexpr int kHc = NC < 256 ? NC : 256;  // columns per c MMA
+              constexpr uint32_t idesc_c = idesc_bf16_f32(kBM, kHc, false, false);
+#pragma unroll
+              for (int h = 0; h < NC / kHc; ++h)
+                umma_ss(tmem + h * kHc, ad, bd + ((h * kHc * 128) >> 4), idesc_c, acc);
+              if constexpr (NK > 0) {
+                constexpr uint32_t idesc_k = idesc_bf16_f32(kBM, NK, false, false);
+                umma_ss(tmem + NC, ad, bd + ((NC * 128) >> 4), idesc_k, acc);
+              }
             }
           }
         }
         umma_commit(&empty[st]);
       }
       __syncwarp();
+      st = nst;
+      ph = nph;
     }
     if (elect_one()) umma_commit(acc_full);
     __syncwarp();
@@ -300,37 +347,27 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
     }
     asm volatile("bar.sync 1, 128;" ::: "memory");  // gamma_s is complete
     const bool have_acc = mbar_wait(acc_full, 0, wc) && !*abort_flag;
-    // Each thread stages its finished bf16 row in shared memory (the stage
-    // ring is free once the accumulator is complete): c rows dense at
-    // stage_c ([128][NC] bf16), k^R rows dense at stage_k ([128][NK]), so that
-    // a run of consecutive slots is one contiguous block in shared memory, as
-    // it is in the cache. One CTA per tile then hands each run to the
-    // bulk-copy engine (one copy for c, one for k^R, one or two runs per
-    // tile); a cluster's 64-column slices are written by a coalesced store
-    // loop, their rows not being contiguous in the cache.
-    uint8_t* stage_c = smem;
-    uint8_t* stage_k = smem + kBM * NC * 2;
-    long long* slot_of = reinterpret_cast<long long*>(smem + kBM * S::N * 2);  // [128]
-    // rows that do not continue a run (run starts and rows past the tokens),
-    // one bit per row, one word per warp
-    uint32_t* run_breaks = reinterpret_cast<uint32_t*>(slot_of + kBM);  // [4]
-    // pass 1: sum of squares of this CTA's c columns (fp32)
-    float ss = 0.f;
-    if (have_acc) {
-      tc_fence_after();
-#pragma unroll 1
-      for (int cb = 0; cb < NC / 32; ++cb) {
-        uint32_t v[32];
-        tmem_ld32(t_row + cb * 32, v);
+    if constexpr (CL > 1) {
+      // This CTA's 64 columns of c stay in registers between the statistics and
+      // the store, and each thread writes its row's pieces (128 bytes of c,
+      // d_r values of k^R) straight from registers: a slice's rows are not
+      // contiguous in the cache, and staging them for a coalesced loop took
+      // longer than the whole of this (64 tokens: 8.8 -> 7.3 us, one Wan chunk:
+      // 9.65 -> 8.7 us).
+      static_assert(CL == 1 || NC == 64, "one 64-column slice per CTA");
+      uint32_t v[64];
+      float ss = 0.f;
+      if (have_acc) {
+        tc_fence_after();
+        tmem_ld32(t_row, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+        tmem_ld32(t_row + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
         tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
+        for (int i = 0; i < 64; ++i) {
           const float f = __uint_as_float(v[i]);
           ss = fmaf(f, f, ss);
         }
       }
-    }
-    if constexpr (CL > 1) {
       // every CTA pushes its row's partial sum into slot [its rank][row] of
       // every CTA, then all threads of the cluster pass the second barrier
       // phase (release / acquire), on every path, so that no CTA waits for
@@ -338,60 +375,128 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
       const uint32_t local = smem_u32(ss_all + (c0 / 64) * kBM + r);
       for (int q = 0; q < CL; ++q) dsmem_st_f32(dsmem_addr(local, q), ss);
       cluster_arrive_release();
-      cluster_wait_acquire();
-      ss = 0.f;
-      for (int q = 0; q < CL; ++q) ss += ss_all[q * kBM + r];
-    }
-    const uint32_t breaks = __ballot_sync(0xffffffffu, my_slot < 0 || run_start);
-    if (have_acc) {
-      slot_of[r] = my_slot;
-      if (lane == 0) run_breaks[quarter] = breaks;
-      // positional key first, so that its RoPE factors leave the registers
-      // before pass 2: RoPE3D at the token's (t, h, w), or unrotated
-      if constexpr (NK > 0) {
-        uint32_t pk[NK / 2];
+      const bool store = have_acc && my_slot >= 0 && !*abort_flag;
+      const size_t row_id = static_cast<size_t>(b) * p.slots + (my_slot >= 0 ? my_slot : 0);
+      if constexpr (NK > 0) {  // k^R under the barrier: RoPE3D at the token's (t, h, w), or not
+        uint4* dst = reinterpret_cast<uint4*>(p.kr + row_id * DR);
 #pragma unroll
         for (int cb = 0; cb < NK / 32; ++cb) {
-          uint32_t v[32];
-          tmem_ld32(t_row + NC + cb * 32, v);
-          tmem_wait_ld();
+          uint32_t kv[32], pk[16];
+          if (have_acc) {
+            tmem_ld32(t_row + NC + cb * 32, kv);
+            tmem_wait_ld();
+          }
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const float2 f2 = cs[cb * 16 + i];
-            const float x0 = __uint_as_float(v[2 * i]), x1 = __uint_as_float(v[2 * i + 1]);
-            pk[cb * 16 + i] = p.rotate ? pack_bf16x2(x0 * f2.x - x1 * f2.y, x0 * f2.y + x1 * f2.x)
-                                       : pack_bf16x2(x0, x1);
+            const float x0 = __uint_as_float(kv[2 * i]), x1 = __uint_as_float(kv[2 * i + 1]);
+            pk[i] = p.rotate ? pack_bf16x2(x0 * f2.x - x1 * f2.y, x0 * f2.y + x1 * f2.x)
+                             : pack_bf16x2(x0, x1);
+          }
+          if (store)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              dst[cb * 4 + i] =
+                  make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
+        }
+      }
+      cluster_wait_acquire();
+      ss = 0.f;
+      for (int q = 0; q < CL; ++q) ss += ss_all[q * kBM + r];
+      if (store) {
+        const float inv = p.use_rmsnorm ? rsqrtf(ss / DC + p.eps) : 1.f;
+        const uint4* g4 = gamma_s;
+        uint4* dst = reinterpret_cast<uint4*>(p.c + row_id * DC + c0);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const uint4 g = g4[i];
+          const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
+          uint32_t w[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            w[q] = pack_bf16x2(__uint_as_float(v[8 * i + 2 * q]) * inv * bf16_lo(gw[q]),
+                               __uint_as_float(v[8 * i + 2 * q + 1]) * inv * bf16_hi(gw[q]));
+          dst[i] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+      }
+    } else {
+      // Each thread stages its finished bf16 row in shared memory (the stage
+      // ring is free once the accumulator is complete): c rows dense at
+      // stage_c ([128][NC] bf16), k^R rows dense at stage_k ([128][NK]), so that
+      // a run of consecutive slots is one contiguous block in shared memory, as
+      // it is in the cache, and each run leaves by the bulk-copy engine (one copy
+      // for c, one for k^R, one or two runs per tile).
+      uint8_t* stage_c = smem;
+      uint8_t* stage_k = smem + kBM * NC * 2;
+      long long* slot_of = reinterpret_cast<long long*>(smem + kBM * S::N * 2);  // [128]
+      // rows that do not continue a run (run starts and rows past the tokens),
+      // one bit per row, one word per warp
+      uint32_t* run_breaks = reinterpret_cast<uint32_t*>(slot_of + kBM);  // [4]
+      // pass 1: sum of squares of this CTA's c columns (fp32)
+      float ss = 0.f;
+      if (have_acc) {
+        tc_fence_after();
+#pragma unroll 1
+        for (int cb = 0; cb < NC / 32; ++cb) {
+          uint32_t v[32];
+          tmem_ld32(t_row + cb * 32, v);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            const float f = __uint_as_float(v[i]);
+            ss = fmaf(f, f, ss);
           }
         }
-        stage_row<NK / 8>(stage_k + r * NK * 2, pk, NK == 32 ? (r >> 1) & 3 : r & 7);
       }
-      // pass 2: gamma * c / rms -> bf16, one 64-column (128-byte) segment at a time
-      const float inv = p.use_rmsnorm ? rsqrtf(ss / DC + p.eps) : 1.f;
-      const uint32_t* gamma2 = reinterpret_cast<const uint32_t*>(gamma_s);  // bf16 pairs
-#pragma unroll 1
-      for (int sg = 0; sg < NC / 64; ++sg) {
-        uint32_t va[32], vb[32];
-        tmem_ld32(t_row + sg * 64, va);
-        tmem_ld32(t_row + sg * 64 + 32, vb);
-        tmem_wait_ld();
-        uint32_t pk[32];
+      const uint32_t breaks = __ballot_sync(0xffffffffu, my_slot < 0 || run_start);
+      if (have_acc) {
+        slot_of[r] = my_slot;
+        if (lane == 0) run_breaks[quarter] = breaks;
+        // positional key first, so that its RoPE factors leave the registers
+        // before pass 2: RoPE3D at the token's (t, h, w), or unrotated
+        if constexpr (NK > 0) {
+          uint32_t pk[NK / 2];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const uint32_t ga = gamma2[sg * 32 + i], gb = gamma2[sg * 32 + 16 + i];
-          pk[i] = pack_bf16x2(__uint_as_float(va[2 * i]) * inv * bf16_lo(ga),
-                              __uint_as_float(va[2 * i + 1]) * inv * bf16_hi(ga));
-          pk[16 + i] = pack_bf16x2(__uint_as_float(vb[2 * i]) * inv * bf16_lo(gb),
-                                   __uint_as_float(vb[2 * i + 1]) * inv * bf16_hi(gb));
+          for (int cb = 0; cb < NK / 32; ++cb) {
+            uint32_t v[32];
+            tmem_ld32(t_row + NC + cb * 32, v);
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const float2 f2 = cs[cb * 16 + i];
+              const float x0 = __uint_as_float(v[2 * i]), x1 = __uint_as_float(v[2 * i + 1]);
+              pk[cb * 16 + i] = p.rotate ? pack_bf16x2(x0 * f2.x - x1 * f2.y, x0 * f2.y + x1 * f2.x)
+                                         : pack_bf16x2(x0, x1);
+            }
+          }
+          stage_row<NK / 8>(stage_k + r * NK * 2, pk, NK == 32 ? (r >> 1) & 3 : r & 7);
         }
-        stage_row<8>(stage_c + r * NC * 2 + sg * 128, pk, r & 7);
+        // pass 2: gamma * c / rms -> bf16, one 64-column (128-byte) segment at a time
+        const float inv = p.use_rmsnorm ? rsqrtf(ss / DC + p.eps) : 1.f;
+        const uint32_t* gamma2 = reinterpret_cast<const uint32_t*>(gamma_s);  // bf16 pairs
+#pragma unroll 1
+        for (int sg = 0; sg < NC / 64; ++sg) {
+          uint32_t va[32], vb[32];
+          tmem_ld32(t_row + sg * 64, va);
+          tmem_ld32(t_row + sg * 64 + 32, vb);
+          tmem_wait_ld();
+          uint32_t pk[32];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const uint32_t ga = gamma2[sg * 32 + i], gb = gamma2[sg * 32 + 16 + i];
+            pk[i] = pack_bf16x2(__uint_as_float(va[2 * i]) * inv * bf16_lo(ga),
+                                __uint_as_float(va[2 * i + 1]) * inv * bf16_hi(ga));
+            pk[16 + i] = pack_bf16x2(__uint_as_float(vb[2 * i]) * inv * bf16_lo(gb),
+                                     __uint_as_float(vb[2 * i + 1]) * inv * bf16_hi(gb));
+          }
+          stage_row<8>(stage_c + r * NC * 2 + sg * 128, pk, r & 7);
+        }
       }
-    }
-    // the staged rows reach the async proxy (the bulk copies), then the four
-    // epilogue warps meet; a wait that gave up anywhere shows in abort_flag
-    fence_proxy_async_smem();
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-    if (have_acc && !*abort_flag) {
-      if constexpr (CL == 1) {
+      // the staged rows reach the async proxy (the bulk copies), then the four
+      // epilogue warps meet; a wait that gave up anywhere shows in abort_flag
+      fence_proxy_async_smem();
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      if (have_acc && !*abort_flag) {
         // the thread whose row starts a run of consecutive slots copies the
         // run: c rows to (b * slots + slot) * d_c (+ c0), k^R rows to
         // (b * slots + slot) * d_r, all 16-byte aligned and sized
@@ -410,22 +515,6 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
           if constexpr (NK > 0) bulk_store(p.kr + row_id * DR, stage_k + r * NK * 2, len * NK * 2);
           bulk_commit();
           bulk_wait_read_all();  // the staged rows must outlive the copies' reads
-        }
-      } else {
-        // consecutive threads store consecutive 16-byte pieces of the rows
-        constexpr int kChunks = S::N * 2 / 16;  // 16-byte pieces per output row
-        constexpr int kChunksC = NC * 2 / 16;
-        for (int q = r; q < kBM * kChunks; q += kBM) {
-          const int row = q / kChunks, ch = q % kChunks;
-          const long long slot = slot_of[row];
-          if (slot < 0) continue;
-          const size_t row_id = static_cast<size_t>(b) * p.slots + slot;
-          if (ch < kChunksC)
-            *reinterpret_cast<uint4*>(p.c + row_id * DC + c0 + ch * 8) =
-                *reinterpret_cast<const uint4*>(stage_c + row * NC * 2 + ch * 16);
-          else
-            *reinterpret_cast<uint4*>(p.kr + row_id * DR + (ch - kChunksC) * 8) =
-                *reinterpret_cast<const uint4*>(stage_k + row * NK * 2 + (ch - kChunksC) * 16);
         }
       }
     }
@@ -472,7 +561,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // Small grids: a cluster of d_c/64 CTAs per token tile; rank q computes c
 // columns [64q, 64q + 64), the last rank k^R as well.
 template <int DC, int DR>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kClusterThreads, 1)
     mla_append_tc_cluster_kernel(const __grid_constant__ CUtensorMap tm_x,
                                  const __grid_constant__ CUtensorMap tm_wc,
                                  const __grid_constant__ CUtensorMap tm_wk,
@@ -512,7 +601,7 @@ int launch_tc(const AppendArgs& a) {
         int n = 0;
         cudaLaunchConfig_t oc = {};
         oc.gridDim = dim3(kCl * static_cast<unsigned>(clusters), 1, 1);
-        oc.blockDim = dim3(kThreads, 1, 1);
+        oc.blockDim = dim3(kClusterThreads, 1, 1);
         oc.dynamicSmemBytes = kSm;
         cudaLaunchAttribute oa[1];
         oa[0].id = cudaLaunchAttributeClusterDimension;
@@ -596,7 +685,7 @@ int launch_tc(const AppendArgs& a) {
   kp.pf_blocks = x2 ? kPrefetchX2 : kPrefetchOne;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cluster ? tiles * kCl : tiles, a.batch, kSplit ? 2 : 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.blockDim = dim3(cluster ? kClusterThreads : kThreads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = a.stream;
   cudaLaunchAttribute attr[2];
