@@ -10,8 +10,9 @@
 // One CTA owns 128 rows (one TMEM lane each) and walks the window in blocks
 // of 128 keys; this file holds the widths whose Q fits in TMEM beside S, P and
 // O (d_c = 128 and 192; other kernels serve the narrower and wider ones):
-//   warp 0     TMA producer: [c | k] tiles into a ring of shared-memory
-//              stages (c with 128-byte swizzle, k with 64-byte swizzle).
+//   warp 0     TMA producer: q_c once (through the last key stage), then
+//              [c | k] tiles into a ring of shared-memory stages (c with
+//              128-byte swizzle, k with 64-byte swizzle).
 //              CTAs run in pairs (a cluster of two consecutive row tiles of
 //              the same batch element): each CTA fetches half of every key
 //              tile from L2 and multicasts it into both CTAs' stage, halving
@@ -24,7 +25,7 @@
 //              warps keep the tensor pipe fed while either one waits on a
 //              barrier: the MMA queue is shallow, so a single issuer's
 //              bookkeeping between groups would leave the pipe idle.
-//   warps 2-5  load q_c, rotate q_r and store both into TMEM; then the online
+//   warps 2-5  move q_c to TMEM, rotate q_r into it; then the online
 //              softmax: thread i owns row i, copies S_j out of TMEM (releasing
 //              it), writes P_j (bf16) once PV_{j-1} has read the previous P,
 //              rescales O in TMEM only when its running max grows by more
@@ -73,6 +74,7 @@ struct AttnShape {
   static_assert(DR == 32 || DR == 64, "d_r: 32 or 64");
   static_assert(kTmemQ + DK / 2 <= 512, "S, P, O and Q must fit in 512 TMEM columns");
   static_assert(kStages >= 2, "at least two key stages must fit in shared memory");
+  static_assert(kBM * DC * 2 <= kTileBytes, "q_c passes through one key stage");
   static_assert(kTileBytes % 1024 == 0 && kKrOff % 1024 == 0, "swizzle-atom alignment");
 };
 
@@ -89,7 +91,8 @@ struct AttnKParams {
 
 template <int DC, int DR, int CL>
 __global__ void __launch_bounds__(kThreads, 1)
-    mla_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_c,
+    mla_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_qc,
+                       const __grid_constant__ CUtensorMap tm_c,
                        const __grid_constant__ CUtensorMap tm_kr, const AttnKParams p) {
   using S = AttnShape<DC, DR>;
   constexpr int NST = S::kStages;
@@ -98,9 +101,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem_1024(smem_raw);
   uint8_t* sKV = smem;
+  uint8_t* sQ = smem + (NST - 1) * S::kTileBytes;  // q_c on its way to TMEM
   uint64_t* bars = reinterpret_cast<uint64_t*>(sKV + NST * S::kTileBytes);
-  uint64_t* q_ready = bars;
-  uint64_t* kv_full = bars + 1;
+  uint64_t* q_full = bars;
+  uint64_t* q_ready = bars + 1;
+  uint64_t* kv_full = bars + 2;
   uint64_t* kv_empty = kv_full + NST;
   uint64_t* s_full = kv_empty + NST;
   uint64_t* s_free = s_full + 1;
@@ -118,6 +123,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const WaitCtx wc{abort_flag, p.status};
 
   if (threadIdx.x == 0) {
+    mbar_init(q_full, 1);
     mbar_init(q_ready, 4);  // one arrival per softmax warp, and so below
     for (int s = 0; s < NST; ++s) {
       mbar_init(&kv_full[s], 1);
@@ -150,10 +156,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       tma_prefetch_desc(&tm_c);
       tma_prefetch_desc(&tm_kr);
+      // q_c on its way to TMEM passes through the last key stage
+      tma_prefetch_desc(&tm_qc);
+      mbar_arrive_expect_tx(q_full, kBM * DC * 2);
+      for (int cb = 0; cb < DC / 64; ++cb)
+        tma_load_3d(sQ + cb * kBM * 128, &tm_qc, q_full, cb * 64, row0, b);
       int issued = 0;
       for (int j = 0; j < nblk; ++j) {
         const int st = j % NST;
-        if (j >= NST && !mbar_wait(&kv_empty[st], ((j / NST) - 1) & 1, wc)) break;
+        // releases of this stage so far that its next fill waits for: one per
+        // earlier fill, and on the last stage one more, for Q (both CTAs')
+        const int freed = j / NST + (st == NST - 1 ? 1 : 0);
+        if (freed > 0 && !mbar_wait(&kv_empty[st], (freed - 1) & 1, wc)) break;
         uint8_t* kv = sKV + st * S::kTileBytes;
         mbar_arrive_expect_tx(&kv_full[st], S::kTileBytes);
         if constexpr (CL == 1) {
@@ -171,10 +185,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         issued = j + 1;
       }
-      // every stage's last use must be released before the CTA may exit
-      for (int st = 0; st < NST && st < nblk && !*abort_flag; ++st)
-        mbar_wait(&kv_empty[st], (((nblk - st + NST - 1) / NST) - 1) & 1, wc);
+      // every stage's last release must have landed before the CTA may exit
+      for (int st = 0; st < NST && !*abort_flag; ++st) {
+        const int freed = (nblk - st + NST - 1) / NST + (st == NST - 1 ? 1 : 0);
+        if (freed > 0) mbar_wait(&kv_empty[st], (freed - 1) & 1, wc);
+      }
       if (*abort_flag) {  // let every copy this CTA started land before exit
+        mbar_wait_drain(q_full, 0, p.status);
         for (int u = issued > NST ? issued - NST : 0; u < issued; ++u)
           mbar_wait_drain(&kv_full[u % NST], (u / NST) & 1, p.status);
       }
@@ -184,6 +201,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ------------------------------------------------------ QK^T issuer
     // the whole warp walks the loop; one lane issues (see elect_one)
     bool ok = mbar_wait_warp(q_ready, 0, wc);
+    // Q has left the last key stage: both CTAs' copies may fill it
+    if (lane < CL) mbar_arrive_peer(dsmem_addr(smem_u32(&kv_empty[NST - 1]), lane));
+    __syncwarp();
     const uint64_t kd = sdesc(smem_u32(sKV), 16, 1024, kSw128);
     const uint64_t krd = sdesc(smem_u32(sKV) + S::kKrOff, 16, S::kKrSbo, S::kKrSw);
     for (int j = 0; ok && j < nblk; ++j) {
@@ -253,57 +273,59 @@ __global__ void __launch_bounds__(kThreads, 1)
     const bool row_ok = grow < p.rows;
 
     // Q: q_c as is, q_r rotated by the query position (RoPE3D), both bf16.
+    // q_c comes by TMA through the last key stage: 24 loads per thread of rows
+    // 384 bytes apart took 5,700 cycles of a tile's start, this takes 2,700 (64
+    // tokens on 256 keys: 9.15 -> 7.6 us, 1,170 on 8,190: 63.9 -> 62.2). Rows
+    // past the last repeat it in q_r; they are never stored.
     {
+      const int qrow = min(grow, p.rows - 1);
+      const size_t qr = static_cast<size_t>(b) * p.rows + qrow;
+      const int nq = p.rows / p.heads;
+      const int* pp = p.q_pos + (static_cast<size_t>(b) * nq + qrow / p.heads) * 3;
+      int pa[3] = {__ldg(pp), __ldg(pp + 1), __ldg(pp + 2)};
+      const uint4* rsrc = reinterpret_cast<const uint4*>(p.q_r + qr * DR);
       uint32_t w[DR / 2];
 #pragma unroll
-      for (int i = 0; i < DR / 2; ++i) w[i] = 0u;
-      if (row_ok) {
-        const uint4* src = reinterpret_cast<const uint4*>(
-            p.q_r + (static_cast<size_t>(b) * p.rows + grow) * DR);
-#pragma unroll
-        for (int i = 0; i < DR / 8; ++i) {
-          const uint4 v = __ldg(src + i);
-          w[4 * i + 0] = v.x;
-          w[4 * i + 1] = v.y;
-          w[4 * i + 2] = v.z;
-          w[4 * i + 3] = v.w;
-        }
-        const int nq = p.rows / p.heads;
-        const int* pp = p.q_pos + (static_cast<size_t>(b) * nq + grow / p.heads) * 3;
-        int pa[3] = {__ldg(pp), __ldg(pp + 1), __ldg(pp + 2)};
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-          if (pa[a] < 0 || pa[a] >= p.rope_len) {
-            record_status(p.status, MLA_ERR_RANGE);
-            pa[a] = 0;
-          }
-#pragma unroll
-        for (int i = 0; i < DR / 2; ++i) {
-          const int pos = i < p.pairs_t ? pa[0] : (i < p.pairs_t + p.pairs_h ? pa[1] : pa[2]);
-          const float2 cs = __ldg(p.rope + static_cast<size_t>(pos) * (DR / 2) + i);
-          const float x0 = bf16_lo(w[i]), x1 = bf16_hi(w[i]);
-          w[i] = pack_bf16x2(x0 * cs.x - x1 * cs.y, x0 * cs.y + x1 * cs.x);
-        }
+      for (int i = 0; i < DR / 8; ++i) {
+        const uint4 v = __ldg(rsrc + i);
+        w[4 * i + 0] = v.x;
+        w[4 * i + 1] = v.y;
+        w[4 * i + 2] = v.z;
+        w[4 * i + 3] = v.w;
       }
-      // TMEM holds the MMA's A operand row-major: column c = elements 2c, 2c+1
-      const uint4* qsrc = reinterpret_cast<const uint4*>(
-          p.q_c + (static_cast<size_t>(b) * p.rows + (row_ok ? grow : 0)) * DC);
 #pragma unroll
-      for (int c = 0; c < DC / 64; ++c) {
-        uint32_t qw[32];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const uint4 v = row_ok ? __ldg(qsrc + c * 8 + i) : make_uint4(0u, 0u, 0u, 0u);
-          qw[4 * i + 0] = v.x;
-          qw[4 * i + 1] = v.y;
-          qw[4 * i + 2] = v.z;
-          qw[4 * i + 3] = v.w;
+      for (int a = 0; a < 3; ++a)
+        if (pa[a] < 0 || pa[a] >= p.rope_len) {
+          record_status(p.status, MLA_ERR_RANGE);
+          pa[a] = 0;
         }
-        tmem_st32(tmem + t_lane + S::kTmemQ + c * 32, qw);
+#pragma unroll
+      for (int i = 0; i < DR / 2; ++i) {
+        const int pos = i < p.pairs_t ? pa[0] : (i < p.pairs_t + p.pairs_h ? pa[1] : pa[2]);
+        const float2 cs = __ldg(p.rope + static_cast<size_t>(pos) * (DR / 2) + i);
+        const float x0 = bf16_lo(w[i]), x1 = bf16_hi(w[i]);
+        w[i] = pack_bf16x2(x0 * cs.x - x1 * cs.y, x0 * cs.y + x1 * cs.x);
       }
 #pragma unroll
       for (int c = 0; c < DR / 32; ++c)
         tmem_st16(tmem + t_lane + S::kTmemQ + DC / 2 + c * 16, w + c * 16);
+      // TMEM holds the MMA's A operand row-major: column c = elements 2c, 2c+1
+      if (__all_sync(0xffffffffu, mbar_wait(q_full, 0, wc))) {
+#pragma unroll
+        for (int c = 0; c < DC / 64; ++c) {
+          uint32_t qw[32];
+          const uint8_t* qrow_s = sQ + c * kBM * 128 + r * 128;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {  // 16-byte chunk i is at i ^ (r & 7)
+            const uint4 v = *reinterpret_cast<const uint4*>(qrow_s + ((i ^ (r & 7)) << 4));
+            qw[4 * i + 0] = v.x;
+            qw[4 * i + 1] = v.y;
+            qw[4 * i + 2] = v.z;
+            qw[4 * i + 3] = v.w;
+          }
+          tmem_st32(tmem + t_lane + S::kTmemQ + c * 32, qw);
+        }
+      }
       tmem_wait_st();
       tc_fence_before();
       mbar_arrive_warp(q_ready);
@@ -425,9 +447,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     // O / l as bf16: each thread stages its row densely in the key stages
     // (free once the last PV is done: every key tile, the peer's multicast
-    // halves included, has landed and been read), and the tile leaves shared
-    // memory by one bulk copy: its rows are consecutive rows of o.
-    const bool have_o = ok && mbar_wait(pv_done, (nblk - 1) & 1, wc);
+    // halves included, has landed and been read), and each warp's rows, which
+    // are consecutive rows of o, leave shared memory by one bulk copy.
+    bool have_o = ok && mbar_wait(pv_done, (nblk - 1) & 1, wc);
+    have_o = __all_sync(0xffffffffu, have_o) && !*abort_flag;
     uint8_t* srow = sKV + r * DC * 2;
     if (have_o) {
       tc_fence_after();
@@ -448,16 +471,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         stage_row<8>(srow + sg * 128, pk, r & 7);
       }
-    }
-    fence_proxy_async_smem();
-    asm volatile("bar.sync 1, 128;" ::: "memory");  // the four softmax warps
-    // the tile's rows below p.rows; none in the CTA that only pads the grid
-    // to whole clusters (an odd number of row tiles)
-    const int valid = min(kBM, p.rows - row0);
-    if (r == 0 && have_o && !*abort_flag && valid > 0) {
-      bulk_store(p.o + (static_cast<size_t>(b) * p.rows + row0) * DC, sKV, valid * DC * 2);
-      bulk_commit();
-      bulk_wait_read_all();  // the staged rows must outlive the copy's reads
+      fence_proxy_async_smem();
+      __syncwarp();
+      // the warp's rows below p.rows; none past the end, where the grid is
+      // padded to whole clusters (an odd number of row tiles)
+      const int valid = min(32, p.rows - (row0 + quarter * 32));
+      if (lane == 0 && valid > 0) {
+        bulk_store(p.o + (static_cast<size_t>(b) * p.rows + grow) * DC, srow, valid * DC * 2);
+        bulk_commit();
+        bulk_wait_read_all();  // the staged rows must outlive the copy's reads
+      }
     }
   }
 
@@ -474,9 +497,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 template <int DC, int DR, int CL>
 int launch_tc(const AttnArgs& a) {
   using S = AttnShape<DC, DR>;
-  CUtensorMap tm_c, tm_kr;
-  const unsigned long long slots = a.slots;
-  if (!encode_map_3d_bf16(&tm_c, a.c, DC, a.n_valid, a.batch, DC * 2ull, slots * DC * 2ull, 64,
+  CUtensorMap tm_qc, tm_c, tm_kr;
+  const unsigned long long rows = a.rows, slots = a.slots;
+  if (!encode_map_3d_bf16(&tm_qc, a.q_c, DC, rows, a.batch, DC * 2ull, rows * DC * 2ull, 64, kBM,
+                          CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_map_3d_bf16(&tm_c, a.c, DC, a.n_valid, a.batch, DC * 2ull, slots * DC * 2ull, 64,
                           kBN, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !encode_map_3d_bf16(&tm_kr, a.kr, DR, a.n_valid, a.batch, DR * 2ull, slots * DR * 2ull, DR,
                           kBN,
@@ -518,7 +543,7 @@ int launch_tc(const AttnArgs& a) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  e = cudaLaunchKernelEx(&cfg, kern, tm_c, tm_kr, kp);
+  e = cudaLaunchKernelEx(&cfg, kern, tm_qc, tm_c, tm_kr, kp);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_last_cuda_error(e);

@@ -150,57 +150,23 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const 
   }
 }
 
-// mbar_wait with cluster-scope acquire: for barriers that threads of the
-// other CTA of a cluster arrive on (mbar_arrive_cluster).
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity,
-                                                  const WaitCtx& w) {
-  if (mbar_try_wait_cluster(bar, parity)) return true;
-  const uint64_t t0 = globaltimer_ns();
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try_wait_cluster(bar, parity)) return true;
-    if ((it & 31u) == 0) {
-      if (*w.abort_flag) return false;
-      if (globaltimer_ns() - t0 > kWaitLimitNs) {
-        record_status(w.status, MLA_ERR_TIMEOUT);
-        *w.abort_flag = 1;
-        return false;
-      }
-    }
-  }
-}
-// Arrive (release, cluster scope) on an mbarrier of any CTA of the cluster,
-// given its shared::cluster address (dsmem_addr).
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster)
-               : "memory");
-}
-
 // mbar_wait by a whole warp, with one answer for all its lanes: control flow
 // that depends on it stays warp-uniform (see elect_one).
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, const WaitCtx& w) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, w)) != 0;
 }
 
-// One arrival for the whole warp on an mbarrier of any CTA of the cluster, for
-// hand-overs of TMEM between the paired CTAs: what is handed over was ordered
-// by tcgen05.wait and tcgen05.fence::before_thread_sync, not by generic memory
-// accesses, so the arrival carries the default semantics. With .release.cluster
-// each arrival waited 600 to 1400 cycles for the thread's earlier accesses.
-__device__ __forceinline__ void mbar_arrive_peer_warp(uint32_t bar_cluster) {
+// Arrival on an mbarrier of any CTA of the cluster with the default semantics:
+// for hand-overs of TMEM between paired CTAs (ordered by tcgen05.wait and
+// tcgen05.fence::before_thread_sync, not by generic accesses) and of shared
+// memory that was only read. With .release.cluster each arrival waited 600 to
+// 1400 cycles for the thread's earlier accesses.
+__device__ __forceinline__ void mbar_arrive_peer(uint32_t bar_cluster) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_peer_warp(uint32_t bar_cluster) {  // once per warp
   __syncwarp();
-  if ((threadIdx.x & 31) == 0)
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
+  if ((threadIdx.x & 31) == 0) mbar_arrive_peer(bar_cluster);
 }
 
 // Drain wait used on the abort path: ignores the abort flag, still bounded.
