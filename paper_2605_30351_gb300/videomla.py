@@ -158,21 +158,27 @@ def mla_rope_table_fill(cfg):
 
 
 def _stream_ptr(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is None:  # the current device's current stream, as a raw handle
+        if not torch.cuda.is_initialized():
+            torch.cuda.init()
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
 def _dev(t, dtype, shape, name):
+    """Device address of a dense CUDA tensor of this type and shape. One chain
+    of cheap tests on the path of a good argument: it runs for every tensor of
+    every call."""
+    if (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is dtype and t.shape == shape
+            and t.is_contiguous()):
+        return t.data_ptr()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if tuple(t.shape) != tuple(shape):
         raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
-    if not t.is_contiguous():
-        raise ValueError(f"{name} must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    raise ValueError(f"{name} must be contiguous")
 
 
 class LatentCache:
@@ -264,7 +270,7 @@ def mla_attention_window_forward(cache, q_c, q_r, q_pos, frame_hw, workspace, o_
                _dev(q_r, bf, (cfg.batch, Nq, cfg.heads, cfg.d_r), "q_r"),
                _dev(q_pos, torch.int32, (cfg.batch, Nq, 3), "q_pos"), int(Nq),
                _dev(frame_hw, torch.int32, (cfg.tokens_per_frame, 2), "frame_hw"),
-               ctypes.c_void_p(workspace.data_ptr()),
+               workspace.data_ptr(),
                workspace.numel() * workspace.element_size(),
                _dev(o_lat, bf, (cfg.batch, Nq, cfg.heads, cfg.d_c), "o_lat"),
                _stream_ptr(stream)))
@@ -304,8 +310,8 @@ def mla_absorb_weights(cfg, w_uq, w_uk, w_qr, gamma_q, w_uv, w_o, stream=None):
     w_qcat = torch.empty(sq, dtype=bf, device=w_uq.device)
     w_b = torch.empty(sb, dtype=bf, device=w_uq.device)
     _check("mla_absorb_weights",
-           load().mla_absorb_weights(ctypes.byref(cfg), *args, ctypes.c_void_p(w_qcat.data_ptr()),
-                                     ctypes.c_void_p(w_b.data_ptr()), _stream_ptr(stream)))
+           load().mla_absorb_weights(ctypes.byref(cfg), *args, w_qcat.data_ptr(),
+                                     w_b.data_ptr(), _stream_ptr(stream)))
     return w_qcat, w_b
 
 
@@ -323,7 +329,7 @@ def mla_query_prologue(cfg, x, w_dq, w_qcat, workspace, q_c, q_r, stream=None):
            load().mla_query_prologue(
                ctypes.byref(cfg), _dev(x, bf, (cfg.batch, Nq, d), "x"),
                _dev(w_dq, bf, (dq, d), "w_dq"), _dev(w_qcat, bf, (H * (dc + dr), dq), "w_qcat"),
-               int(Nq), ctypes.c_void_p(workspace.data_ptr()),
+               int(Nq), workspace.data_ptr(),
                workspace.numel() * workspace.element_size(),
                _dev(q_c, bf, (cfg.batch, Nq, H, dc), "q_c"),
                _dev(q_r, bf, (cfg.batch, Nq, H, dr), "q_r"), _stream_ptr(stream)))
