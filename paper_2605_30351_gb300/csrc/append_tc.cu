@@ -23,12 +23,11 @@
 // one accumulates c (two N = 256 MMAs per K step) and applies RMSNorm, the
 // other accumulates k^R and applies RoPE. Both stream the same x tile.
 // When one CTA per token tile would leave most SMs idle (one chunk at batch
-// 1), a cluster of d_c/64 CTAs shares each token tile, one per 64 columns of
-// c (see AppendShape). When the tiles exceed one wave, two CTAs with fewer
+// 1), a cluster of CTAs shares each token tile, each taking a slice of c's
+// columns (see AppendShape). When the tiles exceed one wave, two CTAs with fewer
 // stages share each SM, so that one's start-up and epilogue overlap the
 // other's K loop.
 #include <cmath>
-#include <type_traits>
 
 #include "internal.h"
 #include "ptx_sm103.cuh"
@@ -59,9 +58,9 @@ constexpr int kPrefetchX2 = 12;
 //    alone, two CTAs per token tile that need nothing from each other
 //    (RMSNorm runs over c alone);
 //  - a grid too small to occupy the SMs (one chunk at batch 1): a cluster
-//    of CL = d_c/64 CTAs per token tile, one per 64 columns of c, the last
-//    also computing k^R, so that each SM streams the token tile and only its
-//    share of the weights. Every CTA fetches the whole x box (from L2 after
+//    of CL CTAs per token tile, one per d_c/CL columns of c, the last also
+//    computing k^R, so that each SM streams the token tile and only its share
+//    of the weights. Every CTA fetches the whole x box (from L2 after
 //    the first), so the CTAs' K loops do not wait on one another; they
 //    exchange their partial RMSNorm sums of squares through distributed
 //    shared memory.
@@ -74,7 +73,7 @@ struct AppendShape {
   // rows of a stage's weight region: in a cluster every CTA takes the widest
   // slice's layout (one shared-memory size for the launch, and the partial
   // sums at the same offset in every CTA)
-  static constexpr int kBRows = CL > 1 ? 64 + DR : N;
+  static constexpr int kBRows = CL > 1 ? NC + DR : N;
   static constexpr int kBBytes = kBRows * kBK * 2;
   static constexpr int kWTxBytes = N * kBK * 2;  // weight bytes of a K block in this CTA
   static constexpr int kBlockBytes = kABytes + kBBytes;  // one K block: x, then weights
@@ -93,13 +92,14 @@ struct AppendShape {
   static constexpr uint32_t kTmemCols = N <= 32 ? 32 : (N <= 64 ? 64 : (N <= 256 ? 256 : 512));
   // output staging: dense c rows, dense k^R rows, then the rows' slots
   static_assert(kBM * N * 2 + kBM * 8 + 16 <= kStages * kStageBytes, "staging fits in the ring");
-  static_assert(NC % 64 == 0 && (NK == 0 || NK == 32 || NK == 64), "staged row segments");
+  static_assert((NC % 64 == 0 || CL > 1) && (NK == 0 || NK == 32 || NK == 64),
+                "staged row segments");
   static_assert(DC % 32 == 0 && DR % 32 == 0 && DR <= 64 && (DC <= 256 || DC % 256 == 0),
                 "shape");
   static_assert(N > 0 && NC % 32 == 0 && (NK == 0 || NK == DR), "parts");
   static_assert((NC == DC && NK == DR && CL == 1) || (DC > 256 && CL == 1) ||
-                    (CL == DC / 64 && CL >= 2 && DC <= 256 && NC == 64),
-                "parts are split for d_c > 256, or over a cluster of 64-column slices");
+                    (CL >= 2 && CL <= 8 && NC * CL == DC && NC <= 128),
+                "parts are split for d_c > 256, or over a cluster of slices");
   static_assert(N <= 512, "accumulator must fit in TMEM");
   static_assert(kStageBytes % 1024 == 0 && kWcBox > 0, "swizzle-atom alignment");
   static_assert(kStages >= 2, "smem");
@@ -348,22 +348,22 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
     asm volatile("bar.sync 1, 128;" ::: "memory");  // gamma_s is complete
     const bool have_acc = mbar_wait(acc_full, 0, wc) && !*abort_flag;
     if constexpr (CL > 1) {
-      // This CTA's 64 columns of c stay in registers between the statistics and
-      // the store, and each thread writes its row's pieces (128 bytes of c,
+      // This CTA's columns of c stay in registers between the statistics and
+      // the store, and each thread writes its row's pieces (NC values of c,
       // d_r values of k^R) straight from registers: a slice's rows are not
       // contiguous in the cache, and staging them for a coalesced loop took
       // longer than the whole of this (64 tokens: 8.8 -> 7.3 us, one Wan chunk:
       // 9.65 -> 8.7 us).
-      static_assert(CL == 1 || NC == 64, "one 64-column slice per CTA");
-      uint32_t v[64];
+      uint32_t v[NC];
       float ss = 0.f;
       if (have_acc) {
         tc_fence_after();
-        tmem_ld32(t_row, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
-        tmem_ld32(t_row + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
+#pragma unroll
+        for (int cb = 0; cb < NC / 32; ++cb)
+          tmem_ld32(t_row + cb * 32, *reinterpret_cast<uint32_t(*)[32]>(&v[cb * 32]));
         tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 64; ++i) {
+        for (int i = 0; i < NC; ++i) {
           const float f = __uint_as_float(v[i]);
           ss = fmaf(f, f, ss);
         }
@@ -372,7 +372,7 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
       // every CTA, then all threads of the cluster pass the second barrier
       // phase (release / acquire), on every path, so that no CTA waits for
       // one that left; after it the sums are read locally, in rank order
-      const uint32_t local = smem_u32(ss_all + (c0 / 64) * kBM + r);
+      const uint32_t local = smem_u32(ss_all + (c0 / NC) * kBM + r);
       for (int q = 0; q < CL; ++q) dsmem_st_f32(dsmem_addr(local, q), ss);
       cluster_arrive_release();
       const bool store = have_acc && my_slot >= 0 && !*abort_flag;
@@ -408,7 +408,7 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
         const uint4* g4 = gamma_s;
         uint4* dst = reinterpret_cast<uint4*>(p.c + row_id * DC + c0);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < NC / 8; ++i) {
           const uint4 g = g4[i];
           const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
           uint32_t w[4];
@@ -558,105 +558,134 @@ __global__ void __launch_bounds__(kThreads, 1)
     append_body<DC, DR, 0, DR, 1>(&tm_x, &tm_wc, &tm_wk, p, blockIdx.x, 0);
 }
 
-// Small grids: a cluster of d_c/64 CTAs per token tile; rank q computes c
-// columns [64q, 64q + 64), the last rank k^R as well.
-template <int DC, int DR>
+// Small grids: a cluster of CL CTAs per token tile; rank q computes c columns
+// [q NC, (q + 1) NC), NC = d_c / CL, the last rank k^R as well.
+template <int DC, int DR, int CL>
 __global__ void __launch_bounds__(kClusterThreads, 1)
     mla_append_tc_cluster_kernel(const __grid_constant__ CUtensorMap tm_x,
                                  const __grid_constant__ CUtensorMap tm_wc,
                                  const __grid_constant__ CUtensorMap tm_wk,
                                  const AppendKParams p) {
-  constexpr int CL = DC / 64;
+  constexpr int NC = DC / CL;
   const int q = static_cast<int>(cluster_ctarank());
   const int tile = blockIdx.x / CL;
   if (q < CL - 1)
-    append_body<DC, DR, 64, 0, CL>(&tm_x, &tm_wc, &tm_wk, p, tile, q * 64);
+    append_body<DC, DR, NC, 0, CL>(&tm_x, &tm_wc, &tm_wk, p, tile, q * NC);
   else
-    append_body<DC, DR, 64, DR, CL>(&tm_x, &tm_wc, &tm_wk, p, tile, q * 64);
+    append_body<DC, DR, NC, DR, CL>(&tm_x, &tm_wc, &tm_wk, p, tile, q * NC);
+}
+
+using KernFn = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, AppendKParams);
+
+// One way to launch an append: the kernel and what it takes.
+struct AppendForm {
+  KernFn kern;
+  int smem, threads;
+  int cl;        // CTAs per token tile (a cluster), 1: none
+  int z;         // grid depth (2: the c and k^R halves of d_c = 512)
+  int wc_box;    // W_dkv rows per TMA box
+  int per_sm;    // CTAs per SM
+  int pf_blocks;
+};
+
+// The cluster form of CL CTAs per tile, when all its clusters fit in `waves`
+// rounds of those that are resident at once.
+template <int DC, int DR, int CL>
+bool cluster_form(long long tiles, AppendForm* f, int waves = 1) {
+  using SC0 = AppendShape<DC, DR, DC / CL, 0, CL>;
+  using SC1 = AppendShape<DC, DR, DC / CL, DR, CL>;
+  constexpr int kSm = SC0::kSmemBytes > SC1::kSmemBytes ? SC0::kSmemBytes : SC1::kSmemBytes;
+  static const int resident = [] {  // per process, for this instantiation
+    auto kern = mla_append_tc_cluster_kernel<DC, DR, CL>;
+    int n = 0;
+    cudaLaunchConfig_t oc = {};
+    oc.gridDim = dim3(CL, 1, 1);
+    oc.blockDim = dim3(kClusterThreads, 1, 1);
+    oc.dynamicSmemBytes = kSm;
+    cudaLaunchAttribute oa[1];
+    oa[0].id = cudaLaunchAttributeClusterDimension;
+    oa[0].val.clusterDim.x = CL;
+    oa[0].val.clusterDim.y = 1;
+    oa[0].val.clusterDim.z = 1;
+    oc.attrs = oa;
+    oc.numAttrs = 1;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSm) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kern, &oc) != cudaSuccess) {
+      cudaGetLastError();  // a failed query only disables the cluster form
+      n = 0;
+    }
+    return n;
+  }();
+  if (tiles > static_cast<long long>(resident) * waves) return false;
+  *f = {mla_append_tc_cluster_kernel<DC, DR, CL>, kSm, kClusterThreads, CL, 1, SC0::kWcBox, 1,
+        kPrefetchOne};
+  return true;
 }
 
 template <int DC, int DR>
-int launch_tc(const AppendArgs& a) {
+AppendForm pick_form(long long tiles, int sms) {
   constexpr bool kSplit = DC > 256;
-  constexpr bool kClusterable = DC >= 128 && DC <= 256;
-  constexpr int kCl = kClusterable ? DC / 64 : 2;  // cluster size of the small-grid form
-  const int tiles = (a.n_tok + kBM - 1) / kBM;
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) == cudaSuccess)
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // the cluster form when its CTAs all fit in one wave (e.g. one Wan chunk at
-  // batch 1: 37 tiles x 3 = 111 CTAs) and every cluster is resident at once;
-  // otherwise one CTA per tile already fills the SMs and streaming the
-  // weights once per tile is the cheaper way
-  bool cluster = false;
-  if constexpr (kClusterable) {
-    const long long clusters = static_cast<long long>(tiles) * a.batch;
-    if (clusters * kCl <= sms) {
-      static int resident = -1;  // co-resident clusters of this shape (per process)
-      if (resident < 0) {
-        using SC0 = AppendShape<DC, DR, 64, 0, kCl>;
-        using SC1 = AppendShape<DC, DR, 64, DR, kCl>;
-        constexpr int kSm = SC0::kSmemBytes > SC1::kSmemBytes ? SC0::kSmemBytes : SC1::kSmemBytes;
-        auto kc = mla_append_tc_cluster_kernel<DC, DR>;
-        int n = 0;
-        cudaLaunchConfig_t oc = {};
-        oc.gridDim = dim3(kCl * static_cast<unsigned>(clusters), 1, 1);
-        oc.blockDim = dim3(kClusterThreads, 1, 1);
-        oc.dynamicSmemBytes = kSm;
-        cudaLaunchAttribute oa[1];
-        oa[0].id = cudaLaunchAttributeClusterDimension;
-        oa[0].val.clusterDim.x = kCl;
-        oa[0].val.clusterDim.y = 1;
-        oa[0].val.clusterDim.z = 1;
-        oc.attrs = oa;
-        oc.numAttrs = 1;
-        if (cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSm) !=
-                cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&n, kc, &oc) != cudaSuccess) {
-          cudaGetLastError();  // a failed query only disables the cluster form
-          n = 0;
-        }
-        resident = n;
-      }
-      cluster = clusters <= resident;
-    }
+  AppendForm f = {};
+  // A cluster per tile when its CTAs all fit in one wave (one Wan chunk at
+  // batch 1, d_c = 192: 37 tiles x 3), the larger clusters first: a CTA's K
+  // loop is as long as its share of the weights makes it. Beyond that one CTA
+  // per tile fills the SMs and streaming the weights once per tile is the
+  // cheaper way; at d_c = 512, whose halves stream all of W_dkv through one SM,
+  // two rounds of clusters still win. One chunk (37 tiles), against one CTA per
+  // tile: d_c = 128 12.1 -> 7.9 us, 192 11.8 (clusters of another make) -> 8.7,
+  // 256 15.1 -> 10.2, 512 23.9 -> 18.7; two chunks 13.4 -> 9.3, 12.7 -> 11.3,
+  // 16.2 -> 11.9; 128 tokens 11.2 -> 7.4, 11.0 -> 7.9, 11.3 -> 7.7, 22.4 -> 7.9.
+  if constexpr (DC == 128) {
+    if (cluster_form<DC, DR, 2>(tiles, &f)) return f;
+  } else if constexpr (DC == 192) {
+    if (cluster_form<DC, DR, 3>(tiles, &f) || cluster_form<DC, DR, 2>(tiles, &f))
+      return f;
+  } else if constexpr (DC == 256) {
+    if (cluster_form<DC, DR, 4>(tiles, &f) || cluster_form<DC, DR, 2>(tiles, &f))
+      return f;
+  } else if constexpr (DC == 512) {
+    if (cluster_form<DC, DR, 8>(tiles, &f) || cluster_form<DC, DR, 4>(tiles, &f, 2))
+      return f;
   }
   // two CTAs per SM when the grid has more than one wave of single CTAs and
   // two stages of the unsplit form fit in half an SM's shared memory
   constexpr int kStageX2 = kBM * kBK * 2 + (DC + DR) * kBK * 2;
   constexpr bool kX2Fits = !kSplit && DC + DR <= 256 &&  // two 256-column TMEM accumulators
                            (kSmemHalf - 1024 - 256 - DC * 2) / kStageX2 >= 2;
-  const bool x2 = kX2Fits && !cluster && static_cast<long long>(tiles) * a.batch > sms;
-  // shapes of the CTAs each form launches (d_c > 256: the c and k^R halves;
-  // the cluster form: a 64-column c slice and k^R; else both parts)
+  if constexpr (kX2Fits) {
+    if (tiles > sms) {
+      using S2 = AppendShape<DC, DR, DC, DR, 1, kSmemHalf>;
+      return {mla_append_tc_kernel_x2<DC, DR>, S2::kSmemBytes, kThreads, 1, 1, S2::kWcBox, 2,
+              kPrefetchX2};
+    }
+  }
+  // one CTA per tile, or the c and k^R halves (d_c > 256)
   using S = AppendShape<DC, DR, DC, kSplit ? 0 : DR>;
   using SK = AppendShape<DC, DR, kSplit ? 0 : DC, DR>;
-  using SCc = std::conditional_t<kClusterable, AppendShape<DC, DR, 64, 0, kCl>, S>;
-  using SCk = std::conditional_t<kClusterable, AppendShape<DC, DR, 64, DR, kCl>, S>;
-  constexpr int kSmemPlain = S::kSmemBytes > SK::kSmemBytes ? S::kSmemBytes : SK::kSmemBytes;
-  constexpr int kSmemCl = SCc::kSmemBytes > SCk::kSmemBytes ? SCc::kSmemBytes : SCk::kSmemBytes;
-  int smem = cluster ? kSmemCl : kSmemPlain;
-  if constexpr (kX2Fits)
-    if (x2) smem = AppendShape<DC, DR, DC, DR, 1, kSmemHalf>::kSmemBytes;
+  constexpr int kSm = S::kSmemBytes > SK::kSmemBytes ? S::kSmemBytes : SK::kSmemBytes;
+  if constexpr (kSplit)
+    return {mla_append_tc_split_kernel<DC, DR>, kSm, kThreads, 1, 2, S::kWcBox, 1, kPrefetchOne};
+  else
+    return {mla_append_tc_kernel<DC, DR>, kSm, kThreads, 1, 1, S::kWcBox, 1, kPrefetchOne};
+}
+
+template <int DC, int DR>
+int launch_tc(const AppendArgs& a) {
+  const int tiles = (a.n_tok + kBM - 1) / kBM;
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) == cudaSuccess)
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const AppendForm f = pick_form<DC, DR>(static_cast<long long>(tiles) * a.batch, sms);
   CUtensorMap tm_x, tm_wc, tm_wk;
   const unsigned long long H = a.hidden, n_tok = a.n_tok;
   if (!encode_map_3d_bf16(&tm_x, a.x, H, n_tok, a.batch, H * 2, n_tok * H * 2, kBK,
                           kBM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !encode_map_2d_bf16(&tm_wc, a.w_dkv, H, DC, H * 2, kBK, cluster ? 64 : S::kWcBox,
+      !encode_map_2d_bf16(&tm_wc, a.w_dkv, H, DC, H * 2, kBK, f.wc_box,
                           CU_TENSOR_MAP_SWIZZLE_128B) ||
       !encode_map_2d_bf16(&tm_wk, a.w_kr, H, DR, H * 2, kBK, DR, CU_TENSOR_MAP_SWIZZLE_128B))
     return MLA_ERR_CUDA;
-  using KernFn = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, AppendKParams);
-  KernFn kern;
-  if constexpr (kSplit)
-    kern = mla_append_tc_split_kernel<DC, DR>;
-  else if constexpr (kClusterable)
-    kern = cluster ? mla_append_tc_cluster_kernel<DC, DR> : mla_append_tc_kernel<DC, DR>;
-  else
-    kern = mla_append_tc_kernel<DC, DR>;
-  if constexpr (kX2Fits)
-    if (x2) kern = mla_append_tc_kernel_x2<DC, DR>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, f.smem);
   if (e != cudaSuccess) {
     set_last_cuda_error(e);
     return MLA_ERR_CUDA;
@@ -681,23 +710,23 @@ int launch_tc(const AppendArgs& a) {
   kp.use_rmsnorm = a.use_rmsnorm;
   kp.eps = a.eps;
   kp.status = a.status;
-  kp.first_wave = sms * (x2 ? 2 : 1);
-  kp.pf_blocks = x2 ? kPrefetchX2 : kPrefetchOne;
+  kp.first_wave = sms * f.per_sm;
+  kp.pf_blocks = f.pf_blocks;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(cluster ? tiles * kCl : tiles, a.batch, kSplit ? 2 : 1);
-  cfg.blockDim = dim3(cluster ? kClusterThreads : kThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
+  cfg.gridDim = dim3(tiles * f.cl, a.batch, f.z);
+  cfg.blockDim = dim3(f.threads, 1, 1);
+  cfg.dynamicSmemBytes = f.smem;
   cfg.stream = a.stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cluster ? kCl : 1;
+  attr[0].val.clusterDim.x = f.cl;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see grid_dep_sync
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  e = cudaLaunchKernelEx(&cfg, kern, tm_x, tm_wc, tm_wk, kp);
+  e = cudaLaunchKernelEx(&cfg, f.kern, tm_x, tm_wc, tm_wk, kp);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_last_cuda_error(e);
