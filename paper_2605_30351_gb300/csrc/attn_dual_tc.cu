@@ -28,12 +28,10 @@
 // follow each other: that form measured no faster than one tile per CTA.
 //
 // Tail of the grid: a tile's key blocks may be split over the CTAs of its
-// cluster. Each CTA then keeps its own running maximum m and sum l; at the end
-// every row has an owner among the CTAs, the others write (O, m, l) of the row
-// to the owner's shared memory, and the owner combines them:
-//     O = sum_s 2^(m_s - m) O_s / sum_s 2^(m_s - m) l_s
+// cluster; the partial results are combined at the end (attn_split.cuh).
 #include <cmath>
 
+#include "attn_split.cuh"
 #include "internal.h"
 #include "ptx_sm103.cuh"
 
@@ -64,8 +62,6 @@ struct DualShape {
   static constexpr int kSmemBytes = 1024 + 2 * kQTile + kRing * kEntry + kBarBytes;
   static constexpr int kTmemP = 2 * kBN;           // P_t at kTmemP + 64 t, two bf16 a column
   static constexpr int kTmemO = kTmemP + kBN;      // O_t at kTmemO + DV t
-  // one row of a split tile on its way to its owner: O, then m and l
-  static constexpr int kRecord = DV * 4 + 16;
   static constexpr uint32_t kKrSw = DR == 32 ? kSw64 : kSw128;
   static constexpr uint32_t kKrRow = DR * 2;
   static constexpr uint32_t kKrSbo = 8 * kKrRow;
@@ -74,7 +70,7 @@ struct DualShape {
   static_assert(DR == 0 || DR == 32 || DR == 64, "d_r");
   static_assert(kRing >= 2 * kEntriesPerBlock, "two key blocks in flight");
   static_assert(kEntry % 1024 == 0 && kQTile % 1024 == 0, "swizzle-atom alignment");
-  static_assert(2 * kBM * kRecord / kMaxCluster * (kMaxCluster - 1) <=
+  static_assert(2 * kBM / kMaxCluster * (2 * kMaxCluster - 1) * kSplitRecord<DV> <=
                     2 * kQTile + kRing * kEntry,
                 "records of a split tile fit where Q and the ring were");
 };
@@ -115,7 +111,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* p_full = s_free + 2;
   uint64_t* pv_done = p_full + 2;
   uint64_t* mma_drain = pv_done + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_drain + 2);
+  uint64_t* split_bar = mma_drain + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(split_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5;
@@ -154,6 +151,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&kv_full[s], 1);
       mbar_init(&kv_empty[s], nt);  // each tile's issuer releases it
     }
+    mbar_init(split_bar, 1);
     for (int t = 0; t < 2; ++t) {
       mbar_init(&q_ready[t], 4);  // one arrival per softmax warp, and so below
       mbar_init(&s_full[t], 1);
@@ -280,11 +278,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     __syncwarp();
-    if (n_split > 1) {  // the two barrier phases of the combination
+    if (n_split > 1) {
       cluster_arrive_release();
-      cluster_wait_acquire();
-      cluster_arrive_release();
-      cluster_wait_acquire();
+      combine_split_pass();
     }
   } else {
     // --------------------------------------------------------- softmax warps
@@ -452,101 +448,37 @@ __global__ void __launch_bounds__(kThreads, 1)
     have_o = __all_sync(0xffffffffu, have_o);
     tc_fence_after();
 
-    const size_t orow =
-        kLatent ? static_cast<size_t>(plane) * p.rows + grow
-                : (static_cast<size_t>(plane / p.heads) * p.rows + grow) * p.heads +
+    const size_t orow0 =  // the tile's first row of o
+        kLatent ? static_cast<size_t>(plane) * p.rows + row0
+                : (static_cast<size_t>(plane / p.heads) * p.rows + row0) * p.heads +
                       plane % p.heads;
-    uint4* dst = reinterpret_cast<uint4*>(p.o + orow * DV);
-    // 32 columns of O, scaled, as bf16
-    auto store32 = [&](int c, const float (&v)[32], float inv) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        dst[c * 4 + i] = make_uint4(pack_bf16x2(v[8 * i] * inv, v[8 * i + 1] * inv),
-                                    pack_bf16x2(v[8 * i + 2] * inv, v[8 * i + 3] * inv),
-                                    pack_bf16x2(v[8 * i + 4] * inv, v[8 * i + 5] * inv),
-                                    pack_bf16x2(v[8 * i + 6] * inv, v[8 * i + 7] * inv));
-    };
-    auto load32 = [&](int c, float (&v)[32]) {
-      uint32_t ov[32];
-      tmem_ld32(tO + c * 32, ov);
-      tmem_wait_ld();
-#pragma unroll
-      for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(ov[i]);
-    };
-    if (n_split == 1) {
-      if (have_o) {
-        const float inv_l = 1.f / l_run;
+    if (n_split > 1) {
+      const size_t stride = kLatent ? DV : static_cast<size_t>(p.heads) * DV;
+      // both tiles' MMAs are done with Q and the ring, where the records go
+      asm volatile("bar.sync 2, 256;" ::: "memory");
+      cluster_arrive_release();  // phase A
+      combine_split<DV, 256>(smem, smem + nt * kBM * kSplitRecord<DV>, split_bar, tO, crank,
+                             n_split, nt * kBM, t * kBM + r, have_o, m_run, l_run,
+                             p.o + orow0 * DV, stride, p.rows - row0, wc);
+    } else if (have_o) {
+      uint4* dst = reinterpret_cast<uint4*>(
+          p.o + (orow0 + static_cast<size_t>(grow - row0) * (kLatent ? 1 : p.heads)) * DV);
+      const float inv_l = 1.f / l_run;
 #pragma unroll 1
-        for (int c = 0; c < DV / 32; ++c) {
-          float v[32];
-          load32(c, v);
-          if (row_ok) store32(c, v, inv_l);
-        }
-      }
-    } else {
-      // phase 1: every CTA of the cluster is done with its shared memory
-      cluster_arrive_release();
-      cluster_wait_acquire();
-      const int per = nt * kBM / n_split;  // rows each CTA owns
-      const int lrow = t * kBM + r;
-      const int owner = lrow / per;
-      const int in_owner = lrow - owner * per;
-      if (have_o) {
-        const int slot = crank < owner ? crank : crank - 1;  // among the owner's n_split - 1
-        const uint32_t rec = dsmem_addr(
-            smem_u32(smem) + (slot * per + in_owner) * S::kRecord,
-            static_cast<uint32_t>(active ? owner : crank));
-        const bool send = owner != crank;
-#pragma unroll 1
-        for (int c = 0; c < DV / 32; ++c) {
-          float v[32];
-          load32(c, v);
-          if (send) {
+      for (int c = 0; c < DV / 32; ++c) {
+        uint32_t ov[32];
+        tmem_ld32(tO + c * 32, ov);
+        tmem_wait_ld();
+        uint32_t pk[16];
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-              dsmem_st_v4(rec + c * 128 + i * 16, v[4 * i], v[4 * i + 1], v[4 * i + 2],
-                          v[4 * i + 3]);
-          }
-        }
-        if (send) dsmem_st_v4(rec + DV * 4, m_run, l_run, 0.f, 0.f);
-      }
-      // phase 2: the records have arrived
-      cluster_arrive_release();
-      cluster_wait_acquire();
-      if (have_o) {
-        const bool mine = owner == crank;
-        const uint8_t* rec = smem + (mine ? in_owner : 0) * S::kRecord;
-        const int step = per * S::kRecord;
-        float m_all = m_run;
-        for (int s = 0; s < n_split - 1; ++s)
-          m_all = fmaxf(m_all, *reinterpret_cast<const float*>(rec + s * step + DV * 4));
-        const float w_own = ex2_approx(m_run - m_all);
-        float l_all = l_run * w_own;
-        for (int s = 0; s < n_split - 1; ++s) {
-          const float2 ml = *reinterpret_cast<const float2*>(rec + s * step + DV * 4);
-          l_all = fmaf(ml.y, ex2_approx(ml.x - m_all), l_all);
-        }
-        const float inv_l = 1.f / l_all;
-#pragma unroll 1
-        for (int c = 0; c < DV / 32; ++c) {
-          float v[32];
-          load32(c, v);
+        for (int i = 0; i < 16; ++i)
+          pk[i] = pack_bf16x2(__uint_as_float(ov[2 * i]) * inv_l,
+                              __uint_as_float(ov[2 * i + 1]) * inv_l);
+        if (row_ok) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) v[i] *= w_own;
-          for (int s = 0; s < n_split - 1; ++s) {
-            const float w = ex2_approx(
-                *reinterpret_cast<const float*>(rec + s * step + DV * 4) - m_all);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const float4 x =
-                  *reinterpret_cast<const float4*>(rec + s * step + c * 128 + i * 16);
-              v[4 * i] = fmaf(x.x, w, v[4 * i]);
-              v[4 * i + 1] = fmaf(x.y, w, v[4 * i + 1]);
-              v[4 * i + 2] = fmaf(x.z, w, v[4 * i + 2]);
-              v[4 * i + 3] = fmaf(x.w, w, v[4 * i + 3]);
-            }
-          }
-          if (mine && row_ok) store32(c, v, inv_l);
+          for (int i = 0; i < 4; ++i)
+            dst[c * 4 + i] =
+                make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
         }
       }
     }

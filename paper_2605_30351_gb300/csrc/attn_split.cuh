@@ -1,0 +1,137 @@
+// Combination of a row tile whose key blocks were split over the CTAs of a
+// cluster: every CTA holds, per row, an unnormalised output O in TMEM and the
+// running maximum m and sum l of its own blocks. Each CTA owns an equal share
+// of the rows and forms for them
+//     O = sum_s 2^(m_s - m) O_s / sum_s 2^(m_s - m) l_s,   m = max_s m_s.
+// Every warp stages its rows in shared memory and sends each owner its share
+// by bulk copies between the CTAs' shared memories; all row threads then
+// combine, n threads per owned row. (Per-thread remote stores, one thread per
+// owned row and releasing barriers took ~8 us at n = 8, d_c = 192; this ~4.)
+//
+// Two cluster barrier phases go with it, which every thread of the cluster
+// passes. A: the CTA's receive area is free and its mbarrier initialised; the
+// caller's threads arrive (cluster_arrive_release) as early as that holds, and
+// combine_split waits. B: every owner has its records, so that no copy reads a
+// CTA that has left.
+#pragma once
+
+#include "ptx_sm103.cuh"
+
+namespace vmla {
+
+// What remains of phases A and B for warps that take no other part.
+__device__ __forceinline__ void combine_split_pass() {
+  cluster_wait_acquire();
+  cluster_arrive_relaxed();
+  cluster_wait_acquire();
+}
+
+// Bytes of one row's record: O (DV fp32), then m and l, padded so that eight
+// consecutive rows start in eight different bank groups.
+template <int DV>
+constexpr int kSplitRecord = DV * 4 + 16;
+
+// Called by all THREADS threads of the warps that hold rows, thread = row `lrow` of
+// the `rows` that the n CTAs of the cluster share (n in {2, 4, 8}; this CTA is
+// number `rank`).
+//  stage     this CTA's own records, rows * kSplitRecord bytes, free now
+//  recv      the receive area, rows / n * (n - 1) * kSplitRecord bytes at the
+//            same offset in every CTA
+//  bar       an mbarrier of count 1 at the same offset in every CTA, unused yet
+//  tO        TMEM address of the thread's O
+//  have_o    warp-uniform: false when this warp has no O (a wait gave up, or
+//            its row tile does not exist); nothing is stored for its share
+//  o, stride row 0 of the shared rows in the output, elements between rows
+//  valid     rows of the output there are
+template <int DV, int THREADS>
+__device__ __forceinline__ void combine_split(uint8_t* stage, uint8_t* recv, uint64_t* bar,
+                                              uint32_t tO, int rank, int n, int rows, int lrow,
+                                              bool have_o, float m_run, float l_run,
+                                              __nv_bfloat16* o, size_t stride, int valid,
+                                              const WaitCtx& wc) {
+  constexpr int kRec = kSplitRecord<DV>;
+  const int per = rows / n;  // rows each CTA owns
+  if (have_o) {
+    float4* rec = reinterpret_cast<float4*>(stage + lrow * kRec);
+#pragma unroll 1
+    for (int c = 0; c < DV / 32; ++c) {
+      uint32_t v[32];
+      tmem_ld32(tO + c * 32, v);
+      tmem_wait_ld();
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        rec[c * 8 + i] = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
+                                     __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
+    }
+    rec[DV / 4] = make_float4(m_run, l_run, 0.f, 0.f);
+  }
+  fence_proxy_async_smem();  // the staged rows reach the bulk copies
+  cluster_wait_acquire();    // phase A
+  if (lrow == 0) mbar_arrive_expect_tx(bar, (n - 1) * per * kRec);
+  __syncwarp();
+  // this warp's rows, in pieces that have one owner each
+  const int w0 = lrow & ~31;
+  if ((lrow & 31) == 0 && w0 < rows) {
+    const int piece = per < 32 ? per : 32;
+    for (int q = w0; q < w0 + 32; q += piece) {
+      const int d = q / per;
+      if (d == rank) continue;
+      const int slot = rank < d ? rank : rank - 1;  // this sender among d's n - 1
+      bulk_copy_to_peer(dsmem_addr(smem_u32(recv + (slot * per + q - d * per) * kRec), d),
+                        stage + q * kRec, piece * kRec, dsmem_addr(smem_u32(bar), d));
+    }
+  }
+  const bool got = mbar_wait(bar, 0, wc);
+  cluster_arrive_relaxed();  // phase B
+  asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");  // own records of all warps
+  const int row = rank * per + lrow / n;  // n threads per owned row, DV / n columns each
+  if (got && lrow < rows && row < valid && !*wc.abort_flag) {
+    const uint8_t* own = stage + row * kRec;
+    const uint8_t* other = recv + (lrow / n) * kRec;
+    const float2 ml0 = *reinterpret_cast<const float2*>(own + DV * 4);
+    float2 ml[7];
+    float m_all = ml0.x;
+#pragma unroll
+    for (int s = 0; s < 7; ++s)
+      if (s < n - 1) {
+        ml[s] = *reinterpret_cast<const float2*>(other + s * per * kRec + DV * 4);
+        m_all = fmaxf(m_all, ml[s].x);
+      }
+    const float w0 = ex2_approx(ml0.x - m_all);
+    float l_all = ml0.y * w0;
+    float w[7];
+#pragma unroll
+    for (int s = 0; s < 7; ++s)
+      if (s < n - 1) {
+        w[s] = ex2_approx(ml[s].x - m_all);
+        l_all = fmaf(ml[s].y, w[s], l_all);
+      }
+    const float inv_l = 1.f / l_all;
+    const int col0 = lrow % n * (DV / n);
+    uint4* out = reinterpret_cast<uint4*>(o + row * stride);
+    for (int c = col0; c < col0 + DV / n; c += 8) {
+      float v[8];
+      const float4 a = *reinterpret_cast<const float4*>(own + c * 4);
+      const float4 b = *reinterpret_cast<const float4*>(own + c * 4 + 16);
+      v[0] = a.x * w0, v[1] = a.y * w0, v[2] = a.z * w0, v[3] = a.w * w0;
+      v[4] = b.x * w0, v[5] = b.y * w0, v[6] = b.z * w0, v[7] = b.w * w0;
+#pragma unroll
+      for (int s = 0; s < 7; ++s)
+        if (s < n - 1) {
+          const float4 x = *reinterpret_cast<const float4*>(other + s * per * kRec + c * 4);
+          const float4 y = *reinterpret_cast<const float4*>(other + s * per * kRec + c * 4 + 16);
+          v[0] = fmaf(x.x, w[s], v[0]), v[1] = fmaf(x.y, w[s], v[1]);
+          v[2] = fmaf(x.z, w[s], v[2]), v[3] = fmaf(x.w, w[s], v[3]);
+          v[4] = fmaf(y.x, w[s], v[4]), v[5] = fmaf(y.y, w[s], v[5]);
+          v[6] = fmaf(y.z, w[s], v[6]), v[7] = fmaf(y.w, w[s], v[7]);
+        }
+      out[c / 8] = make_uint4(pack_bf16x2(v[0] * inv_l, v[1] * inv_l),
+                              pack_bf16x2(v[2] * inv_l, v[3] * inv_l),
+                              pack_bf16x2(v[4] * inv_l, v[5] * inv_l),
+                              pack_bf16x2(v[6] * inv_l, v[7] * inv_l));
+    }
+  }
+  cluster_wait_acquire();  // phase B
+}
+
+}  // namespace vmla

@@ -31,6 +31,8 @@
 //              rescales O in TMEM only when its running max grows by more
 //              than 2^8, and finally writes O / l as bf16.
 // TMEM columns: S [0,128) P [128,192) O [192,192+d_c) Q [192+d_c, +(d_c+d_r)/2).
+// A grid that would leave SMs idle runs the SPLIT form instead: the CTAs of a
+// cluster take one row tile and share out its key blocks (attn_split.cuh).
 // What bounds it (Wan shape): the tensor pipe at d_c = 192 (92 % active; the
 // GPU's power cap in long runs), a block's softmax (~1200 cycles beside 1152 of
 // MMAs) at d_c = 128. Issuing from converged warps and settling the rescale
@@ -39,6 +41,7 @@
 // so the cache is never expanded into per-head keys or values.
 #include <cmath>
 
+#include "attn_split.cuh"
 #include "internal.h"
 #include "ptx_sm103.cuh"
 
@@ -75,7 +78,10 @@ struct AttnShape {
   static_assert(kTmemQ + DK / 2 <= 512, "S, P, O and Q must fit in 512 TMEM columns");
   static_assert(kStages >= 2, "at least two key stages must fit in shared memory");
   static_assert(kBM * DC * 2 <= kTileBytes, "q_c passes through one key stage");
-  static_assert(kTileBytes % 1024 == 0 && kKrOff % 1024 == 0, "swizzle-atom alignment");
+  // the split form's records: this CTA's rows, then the others' of its share
+  static constexpr int kRecv = kBM * kSplitRecord<DC>;
+  static_assert(kRecv + kBM / 8 * 7 * kSplitRecord<DC> <= kStages * kTileBytes,
+                "the records of a split tile fit in the key stages");
 };
 
 struct AttnKParams {
@@ -87,17 +93,18 @@ struct AttnKParams {
   int rows, heads, n_valid, rope_len, pairs_t, pairs_h;
   float scale_log2;
   int* status;
+  int cl;  // SPLIT: CTAs per row tile
 };
 
-template <int DC, int DR, int CL>
+template <int DC, int DR, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
     mla_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_qc,
                        const __grid_constant__ CUtensorMap tm_c,
                        const __grid_constant__ CUtensorMap tm_kr, const AttnKParams p) {
   using S = AttnShape<DC, DR>;
   constexpr int NST = S::kStages;
-  constexpr uint16_t kPair = static_cast<uint16_t>((1u << CL) - 1u);  // every CTA of the cluster
-  static_assert(CL == 1 || CL == 2, "clusters of one or two CTAs");
+  constexpr int CL = SPLIT ? 1 : 2;  // CTAs that share each key tile by multicast
+  constexpr uint16_t kPair = 3;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem_1024(smem_raw);
   uint8_t* sKV = smem;
@@ -112,14 +119,23 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* p_full = s_free + 1;
   uint64_t* pv_done = p_full + 1;
   uint64_t* mma_drain = pv_done + 1;  // [2]: one per issuing thread
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_drain + 2);
+  uint64_t* split_bar = mma_drain + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(split_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.y;
-  const int row0 = blockIdx.x * kBM;
-  const int nblk = (p.n_valid + kBN - 1) / kBN;
+  // SPLIT: the p.cl CTAs of a cluster take the same row tile and a share of
+  // its key blocks each, [jb0, jb0 + nblk)
+  const int crank = SPLIT && p.cl == 1 ? 0 : static_cast<int>(cluster_ctarank());
+  const int row0 = (SPLIT ? blockIdx.x / p.cl : blockIdx.x) * kBM;
+  int jb0 = 0, nblk = (p.n_valid + kBN - 1) / kBN;
+  if constexpr (SPLIT) {
+    const int all = nblk;
+    jb0 = static_cast<int>(static_cast<long long>(all) * crank / p.cl);
+    nblk = static_cast<int>(static_cast<long long>(all) * (crank + 1) / p.cl) - jb0;
+  }
   const WaitCtx wc{abort_flag, p.status};
 
   if (threadIdx.x == 0) {
@@ -135,6 +151,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(pv_done, 1);
     mbar_init(&mma_drain[0], 1);
     mbar_init(&mma_drain[1], 1);
+    mbar_init(split_bar, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -149,7 +166,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   // the peer's barriers must be initialised before any multicast lands
   if constexpr (CL > 1) cluster_sync();
   grid_dep_sync();
-  const int crank = CL > 1 ? static_cast<int>(cluster_ctarank()) : 0;
+  // phase A of the combination; the softmax warps arrive once the last MMA is
+  // done with the key stages, where the records go
+  if (SPLIT && p.cl > 1 && (warp < 2 || warp == 6)) cluster_arrive_release();
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
@@ -164,16 +183,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       int issued = 0;
       for (int j = 0; j < nblk; ++j) {
         const int st = j % NST;
-        // releases of this stage so far that its next fill waits for: one per
-        // earlier fill, and on the last stage one more, for Q (both CTAs')
+        // releases of this stage that its next fill waits for: one per earlier
+        // fill, and on the last stage one more, for Q (a pair: both CTAs')
         const int freed = j / NST + (st == NST - 1 ? 1 : 0);
         if (freed > 0 && !mbar_wait(&kv_empty[st], (freed - 1) & 1, wc)) break;
         uint8_t* kv = sKV + st * S::kTileBytes;
         mbar_arrive_expect_tx(&kv_full[st], S::kTileBytes);
         if constexpr (CL == 1) {
           for (int cb = 0; cb < DC / 64; ++cb)
-            tma_load_3d(kv + cb * S::kCBox, &tm_c, &kv_full[st], cb * 64, j * kBN, b);
-          tma_load_3d(kv + S::kKrOff, &tm_kr, &kv_full[st], 0, j * kBN, b);
+            tma_load_3d(kv + cb * S::kCBox, &tm_c, &kv_full[st], cb * 64, (jb0 + j) * kBN, b);
+          tma_load_3d(kv + S::kKrOff, &tm_kr, &kv_full[st], 0, (jb0 + j) * kBN, b);
         } else {
           // each CTA fetches every other box once and multicasts it to both
           for (int bx = crank; bx <= DC / 64; bx += CL) {
@@ -197,12 +216,17 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     __syncwarp();
+    if (SPLIT && p.cl > 1) combine_split_pass();
   } else if (warp == 1) {
     // ------------------------------------------------------ QK^T issuer
     // the whole warp walks the loop; one lane issues (see elect_one)
     bool ok = mbar_wait_warp(q_ready, 0, wc);
     // Q has left the last key stage: both CTAs' copies may fill it
-    if (lane < CL) mbar_arrive_peer(dsmem_addr(smem_u32(&kv_empty[NST - 1]), lane));
+    if constexpr (SPLIT) {
+      if (lane == 0) mbar_arrive(&kv_empty[NST - 1]);
+    } else if (lane < CL) {
+      mbar_arrive_peer(dsmem_addr(smem_u32(&kv_empty[NST - 1]), lane));
+    }
     __syncwarp();
     const uint64_t kd = sdesc(smem_u32(sKV), 16, 1024, kSw128);
     const uint64_t krd = sdesc(smem_u32(sKV) + S::kKrOff, 16, S::kKrSbo, S::kKrSw);
@@ -235,6 +259,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       mbar_wait_drain(&mma_drain[0], 0, p.status);
     }
+    if (SPLIT && p.cl > 1) combine_split_pass();
   } else if (warp == 6) {
     // --------------------------------------------------------- PV issuer
     bool ok = true;
@@ -264,6 +289,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       mbar_wait_drain(&mma_drain[1], 0, p.status);
     }
+    if (SPLIT && p.cl > 1) combine_split_pass();
   } else {
     // ------------------------------------------------ softmax (warps 2..5)
     const int quarter = warp & 3;  // TMEM lane quarter this warp may access
@@ -352,7 +378,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       float sv[kBN];
 #pragma unroll
       for (int c = 0; c < kBN; ++c) sv[c] = __uint_as_float(sr[c]);
-      const int valid = p.n_valid - j * kBN;
+      const int valid = p.n_valid - (jb0 + j) * kBN;
       if (valid < kBN) {
 #pragma unroll
         for (int c = 0; c < kBN; ++c)
@@ -445,42 +471,50 @@ __global__ void __launch_bounds__(kThreads, 1)
       l_run += ((l8[0] + l8[1]) + (l8[2] + l8[3])) + ((l8[4] + l8[5]) + (l8[6] + l8[7]));
     }
 
-    // O / l as bf16: each thread stages its row densely in the key stages
-    // (free once the last PV is done: every key tile, the peer's multicast
-    // halves included, has landed and been read), and each warp's rows, which
-    // are consecutive rows of o, leave shared memory by one bulk copy.
     bool have_o = ok && mbar_wait(pv_done, (nblk - 1) & 1, wc);
     have_o = __all_sync(0xffffffffu, have_o) && !*abort_flag;
-    uint8_t* srow = sKV + r * DC * 2;
-    if (have_o) {
-      tc_fence_after();
-      const float inv_l = 1.f / l_run;
+    if (!SPLIT || p.cl == 1) {
+      // O / l as bf16: each thread stages its row densely in the key stages
+      // (free once the last PV is done: every key tile, the peer's multicast
+      // halves included, has landed and been read), and each warp's rows, which
+      // are consecutive rows of o, leave shared memory by one bulk copy.
+      uint8_t* srow = sKV + r * DC * 2;
+      if (have_o) {
+        tc_fence_after();
+        const float inv_l = 1.f / l_run;
 #pragma unroll 1
-      for (int sg = 0; sg < DC / 64; ++sg) {
-        uint32_t va[32], vb[32];
-        tmem_ld32(tmem + t_lane + S::kTmemO + sg * 64, va);
-        tmem_ld32(tmem + t_lane + S::kTmemO + sg * 64 + 32, vb);
-        tmem_wait_ld();
-        uint32_t pk[32];
+        for (int sg = 0; sg < DC / 64; ++sg) {
+          uint32_t va[32], vb[32];
+          tmem_ld32(tmem + t_lane + S::kTmemO + sg * 64, va);
+          tmem_ld32(tmem + t_lane + S::kTmemO + sg * 64 + 32, vb);
+          tmem_wait_ld();
+          uint32_t pk[32];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const uint32_t* v = i < 16 ? va : vb;
-          const int j = i & 15;
-          pk[i] = pack_bf16x2(__uint_as_float(v[2 * j]) * inv_l,
-                              __uint_as_float(v[2 * j + 1]) * inv_l);
+          for (int i = 0; i < 32; ++i) {
+            const uint32_t* v = i < 16 ? va : vb;
+            const int j = i & 15;
+            pk[i] = pack_bf16x2(__uint_as_float(v[2 * j]) * inv_l,
+                                __uint_as_float(v[2 * j + 1]) * inv_l);
+          }
+          stage_row<8>(srow + sg * 128, pk, r & 7);
         }
-        stage_row<8>(srow + sg * 128, pk, r & 7);
+        fence_proxy_async_smem();
+        __syncwarp();
+        // the warp's rows below p.rows; none past the end, where the grid is
+        // padded to whole clusters (an odd number of row tiles)
+        const int valid = min(32, p.rows - (row0 + quarter * 32));
+        if (lane == 0 && valid > 0) {
+          bulk_store(p.o + (static_cast<size_t>(b) * p.rows + grow) * DC, srow, valid * DC * 2);
+          bulk_commit();
+          bulk_wait_read_all();  // the staged rows must outlive the copy's reads
+        }
       }
-      fence_proxy_async_smem();
-      __syncwarp();
-      // the warp's rows below p.rows; none past the end, where the grid is
-      // padded to whole clusters (an odd number of row tiles)
-      const int valid = min(32, p.rows - (row0 + quarter * 32));
-      if (lane == 0 && valid > 0) {
-        bulk_store(p.o + (static_cast<size_t>(b) * p.rows + grow) * DC, srow, valid * DC * 2);
-        bulk_commit();
-        bulk_wait_read_all();  // the staged rows must outlive the copy's reads
-      }
+    } else {
+      cluster_arrive_release();  // phase A
+      combine_split<DC, kBM>(sKV, sKV + S::kRecv, split_bar, tmem + t_lane + S::kTmemO, crank, p.cl, kBM, r,
+                             have_o, m_run, l_run,
+                             p.o + (static_cast<size_t>(b) * p.rows + row0) * DC, DC,
+                             p.rows - row0, wc);
     }
   }
 
@@ -494,9 +528,76 @@ __global__ void __launch_bounds__(kThreads, 1)
   if constexpr (CL > 1) cluster_sync();
 }
 
-template <int DC, int DR, int CL>
+template <int DC, int DR>
+cudaLaunchConfig_t attn_config(int ctas, int batch, int cl, cudaStream_t stream,
+                               cudaLaunchAttribute (&attr)[2]) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas, batch, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = AttnShape<DC, DR>::kSmemBytes;
+  cfg.stream = stream;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cl;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see grid_dep_sync
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cfg;
+}
+
+// Clusters of 1, 2, 4 and 8 CTAs of the split form that are resident at once.
+struct Resident {
+  int n[4];
+};
+template <int DC, int DR>
+Resident query_resident() {
+  auto kern = mla_attn_tc_kernel<DC, DR, true>;
+  Resident r = {};
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           AttnShape<DC, DR>::kSmemBytes) != cudaSuccess)
+    cudaGetLastError();
+  for (int i = 0; i < 4; ++i) {
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = attn_config<DC, DR>(1 << i, 1, 1 << i, nullptr, attr);
+    if (cudaOccupancyMaxActiveClusters(&r.n[i], kern, &cfg) != cudaSuccess) {
+      cudaGetLastError();  // a failed query only disables that cluster size
+      r.n[i] = 0;
+    }
+  }
+  return r;
+}
+
+// CTAs per row tile (a cluster that shares out the tile's key blocks), or 0
+// for pairs of whole tiles with multicast key tiles: the shortest estimate in
+// key blocks of ~0.82 us at d_c = 192, a CTA's start and end counted as
+// kFixed, a split tile's combination as kCombine. Measured (d_c = 192, pairs /
+// twos / fours / eights): 6 tiles x 11 blocks 15.7 / 14.1 / 12.1 / 12.8 us, 24 x 42
+// 42.2 / 27.0 / 20.1 / 32.2, 72 x 42 42.7 / 28.1 / 40.1 / 79.6, 46 x 80 75 / 45 /
+// 54 / 75, 110 x 64 63 / 75 / 92 / 142.
+int pick_split(int tiles, int batch, int nblk, const Resident& res) {
+  constexpr long long kFixed = 5, kCombine = 3;
+  const long long n = static_cast<long long>(tiles) * batch;
+  const long long pairs = static_cast<long long>((tiles + 1) / 2) * batch;
+  int best = 0;
+  long long best_t = res.n[1] > 0 ? (pairs + res.n[1] - 1) / res.n[1] * (nblk + kFixed)
+                                  : 1ll << 62;
+  for (int i = 0; i < 4; ++i) {
+    const int cl = 1 << i;
+    if (res.n[i] < 1 || nblk < cl) continue;
+    const long long t = (n + res.n[i] - 1) / res.n[i] *
+                        ((nblk + cl - 1) / cl + kFixed + (cl > 1 ? kCombine : 0));
+    if (t < best_t) {
+      best_t = t;
+      best = cl;
+    }
+  }
+  return best;
+}
+
+template <int DC, int DR>
 int launch_tc(const AttnArgs& a) {
-  using S = AttnShape<DC, DR>;
   CUtensorMap tm_qc, tm_c, tm_kr;
   const unsigned long long rows = a.rows, slots = a.slots;
   if (!encode_map_3d_bf16(&tm_qc, a.q_c, DC, rows, a.batch, DC * 2ull, rows * DC * 2ull, 64, kBM,
@@ -507,9 +608,17 @@ int launch_tc(const AttnArgs& a) {
                           kBN,
                           DR == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B))
     return MLA_ERR_CUDA;
-  auto kern = mla_attn_tc_kernel<DC, DR, CL>;
-  cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmemBytes);
+  static const Resident res = query_resident<DC, DR>();
+  const int tiles = (a.rows + kBM - 1) / kBM;
+  const int cl = pick_split(tiles, a.batch, (a.n_valid + kBN - 1) / kBN, res);
+  // pairs stay within a batch element
+  cudaLaunchAttribute attr[2];
+  const cudaLaunchConfig_t cfg =
+      cl > 0 ? attn_config<DC, DR>(tiles * cl, a.batch, cl, a.stream, attr)
+             : attn_config<DC, DR>((tiles + 1) / 2 * 2, a.batch, 2, a.stream, attr);
+  auto kern = cl > 0 ? mla_attn_tc_kernel<DC, DR, true> : mla_attn_tc_kernel<DC, DR, false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(cfg.dynamicSmemBytes));
   if (e != cudaSuccess) {
     set_last_cuda_error(e);
     return MLA_ERR_CUDA;
@@ -528,21 +637,7 @@ int launch_tc(const AttnArgs& a) {
   kp.pairs_h = a.pairs_h;
   kp.scale_log2 = a.scale_log2;
   kp.status = a.status;
-  const int tiles = (a.rows + kBM - 1) / kBM;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((tiles + CL - 1) / CL * CL, a.batch, 1);  // pairs stay within a batch row
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = S::kSmemBytes;
-  cfg.stream = a.stream;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CL;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see grid_dep_sync
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  kp.cl = cl;
   e = cudaLaunchKernelEx(&cfg, kern, tm_qc, tm_c, tm_kr, kp);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -552,21 +647,14 @@ int launch_tc(const AttnArgs& a) {
   return MLA_OK;
 }
 
-// Pairs of CTAs share every key tile through TMA multicast; a single row tile
-// per batch element runs alone.
-template <int DC, int DR>
-int launch_tc_pick(const AttnArgs& a) {
-  return (a.rows + kBM - 1) / kBM >= 2 ? launch_tc<DC, DR, 2>(a) : launch_tc<DC, DR, 1>(a);
-}
-
 }  // namespace
 
 int launch_attention_tc(const AttnArgs& a) {
   if (a.d_r != 32 && a.d_r != 64) return MLA_ERR_UNSUPPORTED;
   switch (a.d_c) {
     case 64: return launch_attention_dual_tc(a);  // two row tiles per CTA
-    case 128: return a.d_r == 32 ? launch_tc_pick<128, 32>(a) : launch_tc_pick<128, 64>(a);
-    case 192: return a.d_r == 32 ? launch_tc_pick<192, 32>(a) : launch_tc_pick<192, 64>(a);
+    case 128: return a.d_r == 32 ? launch_tc<128, 32>(a) : launch_tc<128, 64>(a);
+    case 192: return a.d_r == 32 ? launch_tc<192, 32>(a) : launch_tc<192, 64>(a);
     case 256:
     case 512: return launch_attention_wide_tc(a);  // paired-SM MMAs
     default: return MLA_ERR_UNSUPPORTED;

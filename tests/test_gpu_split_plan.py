@@ -1,6 +1,6 @@
-"""Attention with two row tiles per CTA (value width 64) where its launch plan
-changes: one or two row tiles, a single key block, blocks split over clusters
-of two, four and eight CTAs, whole and split tiles in one launch."""
+"""Attention where its launch plan changes: one or two row tiles, a single key
+block, blocks split over clusters of two, four and eight CTAs, whole and split
+tiles in one launch; two row tiles per CTA (d_c = 64) and one (128, 192)."""
 
 import numpy as np
 import pytest
@@ -26,6 +26,7 @@ def _gpu():
     assert V.mla_device_status(clear=True) == V.MLA_OK
 
 
+@pytest.mark.parametrize("d_c", [64, 128, 192])
 @pytest.mark.parametrize("grid,frames,nq,batch,d_r", [
     ((1, 1), 1, 1, 1, 32),      # 12 rows, one key: one row tile, one block, no cluster
     ((8, 16), 1, 11, 1, 64),    # 132 rows: the second row tile has four; one full block
@@ -34,16 +35,16 @@ def _gpu():
     ((10, 13), 13, 21, 2, 64),  # 1690 keys: fourteen blocks over a cluster of eight
     ((10, 13), 12, 150, 3, 32), # 1800 rows x 3: eight tiles per element
 ])
-def test_split_key_blocks(grid, frames, nq, batch, d_r):
-    w = small(d_c=64, d_r=d_r, rope_pairs=(6, 5, 5) if d_r == 32 else (12, 10, 10),
+def test_split_key_blocks(d_c, grid, frames, nq, batch, d_r):
+    w = small(d_c=d_c, d_r=d_r, rope_pairs=(6, 5, 5) if d_r == 32 else (12, 10, 10),
               rope_axis_dims=(44, 42, 42) if d_r == 32 else (64, 64, 64), grid_h=grid[0],
               grid_w=grid[1], window_frames=frames, batch=batch)
     cache, c, k = upload_cache(w, 21, frames)
-    q_c, q_r = synth.draw_queries(w, nq, 22, qc_std=2.0)  # scores that differ between splits
+    q_c, q_r = synth.draw_queries(w, nq, 22, qc_std=16.0 / d_c ** 0.5)  # scores that differ between splits
     q_pos = synth.grid_positions(w, 0, frames)[:, -nq:].contiguous()
     if q_pos.shape[1] < nq:
         q_pos = q_pos[:, :1].repeat(1, nq, 1).contiguous()
-    o = torch.empty(batch, nq, w.heads, 64, dtype=torch.bfloat16, device="cuda")
+    o = torch.empty(batch, nq, w.heads, d_c, dtype=torch.bfloat16, device="cuda")
     V.mla_attention_forward(cache, q_c.cuda(), q_r.cuda(), q_pos.cuda(), o)
     torch.cuda.synchronize()
     ref = oracle_latent(w, q_c, q_r, q_pos, c, k, cache.n_valid())
