@@ -1,0 +1,75 @@
+"""The layer GEMMs in every tile width their launchers pick by the number of
+row tiles, with ragged rows, widths that end inside a tile, statistics groups
+that are not whole and an odd number of K blocks, against float64."""
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2605_30351_gb300 import synth
+from paper_2605_30351_gb300 import videomla as V
+
+from test_gpu_parity import assert_close, f64, small
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    V.load()
+    V.mla_device_status(clear=True)
+    yield
+    assert V.mla_device_status(clear=True) == V.MLA_OK
+
+
+@pytest.mark.parametrize("nq,d_q,d_c,d_r,hidden", [
+    (1, 64, 64, 32, 64),        # one row, one K block; one 64-wide tile of a group of three
+    (130, 320, 64, 32, 1472),   # five 64-wide tiles: the second group is not whole
+    (384, 768, 192, 32, 1536),  # 64-wide tiles in both GEMMs (3 row tiles)
+    (500, 768, 128, 64, 1536),  # 128-wide tiles in the second GEMM
+    (1500, 704, 64, 64, 1472),  # 64-wide first GEMM at its last row tile, 11 K blocks
+    (2000, 768, 64, 32, 1536),  # 192-wide first GEMM, persistent second
+])
+def test_query_prologue_forms(nq, d_q, d_c, d_r, hidden):
+    w = small(d_c=d_c, d_r=d_r, d_q=d_q, hidden=hidden,
+              rope_pairs=(6, 5, 5) if d_r == 32 else (12, 10, 10),
+              rope_axis_dims=(44, 42, 42) if d_r == 32 else (64, 64, 64))
+    rng = np.random.default_rng(51)
+    H, n = w.heads, w.heads * (d_c + d_r)
+    x = synth.bf16(rng.standard_normal((1, nq, hidden)))
+    w_dq = synth.bf16(rng.standard_normal((d_q, hidden)) * hidden ** -0.5)
+    w_qcat = synth.bf16(rng.standard_normal((n, d_q)) * d_q ** -0.5)
+    cfg = V.make_config(w)
+    ws = torch.empty(V.mla_query_workspace_bytes(cfg, nq), dtype=torch.uint8, device="cuda")
+    q_c = torch.empty(1, nq, H, d_c, dtype=torch.bfloat16, device="cuda")
+    q_r = torch.empty(1, nq, H, d_r, dtype=torch.bfloat16, device="cuda")
+    V.mla_query_prologue(cfg, x.cuda(), w_dq.cuda(), w_qcat.cuda(), ws, q_c, q_r)
+    torch.cuda.synchronize()
+    ct = f64(x[0]) @ f64(w_dq).T
+    q = (ct / np.sqrt(np.mean(ct * ct, axis=1, keepdims=True) + w.rms_eps)) @ f64(w_qcat).T
+    # unit-variance outputs: one in [4, 8) is off by up to 2^-6 from its own rounding to
+    # bf16 alone, and the rounded c~ adds ~0.003
+    assert_close(f64(q_c[0]).reshape(nq, -1), q[:, :H * d_c], max_abs=4e-2, what="q_c")
+    assert_close(f64(q_r[0]).reshape(nq, -1), q[:, H * d_c:], max_abs=4e-2, what="q_r")
+
+
+@pytest.mark.parametrize("nq,d_c,hidden", [
+    (1, 64, 64),        # one 64-wide tile
+    (700, 192, 1536),   # 64-wide, six row tiles
+    (1500, 64, 1536),   # 128-wide, twelve row tiles
+    (2400, 64, 1472),   # 192-wide, its last tile ragged; 19 row tiles
+    (3000, 128, 1536),  # 256-wide, 24 row tiles
+    (4000, 64, 1536),   # 384-wide
+])
+def test_output_projection_forms(nq, d_c, hidden):
+    w = small(d_c=d_c, hidden=hidden)
+    rng = np.random.default_rng(52)
+    K = w.heads * d_c
+    o = synth.bf16(rng.standard_normal((1, nq, w.heads, d_c)))
+    w_b = synth.bf16(rng.standard_normal((hidden, K)) * K ** -0.5)
+    y = torch.empty(1, nq, hidden, dtype=torch.bfloat16, device="cuda")
+    V.mla_output_projection(V.make_config(w), o.cuda(), w_b.cuda(), y)
+    torch.cuda.synchronize()
+    assert_close(f64(y[0]), f64(o[0]).reshape(nq, K) @ f64(w_b).T, max_abs=4e-2, what="y")
