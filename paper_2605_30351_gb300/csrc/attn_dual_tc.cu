@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       asm volatile("bar.sync 2, 256;" ::: "memory");
       cluster_arrive_release();  // phase A
       combine_split<DV, 256>(smem, smem + nt * kBM * kSplitRecord<DV>, split_bar, tO, crank,
-                             n_split, nt * kBM, t * kBM + r, have_o, m_run, l_run,
+                             n_split, 0, 1, nt * kBM, t * kBM + r, have_o, m_run, l_run,
                              p.o + orow0 * DV, stride, p.rows - row0, wc);
     } else if (have_o) {
       uint4* dst = reinterpret_cast<uint4*>(

@@ -32,8 +32,8 @@ template <int DV>
 constexpr int kSplitRecord = DV * 4 + 16;
 
 // Called by all THREADS threads of the warps that hold rows, thread = row `lrow` of
-// the `rows` that the n CTAs of the cluster share (n in {2, 4, 8}; this CTA is
-// number `rank`).
+// the `rows` that n CTAs of the cluster share (n in {2, 4, 8}; this CTA is
+// number `rank` of them, number d has cluster rank peer0 + d * peer_step).
 //  stage     this CTA's own records, rows * kSplitRecord bytes, free now
 //  recv      the receive area, rows / n * (n - 1) * kSplitRecord bytes at the
 //            same offset in every CTA
@@ -45,8 +45,9 @@ constexpr int kSplitRecord = DV * 4 + 16;
 //  valid     rows of the output there are
 template <int DV, int THREADS>
 __device__ __forceinline__ void combine_split(uint8_t* stage, uint8_t* recv, uint64_t* bar,
-                                              uint32_t tO, int rank, int n, int rows, int lrow,
-                                              bool have_o, float m_run, float l_run,
+                                              uint32_t tO, int rank, int n, int peer0,
+                                              int peer_step, int rows, int lrow, bool have_o,
+                                              float m_run, float l_run,
                                               __nv_bfloat16* o, size_t stride, int valid,
                                               const WaitCtx& wc) {
   constexpr int kRec = kSplitRecord<DV>;
@@ -77,8 +78,9 @@ __device__ __forceinline__ void combine_split(uint8_t* stage, uint8_t* recv, uin
       const int d = q / per;
       if (d == rank) continue;
       const int slot = rank < d ? rank : rank - 1;  // this sender among d's n - 1
-      bulk_copy_to_peer(dsmem_addr(smem_u32(recv + (slot * per + q - d * per) * kRec), d),
-                        stage + q * kRec, piece * kRec, dsmem_addr(smem_u32(bar), d));
+      const int peer = peer0 + d * peer_step;
+      bulk_copy_to_peer(dsmem_addr(smem_u32(recv + (slot * per + q - d * per) * kRec), peer),
+                        stage + q * kRec, piece * kRec, dsmem_addr(smem_u32(bar), peer));
     }
   }
   const bool got = mbar_wait(bar, 0, wc);

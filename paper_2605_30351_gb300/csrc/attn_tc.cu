@@ -511,8 +511,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     } else {
       cluster_arrive_release();  // phase A
-      combine_split<DC, kBM>(sKV, sKV + S::kRecv, split_bar, tmem + t_lane + S::kTmemO, crank, p.cl, kBM, r,
-                             have_o, m_run, l_run,
+      combine_split<DC, kBM>(sKV, sKV + S::kRecv, split_bar, tmem + t_lane + S::kTmemO, crank,
+                             p.cl, 0, 1, kBM, r, have_o, m_run, l_run,
                              p.o + (static_cast<size_t>(b) * p.rows + row0) * DC, DC,
                              p.rows - row0, wc);
     }

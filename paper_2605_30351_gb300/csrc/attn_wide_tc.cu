@@ -16,6 +16,8 @@
 // same box: (256, 32) 1166 -> 938 us, (256, 64) 1325 -> 992 us, (512, 32) 4250
 // -> 3262 us, (512, 64) 4360 -> 3360 us (1190 useful, 1800 issued TFLOP/s, the
 // tensor pipe 89 % busy). In long runs both widths sit at the GPU's power cap.
+// A grid that leaves SMs idle takes clusters of four: two pairs share out the
+// row tiles' key blocks and combine their outputs (pick_wide_split).
 // d_c = 512: O of 512 fp32 columns would fill TMEM, so a row tile's output is
 // split over two clusters of 256 columns each (DV); both compute the full
 // score (3200 issued FLOP for 2112 useful per row-key pair at d_r = 32).
@@ -27,6 +29,7 @@
 // TMEM: S [0,128) P [128,192) O [192,448) Q [448,512).
 #include <cmath>
 
+#include "attn_split.cuh"
 #include "internal.h"
 #include "ptx_sm103.cuh"
 
@@ -67,6 +70,9 @@ struct WideShape {
   static_assert(kTmemQ + 32 + DR / 2 <= 512, "TMEM budget");
   static_assert(kKStages >= 5, "K boxes in flight");
   static_assert(kBM * DV * 2 <= kVStages * kVTile, "output rows staged in the V ring");
+  static_assert((kBM + kBM / 2) * kSplitRecord<DV> <=
+                    kQBytes + kVStages * kVTile + kKStages * kKBox,
+                "the records of a split tile fit where the operands were");
   static_assert(2 * (kKStages + kVStages) + 8 <= kBarBytes / 8 - 1, "barriers, slot, abort flag");
 };
 
@@ -79,6 +85,7 @@ struct WideKParams {
   int rows, heads, n_valid, rope_len, pairs_t, pairs_h;
   float scale_log2;
   int* status;
+  int n_split;  // pairs that share out a row tile's key blocks (1, or 2 in a cluster of four)
 };
 
 template <int DC, int DR>
@@ -106,7 +113,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* p_full = bars + 4;
   uint64_t* pv_done = bars + 5;
   uint64_t* mma_drain = bars + 6;
-  uint64_t* k_full = bars + 7;
+  uint64_t* split_bar = bars + 7;
+  uint64_t* k_full = bars + 8;
   uint64_t* k_empty = k_full + NK;
   uint64_t* v_full = k_empty + NK;
   uint64_t* v_empty = v_full + NV;
@@ -116,9 +124,16 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.y;
-  const int item = blockIdx.x / 2;  // cluster
+  const int item = blockIdx.x / (2 * p.n_split);  // cluster
   const int vpart = item % S::kSplit;
-  const int nblk = (p.n_valid + kBN - 1) / kBN;
+  // this pair of the cluster, its even CTA, and its share of the key blocks
+  const int rank = static_cast<int>(cluster_ctarank());
+  const int part = rank >> 1, even_rank = rank & ~1, crank = rank & 1;
+  const uint16_t pair_mask = static_cast<uint16_t>(3u << even_rank);
+  const int all_blk = (p.n_valid + kBN - 1) / kBN;
+  const int jb0 = static_cast<int>(static_cast<long long>(all_blk) * part / p.n_split);
+  const int nblk =
+      static_cast<int>(static_cast<long long>(all_blk) * (part + 1) / p.n_split) - jb0;
   const WaitCtx wc{abort_flag, p.status};
 
   if (threadIdx.x == 0) {
@@ -129,6 +144,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(p_full, 8);
     mbar_init(pv_done, 1);
     mbar_init(mma_drain, 1);
+    mbar_init(split_bar, 1);
     for (int s = 0; s < NK; ++s) {
       mbar_init(&k_full[s], 1);
       mbar_init(&k_empty[s], 1);
@@ -148,7 +164,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int crank = static_cast<int>(cluster_ctarank());
   const int row0 = (item / S::kSplit * 2 + crank) * kBM;
   cluster_sync();  // the peer's barriers exist before copies, commits and arrivals reach them
   grid_dep_sync();
@@ -160,7 +175,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       tma_prefetch_desc(&tm_k);
       tma_prefetch_desc(&tm_kr);
       tma_prefetch_desc(&tm_v);
-      auto even = [&](uint64_t* bar) { return dsmem_addr(smem_u32(bar), 0); };
+      auto even = [&](uint64_t* bar) { return dsmem_addr(smem_u32(bar), even_rank); };
       if (crank == 0) mbar_arrive_expect_tx(q_full, 2 * S::kQBytes);
       for (int cb = 1; cb < S::kCBoxes; ++cb)
         tma_load_3d_pair(sQ + (cb - 1) * S::kQBox, &tm_q, even(q_full), cb * 64, row0, b);
@@ -172,7 +187,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (crank == 0) mbar_arrive_expect_tx(&v_full[st], 2 * S::kVTile);
         for (int h = 0; h < 2; ++h)
           tma_load_3d_pair(sV + st * S::kVTile + h * S::kVBox, &tm_v, even(&v_full[st]),
-                           vpart * DV + crank * 128 + h * 64, j * kBN, b);
+                           vpart * DV + crank * 128 + h * 64, (jb0 + j) * kBN, b);
         ++vt;
         return true;
       };
@@ -186,7 +201,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const bool is_c = bx < S::kCBoxes;
           if (crank == 0)
             mbar_arrive_expect_tx(&k_full[st], 2 * (is_c ? S::kKBox : S::kKrBytes));
-          const int key = j * kBN + crank * (kBN / 2);
+          const int key = (jb0 + j) * kBN + crank * (kBN / 2);
           if (is_c)
             tma_load_3d_pair(sK + st * S::kKBox, &tm_k, even(&k_full[st]), bx * 64, key, b);
           else
@@ -210,6 +225,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     __syncwarp();
+    if (p.n_split > 1) {
+      cluster_arrive_release();
+      combine_split_pass();
+    }
   } else if (warp == 1) {
     // -------------------------------------------------------- MMA issuer
     // S_0, S_1, PV_0, S_2, PV_1, ...: PV_{j-1} runs while the softmax warps read
@@ -248,8 +267,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                   umma_pair_ts(tmem, tmem + S::kTmemQ + 32 + k * 8, krd + ko + k * 2,
                                S::kIdescQK, 1u);
               }
-              umma_pair_commit_mc(&k_empty[st], 3);
-              if (bx == S::kBoxes - 1) umma_pair_commit_mc(s_full, 3);
+              umma_pair_commit_mc(&k_empty[st], pair_mask);
+              if (bx == S::kBoxes - 1) umma_pair_commit_mc(s_full, pair_mask);
             }
             __syncwarp();
             if (++st == NK) {
@@ -270,17 +289,21 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int s = 0; s < kBN / 16; ++s)
               umma_pair_ts(tmem + S::kTmemO, tmem + S::kTmemP + s * 8, vd + vo + s * (2048 >> 4),
                            S::kIdescPV, (i > 0 || s > 0) ? 1u : 0u);
-            umma_pair_commit_mc(&v_empty[sv], 3);
-            umma_pair_commit_mc(pv_done, 3);
+            umma_pair_commit_mc(&v_empty[sv], pair_mask);
+            umma_pair_commit_mc(pv_done, pair_mask);
           }
           __syncwarp();
         }
       }
       if (!ok) {  // every MMA this warp issued is done before TMEM is freed
-        if (elect_one()) umma_pair_commit_mc(mma_drain, 1);
+        if (elect_one()) umma_pair_commit_mc(mma_drain, static_cast<uint16_t>(1u << even_rank));
         __syncwarp();
         mbar_wait_drain(mma_drain, 0, p.status);
       }
+    }
+    if (p.n_split > 1) {
+      cluster_arrive_release();
+      combine_split_pass();
     }
   } else {
     // ------------------------------------------------ softmax (warps 2..5)
@@ -289,9 +312,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t t_lane = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
     const int grow = row0 + r;
     const bool row_ok = grow < p.rows;
-    const uint32_t q_ready_even = dsmem_addr(smem_u32(q_ready), 0);
-    const uint32_t s_free_even = dsmem_addr(smem_u32(s_free), 0);
-    const uint32_t p_full_even = dsmem_addr(smem_u32(p_full), 0);
+    const uint32_t q_ready_even = dsmem_addr(smem_u32(q_ready), even_rank);
+    const uint32_t s_free_even = dsmem_addr(smem_u32(s_free), even_rank);
+    const uint32_t p_full_even = dsmem_addr(smem_u32(p_full), even_rank);
     {
       // Q's TMEM part: columns [0, 64) of q_c, then q_r rotated by the query
       // position (RoPE3D); column c of the A operand holds elements 2c, 2c + 1
@@ -366,7 +389,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       float sv[kBN];
 #pragma unroll
       for (int c = 0; c < kBN; ++c) sv[c] = __uint_as_float(sr[c]);
-      const int valid = p.n_valid - j * kBN;
+      const int valid = p.n_valid - (jb0 + j) * kBN;
       if (valid < kBN) {
 #pragma unroll
         for (int c = 0; c < kBN; ++c)
@@ -447,45 +470,54 @@ __global__ void __launch_bounds__(kThreads, 1)
       l_run += ((l8[0] + l8[1]) + (l8[2] + l8[3])) + ((l8[4] + l8[5]) + (l8[6] + l8[7]));
     }
 
-    // O / l as bf16: each thread stages its row densely in the V ring (free
-    // once the last PV is done) and the rows leave by bulk copy, the whole
-    // tile at once when its rows are consecutive rows of o (DV = d_c).
-    const bool have_o = ok && mbar_wait(pv_done, (nblk - 1) & 1, wc);
-    uint8_t* srow = sV + r * DV * 2;
-    if (have_o) {
-      tc_fence_after();
-      const float inv_l = 1.f / l_run;
+    bool have_o = ok && mbar_wait(pv_done, (nblk - 1) & 1, wc);
+    have_o = __all_sync(0xffffffffu, have_o) && !*abort_flag;
+    if (p.n_split > 1) {
+      cluster_arrive_release();  // phase A: the pair's MMAs are done with this CTA's operands
+      combine_split<DV, 128>(smem, smem + kBM * kSplitRecord<DV>, split_bar, tO, part, p.n_split,
+                             crank, 2, kBM, r, have_o, m_run, l_run,
+                             p.o + (static_cast<size_t>(b) * p.rows + row0) * DC + vpart * DV, DC,
+                             p.rows - row0, wc);
+    } else {
+      // O / l as bf16: each thread stages its row densely in the V ring (free
+      // once the last PV is done) and the rows leave by bulk copy, the whole
+      // tile at once when its rows are consecutive rows of o (DV = d_c).
+      uint8_t* srow = sV + r * DV * 2;
+      if (have_o) {
+        tc_fence_after();
+        const float inv_l = 1.f / l_run;
 #pragma unroll 1
-      for (int sg = 0; sg < DV / 64; ++sg) {
-        uint32_t va[32], vb[32];
-        tmem_ld32(tO + sg * 64, va);
-        tmem_ld32(tO + sg * 64 + 32, vb);
-        tmem_wait_ld();
-        uint32_t pk[32];
+        for (int sg = 0; sg < DV / 64; ++sg) {
+          uint32_t va[32], vb[32];
+          tmem_ld32(tO + sg * 64, va);
+          tmem_ld32(tO + sg * 64 + 32, vb);
+          tmem_wait_ld();
+          uint32_t pk[32];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const uint32_t* v = i < 16 ? va : vb;
-          const int q = i & 15;
-          pk[i] = pack_bf16x2(__uint_as_float(v[2 * q]) * inv_l,
-                              __uint_as_float(v[2 * q + 1]) * inv_l);
+          for (int i = 0; i < 32; ++i) {
+            const uint32_t* v = i < 16 ? va : vb;
+            const int q = i & 15;
+            pk[i] = pack_bf16x2(__uint_as_float(v[2 * q]) * inv_l,
+                                __uint_as_float(v[2 * q + 1]) * inv_l);
+          }
+          stage_row<8>(srow + sg * 128, pk, r & 7);
         }
-        stage_row<8>(srow + sg * 128, pk, r & 7);
       }
-    }
-    fence_proxy_async_smem();
-    if constexpr (DV == DC) {
-      asm volatile("bar.sync 1, 128;" ::: "memory");  // the four softmax warps
-      // the tile's rows below p.rows; none in a CTA past an odd last tile
-      const int valid = min(kBM, p.rows - row0);
-      if (r == 0 && have_o && !*abort_flag && valid > 0) {
-        bulk_store(p.o + (static_cast<size_t>(b) * p.rows + row0) * DC, sV, valid * DC * 2);
+      fence_proxy_async_smem();
+      if constexpr (DV == DC) {
+        asm volatile("bar.sync 1, 128;" ::: "memory");  // the four softmax warps
+        // the tile's rows below p.rows; none in a CTA past an odd last tile
+        const int valid = min(kBM, p.rows - row0);
+        if (r == 0 && have_o && !*abort_flag && valid > 0) {
+          bulk_store(p.o + (static_cast<size_t>(b) * p.rows + row0) * DC, sV, valid * DC * 2);
+          bulk_commit();
+          bulk_wait_read_all();  // the staged rows must outlive the copy's reads
+        }
+      } else if (have_o && row_ok) {
+        bulk_store(p.o + (static_cast<size_t>(b) * p.rows + grow) * DC + vpart * DV, srow, DV * 2);
         bulk_commit();
-        bulk_wait_read_all();  // the staged rows must outlive the copy's reads
+        bulk_wait_read_all();
       }
-    } else if (have_o && row_ok) {
-      bulk_store(p.o + (static_cast<size_t>(b) * p.rows + grow) * DC + vpart * DV, srow, DV * 2);
-      bulk_commit();
-      bulk_wait_read_all();
     }
   }
 
@@ -496,6 +528,57 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_after();
     tmem_dealloc_pair(tmem, 512);
   }
+}
+
+template <int DC, int DR>
+cudaLaunchConfig_t wide_config(int items, int batch, int cl, cudaStream_t stream,
+                               cudaLaunchAttribute (&attr)[2]) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(items * cl, batch, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = WideShape<DC, DR>::kSmemBytes;
+  cfg.stream = stream;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cl;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see grid_dep_sync
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cfg;
+}
+
+// Clusters of cl CTAs that are resident at once (0 if the query fails).
+template <int DC, int DR>
+int resident_wide(int cl) {
+  auto kern = mla_attn_wide_tc_kernel<DC, DR>;
+  cudaLaunchAttribute attr[2];
+  const cudaLaunchConfig_t cfg = wide_config<DC, DR>(1, 1, cl, nullptr, attr);
+  int n = 0;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           WideShape<DC, DR>::kSmemBytes) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  return n;
+}
+
+// One pair of CTAs per item (256 rows x 256 output columns), or two pairs that
+// share out its key blocks: the shorter estimate in key blocks, with kFixed for
+// a CTA's start and end (7 us; a block takes 1.1 us at d_c = 256, 1.95 at 512)
+// and `combine` for a split item's combination (3.7-4 us). One against two
+// pairs, d_r = 32: d_c = 256, 3 items: 6 blocks 13.9 / 14.2 us, 8: 16.2 / 15.3;
+// d_c = 512, 6 items: 4 blocks 14.9 / 14.7, 6: 18.8 / 16.7, 42 blocks, 24 items:
+// 89.8 / 53.7; d_c = 256, 81 items (two waves of pairs, three of fours): 94 blocks
+// 229 / 194. Four pairs' records would not fit in shared memory.
+int pick_wide_split(long long items, int nblk, int combine, int res2, int res4) {
+  constexpr long long kFixed = 6;
+  if (res2 < 1 || res4 < 1 || nblk < 2) return 1;
+  const long long t1 = (items + res2 - 1) / res2 * (nblk + kFixed);
+  const long long t2 = (items + res4 - 1) / res4 * ((nblk + 1) / 2 + kFixed + combine);
+  return t2 < t1 ? 2 : 1;
 }
 
 template <int DC, int DR>
@@ -534,21 +617,13 @@ int launch_wide(const AttnArgs& a) {
   kp.pairs_h = a.pairs_h;
   kp.scale_log2 = a.scale_log2;
   kp.status = a.status;
-  const int pairs = (a.rows + 2 * kBM - 1) / (2 * kBM);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * pairs * S::kSplit, a.batch, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = S::kSmemBytes;
-  cfg.stream = a.stream;
+  const int items = (a.rows + 2 * kBM - 1) / (2 * kBM) * S::kSplit;
+  static const int res2 = resident_wide<DC, DR>(2), res4 = resident_wide<DC, DR>(4);
+  kp.n_split = pick_wide_split(static_cast<long long>(items) * a.batch,
+                               (a.n_valid + kBN - 1) / kBN, DC == 512 ? 2 : 3, res2, res4);
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see grid_dep_sync
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  const cudaLaunchConfig_t cfg =
+      wide_config<DC, DR>(items, a.batch, 2 * kp.n_split, a.stream, attr);
   e = cudaLaunchKernelEx(&cfg, kern, tm_q, tm_k, tm_kr, tm_v, kp);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {

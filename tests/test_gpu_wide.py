@@ -1,6 +1,6 @@
 """Attention at d_c = 256 and 512 (paired-SM MMAs over two row tiles) where a
-CTA of the pair has no rows or no keys of its own, and at the edges of tiles,
-key blocks and rings."""
+CTA of the pair has no rows or no keys of its own, at the edges of tiles, key
+blocks and rings, and with the key blocks of a small grid split over two pairs."""
 
 import pytest
 import torch
@@ -29,7 +29,8 @@ def _gpu():
     ((4, 16), 1, 10, 1, 64),    # 64 keys: the odd CTA's half is empty; 120 rows
     ((8, 16), 3, 11, 2, 32),    # whole blocks; the odd CTA has four rows
     ((5, 13), 3, 40, 1, 64),    # 195 keys: the last block ends inside the odd half
-    ((10, 13), 13, 22, 3, 32),  # 14 blocks, more K boxes and V tiles than ring stages
+    ((10, 13), 13, 22, 3, 32),  # 14 blocks in two shares, each longer than the rings
+    ((10, 13), 13, 200, 8, 32),  # the grid fills the SMs: 14 blocks in one piece
 ])
 def test_wide_latent_edges(d_c, grid, frames, nq, batch, d_r):
     w = small(d_c=d_c, d_r=d_r, rope_pairs=(6, 5, 5) if d_r == 32 else (12, 10, 10),
