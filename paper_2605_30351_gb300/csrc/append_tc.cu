@@ -19,14 +19,19 @@
 //              sink frames f * T + k for f < S and (S + (f - S) mod (W - S)) * T
 //              + k after them.
 // For d_c = 512 the [128 x (d_c + d_r)] accumulator does not fit the 512
-// TMEM columns; the launch then runs two CTAs per token tile (blockIdx.z):
-// one accumulates c (two N = 256 MMAs per K step) and applies RMSNorm, the
-// other accumulates k^R and applies RoPE. Both stream the same x tile.
+// TMEM columns; beyond the cluster form the launch then runs two CTAs per token
+// tile (blockIdx.z): one accumulates c (two N = 256 MMAs per K step) and applies
+// RMSNorm, the other accumulates k^R and applies RoPE. Both stream the same x tile.
 // When one CTA per token tile would leave most SMs idle (one chunk at batch
 // 1), a cluster of CTAs shares each token tile, each taking a slice of c's
 // columns (see AppendShape). When the tiles exceed one wave, two CTAs with fewer
 // stages share each SM, so that one's start-up and epilogue overlap the
-// other's K loop.
+// other's K loop. Beyond two waves the CTAs are persistent, and two of them
+// (paired-SM MMAs, M = 256) hold half of the weights' rows each: what sets the
+// pace there is HBM reads, that is bytes of x in flight per SM, and a halved
+// weight tile and an epilogue without staging leave room for 7 stages instead of
+// 3. (Boxes of x prefetched into L2 further ahead only slowed the copies:
+// 48 -> 52 us ten K blocks ahead.)
 #include <cmath>
 
 #include "internal.h"
@@ -64,18 +69,31 @@ constexpr int kPrefetchX2 = 12;
 //    the first), so the CTAs' K loops do not wait on one another; they
 //    exchange their partial RMSNorm sums of squares through distributed
 //    shared memory.
-template <int DC, int DR, int NC, int NK, int CL = 1, int BUDGET = kSmemOne>
+//  - PAIR: one CTA per tile as in the first two, but two CTAs multiply as one
+//    M = 256 MMA with half of the weight rows in each; LOOP: persistent, with
+//    two accumulators.
+template <int DC, int DR, int NC, int NK, int CL = 1, bool PAIR = false, bool LOOP = false,
+          int BUDGET = kSmemOne>
 struct AppendShape {
   static constexpr int N = NC + NK;
   static constexpr bool kSplitN = N > 256;  // then MMAs of at most 256: c part(s), k part
-  static constexpr int kWcBox = NC == 0 ? 64 : (NC < 256 ? NC : 256);  // W_dkv rows per TMA box
+  // PAIR: is every MMA's part of the weights halved ([c parts | k] each), or
+  // [W_dkv ; W_kr] as a whole (the even CTA's half is c alone)?
+  static constexpr bool kHalves = kSplitN || NC == 0;
+  static_assert(!PAIR || CL == 1, "pairs or clusters");
+  static constexpr int kWcRows = NC == 0 ? 64 : (NC < 256 ? NC : 256);
+  // W_dkv rows per TMA box; in the odd CTA of a pair; W_kr rows per box
+  static constexpr int kWcBox = !PAIR ? kWcRows : (kHalves ? kWcRows / 2 : N / 2);
+  static constexpr int wc_odd() { return kHalves ? kWcBox : NC - N / 2; }
+  static constexpr int wk_box() { return PAIR && kHalves ? NK / 2 : NK; }
   static constexpr int kABytes = kBM * kBK * 2;
   // rows of a stage's weight region: in a cluster every CTA takes the widest
   // slice's layout (one shared-memory size for the launch, and the partial
   // sums at the same offset in every CTA)
-  static constexpr int kBRows = CL > 1 ? NC + DR : N;
+  static constexpr int kBRows = CL > 1 ? NC + DR : (PAIR ? N / 2 : N);
   static constexpr int kBBytes = kBRows * kBK * 2;
-  static constexpr int kWTxBytes = N * kBK * 2;  // weight bytes of a K block in this CTA
+  // weight bytes of a K block in this CTA
+  static constexpr int kWTxBytes = (PAIR ? N / 2 : N) * kBK * 2;
   static constexpr int kBlockBytes = kABytes + kBBytes;  // one K block: x, then weights
   static constexpr int kKS = CL > 1 ? 2 : 1;             // K blocks per stage
   static constexpr int kStageBytes = kKS * kBlockBytes;
@@ -86,12 +104,19 @@ struct AppendShape {
   static constexpr int kRedOff = CL > 1 ? (CL * kBM * 4 + 1023) / 1024 * 1024 : 0;
   // this CTA's gamma columns, fetched by the epilogue warps during the K loop
   static constexpr int kGammaBytes = NC * 2;
-  static constexpr int kFit = (BUDGET - 1024 - kBarBytes - kGammaBytes - kRedOff) / kStageBytes;
-  static constexpr int kStages = kFit > 6 ? 6 : kFit;
-  static constexpr int kSmemBytes = 1024 + kRedOff + kStages * kStageBytes + kBarBytes + kGammaBytes;
-  static constexpr uint32_t kTmemCols = N <= 32 ? 32 : (N <= 64 ? 64 : (N <= 256 ? 256 : 512));
-  // output staging: dense c rows, dense k^R rows, then the rows' slots
-  static_assert(kBM * N * 2 + kBM * 8 + 16 <= kStages * kStageBytes, "staging fits in the ring");
+  // output staging in the stage ring (not LOOP): dense c rows, dense k^R rows,
+  // then the words of run breaks
+  static constexpr int kOutBytes = kBM * N * 2 + 16;
+  static constexpr int kFit =
+      (BUDGET - 1024 - kBarBytes - kGammaBytes - kRedOff) / kStageBytes;
+  static constexpr int kStages = kFit > 9 ? 9 : kFit;
+  static constexpr int kSmemBytes =
+      1024 + kRedOff + kStages * kStageBytes + kBarBytes + kGammaBytes;
+  static constexpr int kBufs = LOOP ? 2 : 1;  // accumulators
+  static constexpr int kCols = kBufs * N;
+  static constexpr uint32_t kTmemCols =
+      kCols <= 32 ? 32 : (kCols <= 64 ? 64 : (kCols <= 256 ? 256 : 512));
+  static_assert(LOOP || kOutBytes <= kStages * kStageBytes, "staging fits in the ring");
   static_assert((NC % 64 == 0 || CL > 1) && (NK == 0 || NK == 32 || NK == 64),
                 "staged row segments");
   static_assert(DC % 32 == 0 && DR % 32 == 0 && DR <= 64 && (DC <= 256 || DC % 256 == 0),
@@ -100,7 +125,7 @@ struct AppendShape {
   static_assert((NC == DC && NK == DR && CL == 1) || (DC > 256 && CL == 1) ||
                     (CL >= 2 && CL <= 8 && NC * CL == DC && NC <= 128),
                 "parts are split for d_c > 256, or over a cluster of slices");
-  static_assert(N <= 512, "accumulator must fit in TMEM");
+  static_assert(kCols <= 512, "accumulator must fit in TMEM");
   static_assert(kStageBytes % 1024 == 0 && kWcBox > 0, "swizzle-atom alignment");
   static_assert(kStages >= 2, "smem");
 };
@@ -118,14 +143,18 @@ struct AppendKParams {
   int* status;
   int first_wave;  // CTAs resident at once (a linear block index below it: the first wave)
   int pf_blocks;   // x K blocks a first-wave CTA warms into L2
+  int tiles, batch;  // token tiles of each batch element
 };
 
-// tile: the token tile (128 tokens) of this CTA; c0: its first column of c
-template <int DC, int DR, int NC, int NK, int CL, int BUDGET = kSmemOne>
+// b, tile: the batch element and token tile (128 tokens) of this CTA; c0: its
+// first column of c
+template <int DC, int DR, int NC, int NK, int CL, bool PAIR = false, bool LOOP = false,
+          int BUDGET = kSmemOne>
 __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUtensorMap* tm_wc,
                                             const CUtensorMap* tm_wk, const AppendKParams& p,
-                                            int tile, int c0) {
-  using S = AppendShape<DC, DR, NC, NK, CL, BUDGET>;
+                                            int b, int tile, int c0) {
+  using S = AppendShape<DC, DR, NC, NK, CL, PAIR, LOOP, BUDGET>;
+  constexpr int kBufs = S::kBufs;
   constexpr int NST = S::kStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = align_smem_1024(smem_raw);
@@ -135,14 +164,29 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + NST * S::kStageBytes);
   uint64_t* full = bars;
   uint64_t* empty = bars + NST;
-  uint64_t* acc_full = bars + 2 * NST;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
+  uint64_t* acc_full = bars + 2 * NST;     // [kBufs]
+  uint64_t* acc_empty = acc_full + kBufs;  // [kBufs], LOOP: in the even CTA
+  uint64_t* mma_drain = acc_empty + kBufs;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int b = blockIdx.y;
-  const int row0 = tile * kBM;
+  // LOOP: this CTA's items are blockIdx.x, blockIdx.x + gridDim.x, ...; item i
+  // is tile i % tiles of element i / tiles, and one past the last (an odd
+  // number of tiles) a tile past its element's tokens, all zeros and not stored
+  const int n_items = LOOP ? (p.tiles * p.batch + 1) / 2 * 2 : 1;
+  auto locate = [&](int item) {
+    if constexpr (LOOP) {
+      const bool past = item >= p.tiles * p.batch;
+      b = past ? p.batch - 1 : item / p.tiles;
+      tile = past ? p.tiles : item % p.tiles;
+    }
+    return tile * kBM;  // its first token
+  };
+  const int item0 = LOOP ? static_cast<int>(blockIdx.x) : 0;
+  const int item_step = LOOP ? static_cast<int>(gridDim.x) : 1;
+  int row0 = locate(item0);
   const WaitCtx wc{abort_flag, p.status};
 
   if (warp == 0 && lane == 0) {  // kernel parameters: no need to wait for anyone
@@ -155,19 +199,44 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
       mbar_init(&full[s], S::kProducers);
       mbar_init(&empty[s], 1);
     }
-    mbar_init(acc_full, 1);
+    for (int a = 0; a < kBufs; ++a) {
+      mbar_init(&acc_full[a], 1);
+      if constexpr (LOOP) mbar_init(&acc_empty[a], 8);  // the epilogue warps of both CTAs
+    }
+    mbar_init(mma_drain, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
   if (warp == 1) {
-    tmem_alloc(tmem_slot, S::kTmemCols);
-    tmem_relinquish();
+    if constexpr (PAIR) {
+      tmem_alloc_pair(tmem_slot, S::kTmemCols);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(tmem_slot, S::kTmemCols);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int crank = CL > 1 ? static_cast<int>(cluster_ctarank()) : 0;
+  const int crank = CL > 1 || PAIR ? static_cast<int>(cluster_ctarank()) : 0;
+  // this CTA's weight boxes of K block column kc: f(is_c, first row, row in the
+  // stage's weight region)
+  auto weight_boxes = [&](auto&& f) {
+    if constexpr (!PAIR || S::kHalves) {
+      const int half = PAIR ? crank : 0;
+#pragma unroll
+      for (int h = 0; h < NC / S::kWcRows; ++h)
+        f(true, c0 + h * S::kWcRows + half * S::kWcBox, h * S::kWcBox);
+      if constexpr (NK > 0) f(false, half * S::wk_box(), NC / S::kWcRows * S::kWcBox);
+    } else if (crank == 0) {
+      f(true, 0, 0);
+    } else {
+      if constexpr (S::wc_odd() > 0) f(true, S::kWcBox, 0);
+      f(false, 0, S::wc_odd());
+    }
+  };
   // While the previous kernel in the stream finishes, HBM is mostly idle:
   // a CTA of the first wave warms the first x boxes of its tile (its part of
   // them in a cluster) into L2 then, so that the K loop starts on L2 hits.
@@ -178,20 +247,20 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
   const long long lin =
       blockIdx.x + static_cast<long long>(gridDim.x) * (blockIdx.y + gridDim.y * blockIdx.z);
   const bool first_wave = lin < p.first_wave;
-  if (first_wave && warp == 0 && lane == 0 && crank == 0) {
+  if (first_wave && warp == 0 && lane == 0 && (PAIR || crank == 0)) {
     const int kpf = p.k_blocks < p.pf_blocks ? p.k_blocks : p.pf_blocks;
     for (int kb = 0; kb < kpf; ++kb) tma_prefetch_l2_3d(tm_x, kb * kBK, row0, b);
   }
   if (first_wave && warp == 0 && lane == 1) {
-    const int kb = (tile + static_cast<int>(gridDim.x) * b) % p.k_blocks;
-    if constexpr (NC > 0)
-      for (int h = 0; h < NC / S::kWcBox; ++h)
-        tma_prefetch_l2_2d(tm_wc, kb * kBK, c0 + h * S::kWcBox);
-    if constexpr (NK > 0) tma_prefetch_l2_2d(tm_wk, kb * kBK, 0);
+    const int kb = (PAIR ? static_cast<int>(blockIdx.x / 2)
+                         : tile + static_cast<int>(gridDim.x) * b) % p.k_blocks;
+    weight_boxes([&](bool is_c, int row, int) {
+      tma_prefetch_l2_2d(is_c ? tm_wc : tm_wk, kb * kBK, row);
+    });
   }
   // every CTA of the cluster has started before a peer writes its shared
-  // memory (the partial sums of squares)
-  if constexpr (CL > 1) cluster_sync();
+  // memory (the partial sums of squares; in a pair copies, commits and arrivals)
+  if constexpr (CL > 1 || PAIR) cluster_sync();
   grid_dep_sync();
 
   const int n_stage = (p.k_blocks + S::kKS - 1) / S::kKS;
@@ -202,20 +271,27 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
           S::kKS == 1 ? 1 : min(S::kKS, p.k_blocks - i * S::kKS);
       uint8_t* blk = smem + st * S::kStageBytes;
       const bool do_x = warp == 0, do_w = warp == 6 || S::kProducers == 1;
-      mbar_arrive_expect_tx(&full[st],
-                            kn * ((do_x ? S::kABytes : 0) + (do_w ? S::kWTxBytes : 0)));
+      // a pair's copies are counted in the even CTA, whose warp 1 issues the MMAs
+      if (!PAIR || crank == 0)
+        mbar_arrive_expect_tx(&full[st], (PAIR ? 2 : 1) * kn *
+                                             ((do_x ? S::kABytes : 0) + (do_w ? S::kWTxBytes : 0)));
+      const uint32_t full_even = PAIR ? dsmem_addr(smem_u32(&full[st]), 0) : 0u;
 #pragma unroll
       for (int k = 0; k < S::kKS; ++k) {
         if (k >= kn) break;
         const int kc = (i * S::kKS + k) * kBK;
-        if (do_x) tma_load_3d(blk + k * S::kBlockBytes, tm_x, &full[st], kc, row0, b);
-        if (do_w) {
-          uint8_t* bm = blk + k * S::kBlockBytes + S::kABytes;
-          if constexpr (NC > 0)
-#pragma unroll
-            for (int h = 0; h < NC / S::kWcBox; ++h)
-              tma_load_2d(bm + h * S::kWcBox * 128, tm_wc, &full[st], kc, c0 + h * S::kWcBox);
-          if constexpr (NK > 0) tma_load_2d(bm + NC * 128, tm_wk, &full[st], kc, 0);
+        uint8_t* bm = blk + k * S::kBlockBytes + S::kABytes;
+        if constexpr (PAIR) {
+          tma_load_3d_pair(blk, tm_x, full_even, kc, row0, b);
+          weight_boxes([&](bool is_c, int row, int at) {
+            tma_load_2d_pair(bm + at * 128, is_c ? tm_wc : tm_wk, full_even, kc, row);
+          });
+        } else {
+          if (do_x) tma_load_3d(blk + k * S::kBlockBytes, tm_x, &full[st], kc, row0, b);
+          if (do_w)
+            weight_boxes([&](bool is_c, int row, int at) {
+              tma_load_2d(bm + at * 128, is_c ? tm_wc : tm_wk, &full[st], kc, row);
+            });
         }
       }
     };
@@ -229,14 +305,19 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
         issued = i + 1;
       }
     } else if (lane == 0) {
-      for (int i = 0; i < n_stage; ++i) {
-        const int st = i % NST;
-        if (i >= NST && !mbar_wait(&empty[st], ((i / NST) - 1) & 1, wc)) break;
-        fill(i, st);
-        issued = i + 1;
+      bool ok = true;
+      for (int item = item0; ok && item < n_items; item += item_step) {
+        row0 = locate(item);
+        for (int i = 0; i < n_stage; ++i) {
+          const int st = issued % NST;
+          ok = issued < NST || mbar_wait(&empty[st], ((issued / NST) - 1) & 1, wc);
+          if (!ok) break;
+          fill(i, st);
+          ++issued;
+        }
       }
     }
-    if (*abort_flag && lane == 0)
+    if (*abort_flag && lane == 0 && (!PAIR || crank == 0))  // (a pair's copies: the even CTA)
       for (int u = issued > NST ? issued - NST : 0; u < issued; ++u)
         mbar_wait_drain(&full[u % NST], (u / NST) & 1, p.status);
     __syncwarp();
@@ -249,51 +330,87 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
     bool ok = true;
     bool now = false;  // a poll has seen the next stage
     int st = 0, ph = 0;
+    constexpr int kM = PAIR ? 2 * kBM : kBM;
+    auto mma = [](uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc) {
+      if constexpr (PAIR)
+        umma_pair_ss(d, ad, bd, idesc, acc);
+      else
+        umma_ss(d, ad, bd, idesc, acc);
+    };
     const uint64_t a0 = sdesc(smem_u32(smem), 16, 1024, kSw128);
     const uint64_t b0 = sdesc(smem_u32(smem) + S::kABytes, 16, 1024, kSw128);
-    for (int i = 0; i < n_stage; ++i) {
-      ok = now || mbar_wait_warp(&full[st], ph, wc);
-      if (!ok) break;
-      const int nst = st + 1 == NST ? 0 : st + 1, nph = st + 1 == NST ? ph ^ 1 : ph;
-      // (where the copies set the pace the poll only delays the MMAs)
-      if constexpr (CL > 1) now = __all_sync(0xffffffffu, mbar_test(&full[nst], nph));
-      tc_fence_after();
-      const int kn = S::kKS == 1 ? 1 : min(S::kKS, p.k_blocks - i * S::kKS);
-      if (elect_one()) {
+    int n = 0;  // tiles begun
+    for (int item = item0; ok && (!PAIR || crank == 0) && item < n_items;
+         item += item_step, ++n) {
+      const int buf = LOOP ? n & 1 : 0;
+      if (LOOP && n >= 2) {  // the epilogues of both CTAs have left this accumulator
+        ok = mbar_wait_warp(&acc_empty[buf], ((n >> 1) - 1) & 1, wc);
+        if (!ok) break;
+        tc_fence_after();
+      }
+      const uint32_t acc_tmem = tmem + buf * S::N;
+      for (int i = 0; i < n_stage; ++i) {
+        ok = now || mbar_wait_warp(&full[st], ph, wc);
+        if (!ok) break;
+        const int nst = st + 1 == NST ? 0 : st + 1, nph = st + 1 == NST ? ph ^ 1 : ph;
+        // (where the copies set the pace the poll only delays the MMAs)
+        if constexpr (CL > 1) now = __all_sync(0xffffffffu, mbar_test(&full[nst], nph));
+        tc_fence_after();
+        const int kn = S::kKS == 1 ? 1 : min(S::kKS, p.k_blocks - i * S::kKS);
+        if (elect_one()) {
 #pragma unroll
-        for (int q = 0; q < S::kKS; ++q) {
-          if (q >= kn) break;
-          const uint64_t so =
-              static_cast<uint64_t>((st * S::kStageBytes + q * S::kBlockBytes) >> 4);
+          for (int q = 0; q < S::kKS; ++q) {
+            if (q >= kn) break;
+            const uint64_t so =
+                static_cast<uint64_t>((st * S::kStageBytes + q * S::kBlockBytes) >> 4);
 #pragma unroll
-          for (int k = 0; k < kBK / 16; ++k) {
-            const uint32_t acc = (i | q | k) != 0 ? 1u : 0u;
-            const uint64_t ad = a0 + so + k * 2, bd = b0 + so + k * 2;
-            if constexpr (!S::kSplitN) {
-              constexpr uint32_t idesc = idesc_bf16_f32(kBM, S::N, false, false);
-              umma_ss(tmem, ad, bd, idesc, acc);
-            } else {
-              constexpr int kHc = NC < 256 ? NC : 256;  // columns per c MMA
-              constexpr uint32_t idesc_c = idesc_bf16_f32(kBM, kHc, false, false);
+            for (int k = 0; k < kBK / 16; ++k) {
+              const uint32_t acc = (i | q | k) != 0 ? 1u : 0u;
+              const uint64_t ad = a0 + so + k * 2, bd = b0 + so + k * 2;
+              if constexpr (!S::kSplitN) {
+                constexpr uint32_t idesc = idesc_bf16_f32(kM, S::N, false, false);
+                mma(acc_tmem, ad, bd, idesc, acc);
+              } else {
+                constexpr int kHc = NC < 256 ? NC : 256;  // columns per c MMA
+                constexpr uint32_t idesc_c = idesc_bf16_f32(kM, kHc, false, false);
+                constexpr int kHr = PAIR ? kHc / 2 : kHc;  // their rows in this CTA
 #pragma unroll
-              for (int h = 0; h < NC / kHc; ++h)
-                umma_ss(tmem + h * kHc, ad, bd + ((h * kHc * 128) >> 4), idesc_c, acc);
-              if constexpr (NK > 0) {
-                constexpr uint32_t idesc_k = idesc_bf16_f32(kBM, NK, false, false);
-                umma_ss(tmem + NC, ad, bd + ((NC * 128) >> 4), idesc_k, acc);
+                for (int h = 0; h < NC / kHc; ++h)
+                  mma(acc_tmem + h * kHc, ad, bd + ((h * kHr * 128) >> 4), idesc_c, acc);
+                if constexpr (NK > 0) {
+                  constexpr uint32_t idesc_k = idesc_bf16_f32(kM, NK, false, false);
+                  mma(acc_tmem + NC, ad, bd + ((NC / kHc * kHr * 128) >> 4), idesc_k, acc);
+                }
               }
             }
           }
+          if constexpr (PAIR)
+            umma_pair_commit_mc(&empty[st], 3);
+          else
+            umma_commit(&empty[st]);
         }
-        umma_commit(&empty[st]);
+        __syncwarp();
+        st = nst;
+        ph = nph;
+      }
+      if (elect_one() && ok) {
+        if constexpr (PAIR)
+          umma_pair_commit_mc(&acc_full[buf], 3);
+        else
+          umma_commit(&acc_full[buf]);
       }
       __syncwarp();
-      st = nst;
-      ph = nph;
     }
-    if (elect_one()) umma_commit(acc_full);
-    __syncwarp();
-    if (!ok) mbar_wait_drain(acc_full, 0, p.status);
+    if (!ok) {  // every MMA issued is done before TMEM and the stages are given up
+      if (elect_one()) {
+        if constexpr (PAIR)
+          umma_pair_commit_mc(mma_drain, 1);
+        else
+          umma_commit(mma_drain);
+      }
+      __syncwarp();
+      mbar_wait_drain(mma_drain, 0, p.status);
+    }
     if constexpr (CL > 1) {  // the cluster's second barrier phase
       cluster_arrive_release();
       cluster_wait_acquire();
@@ -302,8 +419,6 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
     const int quarter = warp & 3;
     const int r = quarter * 32 + lane;
     const uint32_t t_row = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
-    const int n = row0 + r;
-    const bool row_ok = n < p.n_tok;
     // What the epilogue reads from global memory is fetched while the MMAs
     // run, so that no load latency follows the accumulator: this CTA's gamma
     // columns into shared memory (read by every row), the row's ring slot
@@ -312,209 +427,269 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
     for (int i = threadIdx.x - 64; i < NC / 8; i += 128)
       gamma_s[i] = p.gamma ? __ldg(reinterpret_cast<const uint4*>(p.gamma + c0) + i)
                            : make_uint4(0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u);
-    const long long f = p.first_frame + n / p.T;
-    const long long slot_n = frame_base_slot(f, p.T, p.W, p.S) + n % p.T;
-    const long long my_slot =
-        row_ok && debug_in_range(slot_n, 0, p.slots, p.status) ? slot_n : -1;
-    // does this row start a run of consecutive slots (row n - 1 not in the
-    // slot just below)? the tile's first row always does
-    bool run_start = my_slot >= 0 && r == 0;
-    if (my_slot >= 0 && r > 0) {
-      const long long f1 = p.first_frame + (n - 1) / p.T;
-      run_start = frame_base_slot(f1, p.T, p.W, p.S) + (n - 1) % p.T != my_slot - 1;
-    }
-    float2 cs[NK > 0 ? NK / 2 : 1];
-    if constexpr (NK > 0) {
-      int pa[3] = {0, 0, 0};
-      if (row_ok && p.rotate) {
-        const int* pp = p.pos + (static_cast<size_t>(b) * p.n_tok + n) * 3;
-        pa[0] = __ldg(pp);
-        pa[1] = __ldg(pp + 1);
-        pa[2] = __ldg(pp + 2);
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-          if (pa[a] < 0 || pa[a] >= p.rope_len) {
-            record_status(p.status, MLA_ERR_RANGE);
-            pa[a] = 0;
-          }
+    int it = 0;
+    for (int item = item0; item < n_items; item += item_step, ++it) {
+      row0 = locate(item);
+      const int buf = LOOP ? it & 1 : 0;
+      const uint32_t t_acc = t_row + buf * S::N;
+      const int n = row0 + r;
+      const bool row_ok = n < p.n_tok;
+      const long long f = p.first_frame + n / p.T;
+      const long long slot_n = frame_base_slot(f, p.T, p.W, p.S) + n % p.T;
+      const long long my_slot =
+          row_ok && debug_in_range(slot_n, 0, p.slots, p.status) ? slot_n : -1;
+      // does this row start a run of consecutive slots (row n - 1 not in the
+      // slot just below)? the tile's first row always does
+      bool run_start = my_slot >= 0 && r == 0;
+      if (my_slot >= 0 && r > 0) {
+        const long long f1 = p.first_frame + (n - 1) / p.T;
+        run_start = frame_base_slot(f1, p.T, p.W, p.S) + (n - 1) % p.T != my_slot - 1;
       }
+      float2 cs[NK > 0 ? NK / 2 : 1];
+      if constexpr (NK > 0) {
+        int pa[3] = {0, 0, 0};
+        if (row_ok && p.rotate) {
+          const int* pp = p.pos + (static_cast<size_t>(b) * p.n_tok + n) * 3;
+          pa[0] = __ldg(pp);
+          pa[1] = __ldg(pp + 1);
+          pa[2] = __ldg(pp + 2);
 #pragma unroll
-      for (int pr = 0; pr < NK / 2; ++pr) {
-        const int ps = pr < p.pairs_t ? pa[0] : (pr < p.pairs_t + p.pairs_h ? pa[1] : pa[2]);
-        cs[pr] = p.rotate ? __ldg(p.rope + static_cast<size_t>(ps) * (DR / 2) + pr)
-                          : make_float2(1.f, 0.f);
-      }
-    }
-    asm volatile("bar.sync 1, 128;" ::: "memory");  // gamma_s is complete
-    const bool have_acc = mbar_wait(acc_full, 0, wc) && !*abort_flag;
-    if constexpr (CL > 1) {
-      // This CTA's columns of c stay in registers between the statistics and
-      // the store, and each thread writes its row's pieces (NC values of c,
-      // d_r values of k^R) straight from registers: a slice's rows are not
-      // contiguous in the cache, and staging them for a coalesced loop took
-      // longer than the whole of this (64 tokens: 8.8 -> 7.3 us, one Wan chunk:
-      // 9.65 -> 8.7 us).
-      uint32_t v[NC];
-      float ss = 0.f;
-      if (have_acc) {
-        tc_fence_after();
+          for (int a = 0; a < 3; ++a)
+            if (pa[a] < 0 || pa[a] >= p.rope_len) {
+              record_status(p.status, MLA_ERR_RANGE);
+              pa[a] = 0;
+            }
+        }
 #pragma unroll
-        for (int cb = 0; cb < NC / 32; ++cb)
-          tmem_ld32(t_row + cb * 32, *reinterpret_cast<uint32_t(*)[32]>(&v[cb * 32]));
-        tmem_wait_ld();
-#pragma unroll
-        for (int i = 0; i < NC; ++i) {
-          const float f = __uint_as_float(v[i]);
-          ss = fmaf(f, f, ss);
+        for (int pr = 0; pr < NK / 2; ++pr) {
+          const int ps = pr < p.pairs_t ? pa[0] : (pr < p.pairs_t + p.pairs_h ? pa[1] : pa[2]);
+          cs[pr] = p.rotate ? __ldg(p.rope + static_cast<size_t>(ps) * (DR / 2) + pr)
+                            : make_float2(1.f, 0.f);
         }
       }
-      // every CTA pushes its row's partial sum into slot [its rank][row] of
-      // every CTA, then all threads of the cluster pass the second barrier
-      // phase (release / acquire), on every path, so that no CTA waits for
-      // one that left; after it the sums are read locally, in rank order
-      const uint32_t local = smem_u32(ss_all + (c0 / NC) * kBM + r);
-      for (int q = 0; q < CL; ++q) dsmem_st_f32(dsmem_addr(local, q), ss);
-      cluster_arrive_release();
-      const bool store = have_acc && my_slot >= 0 && !*abort_flag;
-      const size_t row_id = static_cast<size_t>(b) * p.slots + (my_slot >= 0 ? my_slot : 0);
-      if constexpr (NK > 0) {  // k^R under the barrier: RoPE3D at the token's (t, h, w), or not
-        uint4* dst = reinterpret_cast<uint4*>(p.kr + row_id * DR);
+      // k^R of this row straight from registers: RoPE3D at the token's (t, h, w), or not
+      auto store_kr = [&](bool have_acc, bool store, size_t row_id) {
+        if constexpr (NK > 0) {
+          uint4* dst = reinterpret_cast<uint4*>(p.kr + row_id * DR);
 #pragma unroll
-        for (int cb = 0; cb < NK / 32; ++cb) {
-          uint32_t kv[32], pk[16];
-          if (have_acc) {
-            tmem_ld32(t_row + NC + cb * 32, kv);
-            tmem_wait_ld();
+          for (int cb = 0; cb < NK / 32; ++cb) {
+            uint32_t kv[32], pk[16];
+            if (have_acc) {
+              tmem_ld32(t_acc + NC + cb * 32, kv);
+              tmem_wait_ld();
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const float2 f2 = cs[cb * 16 + i];
+              const float x0 = __uint_as_float(kv[2 * i]), x1 = __uint_as_float(kv[2 * i + 1]);
+              pk[i] = p.rotate ? pack_bf16x2(x0 * f2.x - x1 * f2.y, x0 * f2.y + x1 * f2.x)
+                               : pack_bf16x2(x0, x1);
+            }
+            if (store)
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                dst[cb * 4 + i] =
+                    make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
           }
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const float2 f2 = cs[cb * 16 + i];
-            const float x0 = __uint_as_float(kv[2 * i]), x1 = __uint_as_float(kv[2 * i + 1]);
-            pk[i] = p.rotate ? pack_bf16x2(x0 * f2.x - x1 * f2.y, x0 * f2.y + x1 * f2.x)
-                             : pack_bf16x2(x0, x1);
-          }
-          if (store)
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              dst[cb * 4 + i] =
-                  make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
         }
-      }
-      cluster_wait_acquire();
-      ss = 0.f;
-      for (int q = 0; q < CL; ++q) ss += ss_all[q * kBM + r];
-      if (store) {
-        const float inv = p.use_rmsnorm ? rsqrtf(ss / DC + p.eps) : 1.f;
-        const uint4* g4 = gamma_s;
-        uint4* dst = reinterpret_cast<uint4*>(p.c + row_id * DC + c0);
+      };
+      if (it == 0) asm volatile("bar.sync 1, 128;" ::: "memory");  // gamma_s is complete
+      const bool have_acc =
+          mbar_wait(&acc_full[buf], LOOP ? (it >> 1) & 1 : 0, wc) && !*abort_flag;
+      if constexpr (CL > 1) {
+        // This CTA's columns of c stay in registers between the statistics and
+        // the store, and each thread writes its row's pieces (NC values of c,
+        // d_r values of k^R) straight from registers: a slice's rows are not
+        // contiguous in the cache, and staging them for a coalesced loop took
+        // longer than the whole of this (64 tokens: 8.8 -> 7.3 us, one Wan chunk:
+        // 9.65 -> 8.7 us).
+        uint32_t v[NC];
+        float ss = 0.f;
+        if (have_acc) {
+          tc_fence_after();
 #pragma unroll
-        for (int i = 0; i < NC / 8; ++i) {
-          const uint4 g = g4[i];
-          const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
-          uint32_t w[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            w[q] = pack_bf16x2(__uint_as_float(v[8 * i + 2 * q]) * inv * bf16_lo(gw[q]),
-                               __uint_as_float(v[8 * i + 2 * q + 1]) * inv * bf16_hi(gw[q]));
-          dst[i] = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-      }
-    } else {
-      // Each thread stages its finished bf16 row in shared memory (the stage
-      // ring is free once the accumulator is complete): c rows dense at
-      // stage_c ([128][NC] bf16), k^R rows dense at stage_k ([128][NK]), so that
-      // a run of consecutive slots is one contiguous block in shared memory, as
-      // it is in the cache, and each run leaves by the bulk-copy engine (one copy
-      // for c, one for k^R, one or two runs per tile).
-      uint8_t* stage_c = smem;
-      uint8_t* stage_k = smem + kBM * NC * 2;
-      long long* slot_of = reinterpret_cast<long long*>(smem + kBM * S::N * 2);  // [128]
-      // rows that do not continue a run (run starts and rows past the tokens),
-      // one bit per row, one word per warp
-      uint32_t* run_breaks = reinterpret_cast<uint32_t*>(slot_of + kBM);  // [4]
-      // pass 1: sum of squares of this CTA's c columns (fp32)
-      float ss = 0.f;
-      if (have_acc) {
-        tc_fence_after();
-#pragma unroll 1
-        for (int cb = 0; cb < NC / 32; ++cb) {
-          uint32_t v[32];
-          tmem_ld32(t_row + cb * 32, v);
+          for (int cb = 0; cb < NC / 32; ++cb)
+            tmem_ld32(t_row + cb * 32, *reinterpret_cast<uint32_t(*)[32]>(&v[cb * 32]));
           tmem_wait_ld();
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
+          for (int i = 0; i < NC; ++i) {
             const float f = __uint_as_float(v[i]);
             ss = fmaf(f, f, ss);
           }
         }
-      }
-      const uint32_t breaks = __ballot_sync(0xffffffffu, my_slot < 0 || run_start);
-      if (have_acc) {
-        slot_of[r] = my_slot;
-        if (lane == 0) run_breaks[quarter] = breaks;
-        // positional key first, so that its RoPE factors leave the registers
-        // before pass 2: RoPE3D at the token's (t, h, w), or unrotated
-        if constexpr (NK > 0) {
-          uint32_t pk[NK / 2];
+        // every CTA pushes its row's partial sum into slot [its rank][row] of
+        // every CTA, then all threads of the cluster pass the second barrier
+        // phase (release / acquire), on every path, so that no CTA waits for
+        // one that left; after it the sums are read locally, in rank order
+        const uint32_t local = smem_u32(ss_all + (c0 / NC) * kBM + r);
+        for (int q = 0; q < CL; ++q) dsmem_st_f32(dsmem_addr(local, q), ss);
+        cluster_arrive_release();
+        const bool store = have_acc && my_slot >= 0 && !*abort_flag;
+        const size_t row_id = static_cast<size_t>(b) * p.slots + (my_slot >= 0 ? my_slot : 0);
+        store_kr(have_acc, store, row_id);  // under the barrier
+        cluster_wait_acquire();
+        ss = 0.f;
+        for (int q = 0; q < CL; ++q) ss += ss_all[q * kBM + r];
+        if (store) {
+          const float inv = p.use_rmsnorm ? rsqrtf(ss / DC + p.eps) : 1.f;
+          const uint4* g4 = gamma_s;
+          uint4* dst = reinterpret_cast<uint4*>(p.c + row_id * DC + c0);
 #pragma unroll
-          for (int cb = 0; cb < NK / 32; ++cb) {
+          for (int i = 0; i < NC / 8; ++i) {
+            const uint4 g = g4[i];
+            const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
+            uint32_t w[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              w[q] = pack_bf16x2(__uint_as_float(v[8 * i + 2 * q]) * inv * bf16_lo(gw[q]),
+                                 __uint_as_float(v[8 * i + 2 * q + 1]) * inv * bf16_hi(gw[q]));
+            dst[i] = make_uint4(w[0], w[1], w[2], w[3]);
+          }
+        }
+      } else if constexpr (LOOP) {
+        // Each thread writes its row straight from registers: staging the tile would
+        // take 57 KB from the ring (d_c = 192, one Wan chunk of 16 elements: 47.9 us
+        // with 5 stages left, 51.6 with 4, 56.4 with 3; 46.7 with all 7 and no staging).
+        const bool store = have_acc && my_slot >= 0;
+        const size_t row_id = static_cast<size_t>(b) * p.slots + (my_slot >= 0 ? my_slot : 0);
+        float ss = 0.f;
+        if (have_acc) {
+          tc_fence_after();
+#pragma unroll 1
+          for (int cb = 0; cb < NC / 32; ++cb) {
             uint32_t v[32];
-            tmem_ld32(t_row + NC + cb * 32, v);
+            tmem_ld32(t_acc + cb * 32, v);
             tmem_wait_ld();
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float2 f2 = cs[cb * 16 + i];
-              const float x0 = __uint_as_float(v[2 * i]), x1 = __uint_as_float(v[2 * i + 1]);
-              pk[cb * 16 + i] = p.rotate ? pack_bf16x2(x0 * f2.x - x1 * f2.y, x0 * f2.y + x1 * f2.x)
-                                         : pack_bf16x2(x0, x1);
+            for (int i = 0; i < 32; ++i) {
+              const float f = __uint_as_float(v[i]);
+              ss = fmaf(f, f, ss);
             }
           }
-          stage_row<NK / 8>(stage_k + r * NK * 2, pk, NK == 32 ? (r >> 1) & 3 : r & 7);
         }
-        // pass 2: gamma * c / rms -> bf16, one 64-column (128-byte) segment at a time
-        const float inv = p.use_rmsnorm ? rsqrtf(ss / DC + p.eps) : 1.f;
-        const uint32_t* gamma2 = reinterpret_cast<const uint32_t*>(gamma_s);  // bf16 pairs
+        store_kr(have_acc, store, row_id);
+        if (have_acc) {
+          const float inv = p.use_rmsnorm ? rsqrtf(ss / DC + p.eps) : 1.f;
+          uint4* dst = reinterpret_cast<uint4*>(p.c + row_id * DC);
 #pragma unroll 1
-        for (int sg = 0; sg < NC / 64; ++sg) {
-          uint32_t va[32], vb[32];
-          tmem_ld32(t_row + sg * 64, va);
-          tmem_ld32(t_row + sg * 64 + 32, vb);
-          tmem_wait_ld();
-          uint32_t pk[32];
+          for (int cb = 0; cb < NC / 32; ++cb) {
+            uint32_t v[32];
+            tmem_ld32(t_acc + cb * 32, v);
+            tmem_wait_ld();
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const uint32_t ga = gamma2[sg * 32 + i], gb = gamma2[sg * 32 + 16 + i];
-            pk[i] = pack_bf16x2(__uint_as_float(va[2 * i]) * inv * bf16_lo(ga),
-                                __uint_as_float(va[2 * i + 1]) * inv * bf16_hi(ga));
-            pk[16 + i] = pack_bf16x2(__uint_as_float(vb[2 * i]) * inv * bf16_lo(gb),
-                                     __uint_as_float(vb[2 * i + 1]) * inv * bf16_hi(gb));
+            for (int i = 0; i < 4; ++i) {
+              const uint4 g = gamma_s[cb * 4 + i];
+              const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
+              uint32_t w[4];
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                w[q] = pack_bf16x2(__uint_as_float(v[8 * i + 2 * q]) * inv * bf16_lo(gw[q]),
+                                   __uint_as_float(v[8 * i + 2 * q + 1]) * inv * bf16_hi(gw[q]));
+              if (store) dst[cb * 4 + i] = make_uint4(w[0], w[1], w[2], w[3]);
+            }
           }
-          stage_row<8>(stage_c + r * NC * 2 + sg * 128, pk, r & 7);
         }
-      }
-      // the staged rows reach the async proxy (the bulk copies), then the four
-      // epilogue warps meet; a wait that gave up anywhere shows in abort_flag
-      fence_proxy_async_smem();
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      if (have_acc && !*abort_flag) {
-        // the thread whose row starts a run of consecutive slots copies the
-        // run: c rows to (b * slots + slot) * d_c (+ c0), k^R rows to
-        // (b * slots + slot) * d_r, all 16-byte aligned and sized
-        if (run_start) {
-          int end = kBM;  // the next row that does not continue this run
+        // the accumulator has been read: the tile after the next may take it
+        tc_fence_before();
+        __syncwarp();
+        mbar_arrive_peer_warp(dsmem_addr(smem_u32(&acc_empty[buf]), 0));
+      } else {
+        // Each thread stages its finished bf16 row in shared memory (the stage
+        // ring is free once the accumulator is complete): c rows dense at
+        // stage_c ([128][NC] bf16), k^R rows dense at stage_k ([128][NK]), so that
+        // a run of consecutive slots is one contiguous block in shared memory, as
+        // it is in the cache, and each run leaves by the bulk-copy engine (one copy
+        // for c, one for k^R, one or two runs per tile).
+        uint8_t* stage_c = smem;
+        uint8_t* stage_k = stage_c + kBM * NC * 2;
+        // rows that do not continue a run (run starts and rows past the tokens),
+        // one bit per row, one word per warp
+        uint32_t* run_breaks = reinterpret_cast<uint32_t*>(stage_c + kBM * S::N * 2);  // [4]
+        // pass 1: sum of squares of this CTA's c columns (fp32)
+        float ss = 0.f;
+        if (have_acc) {
+          tc_fence_after();
+#pragma unroll 1
+          for (int cb = 0; cb < NC / 32; ++cb) {
+            uint32_t v[32];
+            tmem_ld32(t_acc + cb * 32, v);
+            tmem_wait_ld();
 #pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            uint32_t m = w < quarter ? 0u : run_breaks[w];
-            if (w == quarter) m &= ~((2u << lane) - 1u);  // rows after this one
-            if (m != 0u && end == kBM) end = w * 32 + __ffs(static_cast<int>(m)) - 1;
+            for (int i = 0; i < 32; ++i) {
+              const float f = __uint_as_float(v[i]);
+              ss = fmaf(f, f, ss);
+            }
           }
-          const int len = end - r;
-          const size_t row_id = static_cast<size_t>(b) * p.slots + my_slot;
-          if constexpr (NC > 0)
-            bulk_store(p.c + row_id * DC + c0, stage_c + r * NC * 2, len * NC * 2);
-          if constexpr (NK > 0) bulk_store(p.kr + row_id * DR, stage_k + r * NK * 2, len * NK * 2);
-          bulk_commit();
-          bulk_wait_read_all();  // the staged rows must outlive the copies' reads
+        }
+        const uint32_t breaks = __ballot_sync(0xffffffffu, my_slot < 0 || run_start);
+        if (have_acc) {
+          if (lane == 0) run_breaks[quarter] = breaks;
+          // positional key first, so that its RoPE factors leave the registers
+          // before pass 2: RoPE3D at the token's (t, h, w), or unrotated
+          if constexpr (NK > 0) {
+            uint32_t pk[NK / 2];
+#pragma unroll
+            for (int cb = 0; cb < NK / 32; ++cb) {
+              uint32_t v[32];
+              tmem_ld32(t_acc + NC + cb * 32, v);
+              tmem_wait_ld();
+#pragma unroll
+              for (int i = 0; i < 16; ++i) {
+                const float2 f2 = cs[cb * 16 + i];
+                const float x0 = __uint_as_float(v[2 * i]), x1 = __uint_as_float(v[2 * i + 1]);
+                pk[cb * 16 + i] = p.rotate
+                                      ? pack_bf16x2(x0 * f2.x - x1 * f2.y, x0 * f2.y + x1 * f2.x)
+                                      : pack_bf16x2(x0, x1);
+              }
+            }
+            stage_row<NK / 8>(stage_k + r * NK * 2, pk, NK == 32 ? (r >> 1) & 3 : r & 7);
+          }
+          // pass 2: gamma * c / rms -> bf16, one 64-column (128-byte) segment at a time
+          const float inv = p.use_rmsnorm ? rsqrtf(ss / DC + p.eps) : 1.f;
+          const uint32_t* gamma2 = reinterpret_cast<const uint32_t*>(gamma_s);  // bf16 pairs
+#pragma unroll 1
+          for (int sg = 0; sg < NC / 64; ++sg) {
+            uint32_t va[32], vb[32];
+            tmem_ld32(t_acc + sg * 64, va);
+            tmem_ld32(t_acc + sg * 64 + 32, vb);
+            tmem_wait_ld();
+            uint32_t pk[32];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const uint32_t ga = gamma2[sg * 32 + i], gb = gamma2[sg * 32 + 16 + i];
+              pk[i] = pack_bf16x2(__uint_as_float(va[2 * i]) * inv * bf16_lo(ga),
+                                  __uint_as_float(va[2 * i + 1]) * inv * bf16_hi(ga));
+              pk[16 + i] = pack_bf16x2(__uint_as_float(vb[2 * i]) * inv * bf16_lo(gb),
+                                       __uint_as_float(vb[2 * i + 1]) * inv * bf16_hi(gb));
+            }
+            stage_row<8>(stage_c + r * NC * 2 + sg * 128, pk, r & 7);
+          }
+        }
+        // the staged rows reach the async proxy (the bulk copies), then the four
+        // epilogue warps meet; a wait that gave up anywhere shows in abort_flag
+        fence_proxy_async_smem();
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        if (have_acc && !*abort_flag) {
+          // the thread whose row starts a run of consecutive slots copies the
+          // run: c rows to (b * slots + slot) * d_c (+ c0), k^R rows to
+          // (b * slots + slot) * d_r, all 16-byte aligned and sized
+          if (run_start) {
+            int end = kBM;  // the next row that does not continue this run
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+              uint32_t m = w < quarter ? 0u : run_breaks[w];
+              if (w == quarter) m &= ~((2u << lane) - 1u);  // rows after this one
+              if (m != 0u && end == kBM) end = w * 32 + __ffs(static_cast<int>(m)) - 1;
+            }
+            const int len = end - r;
+            const size_t row_id = static_cast<size_t>(b) * p.slots + my_slot;
+            if constexpr (NC > 0)
+              bulk_store(p.c + row_id * DC + c0, stage_c + r * NC * 2, len * NC * 2);
+            if constexpr (NK > 0)
+              bulk_store(p.kr + row_id * DR, stage_k + r * NK * 2, len * NK * 2);
+            bulk_commit();
+            bulk_wait_read_all();  // the staged rows must outlive the copies' reads
+          }
         }
       }
     }
@@ -522,9 +697,18 @@ __device__ __forceinline__ void append_body(const CUtensorMap* tm_x, const CUten
 
   tc_fence_before();
   __syncthreads();
+  // both CTAs of a pair are done with its MMAs, barriers and operands (the
+  // output leaves by bulk copies: nothing to release)
+  if constexpr (PAIR) {
+    cluster_arrive_relaxed();
+    cluster_wait_acquire();
+  }
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, S::kTmemCols);
+    if constexpr (PAIR)
+      tmem_dealloc_pair(tmem, S::kTmemCols);
+    else
+      tmem_dealloc(tmem, S::kTmemCols);
   }
 }
 
@@ -533,29 +717,46 @@ __global__ void __launch_bounds__(kThreads, 1)
     mla_append_tc_kernel(const __grid_constant__ CUtensorMap tm_x,
                          const __grid_constant__ CUtensorMap tm_wc,
                          const __grid_constant__ CUtensorMap tm_wk, const AppendKParams p) {
-  append_body<DC, DR, DC, DR, 1>(&tm_x, &tm_wc, &tm_wk, p, blockIdx.x, 0);
+  append_body<DC, DR, DC, DR, 1>(&tm_x, &tm_wc, &tm_wk, p, blockIdx.y, blockIdx.x, 0);
 }
 
-// Grids of more than one wave: two CTAs share each SM (fewer stages each), so
-// that one CTA's start-up and epilogue run under the other's K loop.
+// Two CTAs share each SM (fewer stages each), so that one CTA's start-up and
+// epilogue run under the other's K loop.
 template <int DC, int DR>
 __global__ void __launch_bounds__(kThreads, 2)
     mla_append_tc_kernel_x2(const __grid_constant__ CUtensorMap tm_x,
                             const __grid_constant__ CUtensorMap tm_wc,
                             const __grid_constant__ CUtensorMap tm_wk, const AppendKParams p) {
-  append_body<DC, DR, DC, DR, 1, kSmemHalf>(&tm_x, &tm_wc, &tm_wk, p, blockIdx.x, 0);
+  append_body<DC, DR, DC, DR, 1, false, false, kSmemHalf>(&tm_x, &tm_wc, &tm_wk, p, blockIdx.y,
+                                                          blockIdx.x, 0);
 }
 
-// d_c > 256: blockIdx.z = 0 computes c, 1 computes k^R, for the same tokens
+// Any two consecutive token tiles as a pair of paired MMAs (also the last of one
+// batch element and the first of the next). tm_wo: W_dkv in the odd CTA's box.
+// d_c <= 192: persistent pairs with two accumulators. d_c = 512: blockIdx.z = 0
+// computes c, 1 computes k^R, for the same tokens.
 template <int DC, int DR>
 __global__ void __launch_bounds__(kThreads, 1)
-    mla_append_tc_split_kernel(const __grid_constant__ CUtensorMap tm_x,
-                               const __grid_constant__ CUtensorMap tm_wc,
-                               const __grid_constant__ CUtensorMap tm_wk, const AppendKParams p) {
-  if (blockIdx.z == 0)
-    append_body<DC, DR, DC, 0, 1>(&tm_x, &tm_wc, &tm_wk, p, blockIdx.x, 0);
-  else
-    append_body<DC, DR, 0, DR, 1>(&tm_x, &tm_wc, &tm_wk, p, blockIdx.x, 0);
+    mla_append_tc_pair_kernel(const __grid_constant__ CUtensorMap tm_x,
+                              const __grid_constant__ CUtensorMap tm_wc,
+                              const __grid_constant__ CUtensorMap tm_wk,
+                              const __grid_constant__ CUtensorMap tm_wo, const AppendKParams p) {
+  const CUtensorMap* wc = cluster_ctarank() == 0 ? &tm_wc : &tm_wo;
+  if constexpr (2 * (DC + DR) <= 512) {
+    append_body<DC, DR, DC, DR, 1, true, true>(&tm_x, wc, &tm_wk, p, 0, 0, 0);
+  } else {
+    // an odd last item: a tile past its element's tokens, zeros and not stored
+    const bool past = static_cast<int>(blockIdx.x) >= p.tiles * p.batch;
+    const int b = past ? p.batch - 1 : blockIdx.x / p.tiles;
+    const int tile = past ? p.tiles : blockIdx.x % p.tiles;
+    if constexpr (DC <= 256) {
+      append_body<DC, DR, DC, DR, 1, true>(&tm_x, wc, &tm_wk, p, b, tile, 0);
+    } else if (blockIdx.z == 0) {
+      append_body<DC, DR, DC, 0, 1, true>(&tm_x, wc, &tm_wk, p, b, tile, 0);
+    } else {
+      append_body<DC, DR, 0, DR, 1, true>(&tm_x, wc, &tm_wk, p, b, tile, 0);
+    }
+  }
 }
 
 // Small grids: a cluster of CL CTAs per token tile; rank q computes c columns
@@ -570,28 +771,29 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
   const int q = static_cast<int>(cluster_ctarank());
   const int tile = blockIdx.x / CL;
   if (q < CL - 1)
-    append_body<DC, DR, NC, 0, CL>(&tm_x, &tm_wc, &tm_wk, p, tile, q * NC);
+    append_body<DC, DR, NC, 0, CL>(&tm_x, &tm_wc, &tm_wk, p, blockIdx.y, tile, q * NC);
   else
-    append_body<DC, DR, NC, DR, CL>(&tm_x, &tm_wc, &tm_wk, p, tile, q * NC);
+    append_body<DC, DR, NC, DR, CL>(&tm_x, &tm_wc, &tm_wk, p, blockIdx.y, tile, q * NC);
 }
-
-using KernFn = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, AppendKParams);
 
 // One way to launch an append: the kernel and what it takes.
 struct AppendForm {
-  KernFn kern;
+  const void* kern;
   int smem, threads;
   int cl;        // CTAs per token tile (a cluster), 1: none
   int z;         // grid depth (2: the c and k^R halves of d_c = 512)
   int wc_box;    // W_dkv rows per TMA box
-  int per_sm;    // CTAs per SM
+  int wk_box;    // W_kr rows per box
   int pf_blocks;
+  int wo_box;    // a pair's odd CTA: its W_dkv rows per box (-1: no pairs)
+  int grid;      // persistent pairs: CTAs at most (0: not persistent)
+  int first_wave;
 };
 
 // The cluster form of CL CTAs per tile, when all its clusters fit in `waves`
 // rounds of those that are resident at once.
 template <int DC, int DR, int CL>
-bool cluster_form(long long tiles, AppendForm* f, int waves = 1) {
+bool cluster_form(long long tiles, int sms, AppendForm* f, int waves = 1) {
   using SC0 = AppendShape<DC, DR, DC / CL, 0, CL>;
   using SC1 = AppendShape<DC, DR, DC / CL, DR, CL>;
   constexpr int kSm = SC0::kSmemBytes > SC1::kSmemBytes ? SC0::kSmemBytes : SC1::kSmemBytes;
@@ -618,14 +820,13 @@ bool cluster_form(long long tiles, AppendForm* f, int waves = 1) {
     return n;
   }();
   if (tiles > static_cast<long long>(resident) * waves) return false;
-  *f = {mla_append_tc_cluster_kernel<DC, DR, CL>, kSm, kClusterThreads, CL, 1, SC0::kWcBox, 1,
-        kPrefetchOne};
+  *f = {reinterpret_cast<const void*>(mla_append_tc_cluster_kernel<DC, DR, CL>), kSm,
+        kClusterThreads, CL, 1, SC0::kWcBox, DR, kPrefetchOne, -1, 0, sms};
   return true;
 }
 
 template <int DC, int DR>
 AppendForm pick_form(long long tiles, int sms) {
-  constexpr bool kSplit = DC > 256;
   AppendForm f = {};
   // A cluster per tile when its CTAs all fit in one wave (one Wan chunk at
   // batch 1, d_c = 192: 37 tiles x 3), the larger clusters first: a CTA's K
@@ -637,37 +838,48 @@ AppendForm pick_form(long long tiles, int sms) {
   // 256 15.1 -> 10.2, 512 23.9 -> 18.7; two chunks 13.4 -> 9.3, 12.7 -> 11.3,
   // 16.2 -> 11.9; 128 tokens 11.2 -> 7.4, 11.0 -> 7.9, 11.3 -> 7.7, 22.4 -> 7.9.
   if constexpr (DC == 128) {
-    if (cluster_form<DC, DR, 2>(tiles, &f)) return f;
+    if (cluster_form<DC, DR, 2>(tiles, sms, &f)) return f;
   } else if constexpr (DC == 192) {
-    if (cluster_form<DC, DR, 3>(tiles, &f) || cluster_form<DC, DR, 2>(tiles, &f))
+    if (cluster_form<DC, DR, 3>(tiles, sms, &f) || cluster_form<DC, DR, 2>(tiles, sms, &f))
       return f;
   } else if constexpr (DC == 256) {
-    if (cluster_form<DC, DR, 4>(tiles, &f) || cluster_form<DC, DR, 2>(tiles, &f))
+    if (cluster_form<DC, DR, 4>(tiles, sms, &f) || cluster_form<DC, DR, 2>(tiles, sms, &f))
       return f;
   } else if constexpr (DC == 512) {
-    if (cluster_form<DC, DR, 8>(tiles, &f) || cluster_form<DC, DR, 4>(tiles, &f, 2))
+    if (cluster_form<DC, DR, 8>(tiles, sms, &f) || cluster_form<DC, DR, 4>(tiles, sms, &f, 2))
       return f;
   }
-  // two CTAs per SM when the grid has more than one wave of single CTAs and
-  // two stages of the unsplit form fit in half an SM's shared memory
-  constexpr int kStageX2 = kBM * kBK * 2 + (DC + DR) * kBK * 2;
-  constexpr bool kX2Fits = !kSplit && DC + DR <= 256 &&  // two 256-column TMEM accumulators
-                           (kSmemHalf - 1024 - 256 - DC * 2) / kStageX2 >= 2;
-  if constexpr (kX2Fits) {
-    if (tiles > sms) {
-      using S2 = AppendShape<DC, DR, DC, DR, 1, kSmemHalf>;
-      return {mla_append_tc_kernel_x2<DC, DR>, S2::kSmemBytes, kThreads, 1, 1, S2::kWcBox, 2,
-              kPrefetchX2};
+  // More tiles than clusters take: up to one wave one CTA per tile, up to two
+  // waves two CTAs per SM, then persistent pairs, whose copies run on under the
+  // epilogues and which have no last wave of their own length; d_c = 256 and 512,
+  // of which one accumulator fits in TMEM, pairs of one tile each. Before (two
+  // CTAs per SM from one wave on; no pairs at d_c = 256 and 512) and after, batch
+  // elements of one Wan chunk (37 tiles), d_r = 32: d_c = 192, 9: 44.9 -> 34.3 us,
+  // 12: 48.9 -> 36.8, 16: 52.4 -> 46.7 (248 MB, 5.3 TB/s); d_c = 128, 16: 45.7 ->
+  // 42.4; 64, 16: 42.0 -> 39.8; d_c = 256, 4: 17.9 -> 17.0; 512, 3: 27.4 -> 25.5;
+  // (512, 64), 16: 155 -> 138. Not better up to two waves (two CTAs per SM against
+  // persistent pairs): d_c = 192, 5: 24.6 / 24.3; 128, 5: 19.6 / 21.8; d_c = 64, 160
+  // tiles 12.3 / 17.9. Up to one wave (one CTA per tile against pairs): d_c = 128, 3:
+  // 12.0 / 12.7.
+  constexpr bool kLoop = 2 * (DC + DR) <= 512;  // two accumulators fit in TMEM
+  if constexpr (kLoop) {
+    if (tiles <= sms) {
+      using S = AppendShape<DC, DR, DC, DR>;
+      return {reinterpret_cast<const void*>(mla_append_tc_kernel<DC, DR>), S::kSmemBytes, kThreads,
+              1, 1, S::kWcBox, DR, kPrefetchOne, -1, 0, sms};
+    }
+    if (tiles <= 2ll * sms) {
+      using S = AppendShape<DC, DR, DC, DR, 1, false, false, kSmemHalf>;
+      return {reinterpret_cast<const void*>(mla_append_tc_kernel_x2<DC, DR>), S::kSmemBytes,
+              kThreads, 1, 1, S::kWcBox, DR, kPrefetchX2, -1, 0, 2 * sms};
     }
   }
-  // one CTA per tile, or the c and k^R halves (d_c > 256)
-  using S = AppendShape<DC, DR, DC, kSplit ? 0 : DR>;
-  using SK = AppendShape<DC, DR, kSplit ? 0 : DC, DR>;
+  using S = AppendShape<DC, DR, DC, (DC > 256 ? 0 : DR), 1, true, kLoop>;
+  using SK = AppendShape<DC, DR, (DC > 256 ? 0 : DC), DR, 1, true, kLoop>;
   constexpr int kSm = S::kSmemBytes > SK::kSmemBytes ? S::kSmemBytes : SK::kSmemBytes;
-  if constexpr (kSplit)
-    return {mla_append_tc_split_kernel<DC, DR>, kSm, kThreads, 1, 2, S::kWcBox, 1, kPrefetchOne};
-  else
-    return {mla_append_tc_kernel<DC, DR>, kSm, kThreads, 1, 1, S::kWcBox, 1, kPrefetchOne};
+  return {reinterpret_cast<const void*>(mla_append_tc_pair_kernel<DC, DR>), kSm, kThreads, 1,
+          DC > 256 ? 2 : 1, S::kWcBox, SK::wk_box(), kPrefetchOne, S::wc_odd(),
+          kLoop ? sms / 2 * 2 : 0, sms};
 }
 
 template <int DC, int DR>
@@ -677,14 +889,22 @@ int launch_tc(const AppendArgs& a) {
   if (cudaGetDevice(&dev) == cudaSuccess)
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const AppendForm f = pick_form<DC, DR>(static_cast<long long>(tiles) * a.batch, sms);
-  CUtensorMap tm_x, tm_wc, tm_wk;
+  CUtensorMap tm_x, tm_wc, tm_wk, tm_wo;
   const unsigned long long H = a.hidden, n_tok = a.n_tok;
   if (!encode_map_3d_bf16(&tm_x, a.x, H, n_tok, a.batch, H * 2, n_tok * H * 2, kBK,
                           kBM, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !encode_map_2d_bf16(&tm_wc, a.w_dkv, H, DC, H * 2, kBK, f.wc_box,
                           CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !encode_map_2d_bf16(&tm_wk, a.w_kr, H, DR, H * 2, kBK, DR, CU_TENSOR_MAP_SWIZZLE_128B))
+      !encode_map_2d_bf16(&tm_wk, a.w_kr, H, DR, H * 2, kBK, f.wk_box, CU_TENSOR_MAP_SWIZZLE_128B))
     return MLA_ERR_CUDA;
+  const bool pair = f.wo_box >= 0;
+  if (f.wo_box > 0) {
+    if (!encode_map_2d_bf16(&tm_wo, a.w_dkv, H, DC, H * 2, kBK, f.wo_box,
+                            CU_TENSOR_MAP_SWIZZLE_128B))
+      return MLA_ERR_CUDA;
+  } else {
+    tm_wo = tm_wc;  // not used: the odd CTA's rows are all k^R's, or there are no pairs
+  }
   cudaError_t e = cudaFuncSetAttribute(f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, f.smem);
   if (e != cudaSuccess) {
     set_last_cuda_error(e);
@@ -710,23 +930,31 @@ int launch_tc(const AppendArgs& a) {
   kp.use_rmsnorm = a.use_rmsnorm;
   kp.eps = a.eps;
   kp.status = a.status;
-  kp.first_wave = sms * f.per_sm;
+  kp.tiles = tiles;
+  kp.batch = a.batch;
+  kp.first_wave = f.first_wave;
   kp.pf_blocks = f.pf_blocks;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(tiles * f.cl, a.batch, f.z);
+  long long items = static_cast<long long>(tiles) * a.batch;
+  if (pair) items += items & 1;
+  if (f.grid > 0 && items > f.grid) items = f.grid;
+  cfg.gridDim = pair ? dim3(static_cast<unsigned>(items), 1, f.z)
+                     : dim3(tiles * f.cl, a.batch, f.z);
   cfg.blockDim = dim3(f.threads, 1, 1);
   cfg.dynamicSmemBytes = f.smem;
   cfg.stream = a.stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = f.cl;
+  attr[0].val.clusterDim.x = pair ? 2 : f.cl;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see grid_dep_sync
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  e = cudaLaunchKernelEx(&cfg, f.kern, tm_x, tm_wc, tm_wk, kp);
+  void* args_one[] = {&tm_x, &tm_wc, &tm_wk, &kp};
+  void* args_pair[] = {&tm_x, &tm_wc, &tm_wk, &tm_wo, &kp};
+  e = cudaLaunchKernelExC(&cfg, f.kern, pair ? args_pair : args_one);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_last_cuda_error(e);

@@ -1,6 +1,8 @@
 """The append's cluster forms (a token tile's columns of c over 2, 3, 4 or 8
 CTAs) against the oracle: every cluster size a width picks, clusters in two
-rounds, ragged tiles, and an odd number of K blocks (a short last stage)."""
+rounds, ragged tiles, and an odd number of K blocks (a short last stage). And
+its pairs of tiles: odd numbers of tiles, tiles of two batch elements in a pair,
+fewer and more K blocks than ring stages, one to six rounds per pair."""
 
 import pytest
 import torch
@@ -32,8 +34,16 @@ def _gpu():
     (512, 32, (1, 1), 1, 1536),     # one token: eights
     (512, 64, (8, 8), 30, 1472),    # fours
     (512, 32, (8, 8), 45, 1536),    # fours in two rounds
+    (192, 32, (5, 7), 331, 192),    # persistent pairs: 331 tiles, three K blocks
+    (192, 64, (10, 13), 155, 640),  # 310 tiles, two per element, both accumulators full
+    (128, 32, (10, 13), 201, 64),   # one K block: every tile its own stage
+    (64, 64, (1, 1), 807, 128),     # the odd CTA's weights are k^R alone; six rounds
+    (64, 32, (5, 7), 305, 1536),    # one tile past two waves; the odd CTA has both
+    (256, 32, (8, 8), 153, 1472),   # pairs of one tile each
+    (512, 64, (8, 8), 101, 1536),   # and halves of c and k^R
+    (512, 32, (10, 13), 40, 64),
 ])
-def test_append_cluster_forms(d_c, d_r, grid, batch, hidden):
+def test_append_cluster_and_pair_forms(d_c, d_r, grid, batch, hidden):
     w = small(d_c=d_c, d_r=d_r, rope_pairs=(6, 5, 5) if d_r == 32 else (12, 10, 10),
               rope_axis_dims=(44, 42, 42) if d_r == 32 else (64, 64, 64), grid_h=grid[0],
               grid_w=grid[1], window_frames=3, batch=batch, hidden=hidden)
