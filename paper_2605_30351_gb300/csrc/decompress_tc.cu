@@ -13,21 +13,24 @@
 // Accumulators alternate between two TMEM buffers, so the epilogue of one
 // tile overlaps the MMA of the next. The weights leave L2 once per CTA and c
 // once per column tile, and every output byte is written once; at the Wan
-// window the 201 MB of keys and values written dominate, so the kernel is
-// bound by HBM writes.
+// window the 201 MB of keys and values written dominate. Writing is what bounds
+// the kernel: 53.2 us there at d_c = 192, where a plain fill of as many bytes
+// takes 53.3 (61.5 with a tile's boxes staged and stored by all warps together:
+// every store waited for the slowest warp). d_c = 256: 90.5 -> 67.3 us, with
+// tiles of 128 columns in place of 96 (a third less of c read again).
 //   warp 0     TMA producer (weights once, then c tiles)
 //   warp 1     TMEM allocation; issues tcgen05.mma (M = 128, N = BN)
-//   warps 2-13 epilogue: warps w, w + 4, w + 8 read TMEM lane quarter w % 4
-//              (slot rows), each a third of the columns, into shared staging
-//              as bf16: one [128 slots x 32 columns] box per 32 columns, in
-//              the 64-byte swizzle of the output tensor maps. One thread then
-//              writes the tile with a TMA tensor store per box (a box never
-//              spans two heads: d_nope and head_dim are multiples of 32; slots
-//              past the element's last are clipped by the map). Key tiles
-//              also copy each slot's cached positional key behind every head
-//              that starts in the tile, with 16-byte stores from registers;
-//              those loads are issued before the TMEM reads so their latency
-//              hides.
+//   the others epilogue, each warp by itself: warps w, w + 4, ... read TMEM lane
+//              quarter w % 4 (slot rows), each 64 columns, release the
+//              accumulator and stage them as bf16, [32 slots x 64 columns] in
+//              the swizzle of the output tensor maps; one lane writes them with
+//              a TMA tensor store of 64 columns (values, where heads are whole
+//              64-column boxes) or two of 32 (a box never spans two heads:
+//              d_nope and head_dim are multiples of 32; slots past the
+//              element's last are clipped by the map). Key tiles also copy each
+//              slot's cached positional key behind every head that starts in
+//              the tile, with 16-byte stores from registers; those loads are
+//              issued before the TMEM reads so their latency hides.
 #include "internal.h"
 #include "ptx_sm103.cuh"
 
@@ -35,30 +38,26 @@ namespace vmla {
 namespace {
 
 constexpr int kBM = 128;
-constexpr int kParts = 3;                // epilogue warps per TMEM lane quarter
-constexpr int kEpiWarps = 4 * kParts;
-constexpr int kEpiThreads = 32 * kEpiWarps;
-constexpr int kThreads = 64 + kEpiThreads;
-
 template <int DC>
 struct DecShape {
-  static constexpr int BN = DC <= 192 ? 192 : 96;
+  static constexpr int BN = DC <= 192 ? 192 : 128;
+  static constexpr int kParts = BN / 64;  // epilogue warps per TMEM lane quarter, 64 columns each
+  static constexpr int kEpiWarps = 4 * kParts;
+  static constexpr int kThreads = 64 + 32 * kEpiWarps;
   static constexpr int kChunkBytesC = kBM * 128;  // one [128 x 64] bf16 K-chunk, SW128
   static constexpr int kChunkBytesW = BN * 128;   // one [BN x 64] bf16 K-chunk
   static constexpr int kWBytes = (DC / 64) * kChunkBytesW;
   static constexpr int kCBytes = (DC / 64) * kChunkBytesC;
-  static constexpr int kBoxBytes = kBM * 64;  // one staged [128 slots x 32 columns] box, SW64
+  static constexpr int kWarpStage = 32 * 128;  // a warp's staged 32 slots x 64 columns
   static constexpr int kStageOff = kWBytes + 2 * kCBytes;
-  static constexpr int kBarOff = kStageOff + (BN / 32) * kBoxBytes;
-  // per-row output offsets of the positional-key copies
-  static constexpr int kRowTabOff = kBarOff + 128;             // long long [2][128]
-  static constexpr int kHeadTabOff = kRowTabOff + 2 * kBM * 8;  // long long [BN/8]
+  static constexpr int kBarOff = kStageOff + kEpiWarps * kWarpStage;
+  // output offsets of the heads' positional parts
+  static constexpr int kHeadTabOff = kBarOff + 128;  // long long [BN/8]
   static constexpr int kSmemBytes = 1024 + kHeadTabOff + (BN / 8) * 8;
   static constexpr uint32_t kTmemCols = 2 * BN <= 256 ? 256 : 512;
   static constexpr uint32_t kIdesc = idesc_bf16_f32(kBM, BN, false, false);
   static_assert(DC % 64 == 0 && DC <= 256, "latent width");
-  static_assert(BN % 32 == 0 && BN <= 256 && (BN / 32) % kParts == 0 && BN / 32 <= 2 * kParts,
-                "tile width: whole 32-column boxes, one or two per epilogue warp");
+  static_assert(BN % 64 == 0 && BN <= 256, "whole 64-column parts");
   static_assert(kChunkBytesW % 1024 == 0 && kStageOff % 1024 == 0, "swizzle-atom alignment");
   static_assert(kSmemBytes <= 232448, "shared memory");
 };
@@ -71,26 +70,8 @@ struct DecKParams {
   int* status;
 };
 
-// All epilogue threads agree on one flag (named barrier 1 with an AND).
-__device__ __forceinline__ bool epilogue_all(bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 q, %1, 0;\n\t"
-      "bar.red.and.pred p, 1, %2, q;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(r)
-      : "r"(static_cast<uint32_t>(v)), "n"(kEpiThreads)
-      : "memory");
-  return r != 0;
-}
-
-__device__ __forceinline__ void epilogue_sync() {
-  asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
-}
-
 template <int DC>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(DecShape<DC>::kThreads, 1)
     mla_decompress_tc_kernel(const __grid_constant__ CUtensorMap tm_c,
                              const __grid_constant__ CUtensorMap tm_wk,
                              const __grid_constant__ CUtensorMap tm_wv,
@@ -113,7 +94,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* mma_done = bars + 9;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 10);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  long long* row_base = reinterpret_cast<long long*>(smem + S::kRowTabOff);
   long long* head_off = reinterpret_cast<long long*>(smem + S::kHeadTabOff);
 
   const int warp = threadIdx.x >> 5;
@@ -132,7 +112,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&c_full[s], 1);
       mbar_init(&c_empty[s], 1);
       mbar_init(&acc_full[s], 1);
-      mbar_init(&acc_empty[s], kEpiWarps);  // one arrival per epilogue warp
+      mbar_init(&acc_empty[s], S::kEpiWarps);  // one arrival per epilogue warp
     }
     mbar_init(mma_done, 1);
     *abort_flag = 0;
@@ -205,119 +185,113 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else {
     const int quarter = warp & 3;
     const int part = (warp - 2) >> 2;       // which share of the columns this warp reads
-    const int rl = quarter * 32 + lane;     // slot row of the tile this thread reads
-    const int et = part * kBM + rl;         // index among the epilogue threads
     const uint32_t t_row = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
     const int seg = is_k ? p.dn : p.head_dim;
     const CUtensorMap* tm_out = is_k ? &tm_ko : &tm_vo;
     __nv_bfloat16* out = is_k ? p.k : p.v;
-    const int boxes = n_valid / 32;  // staged 32-column boxes (n_valid is a multiple of 32)
-    constexpr int kPhases = BN / 32 / kParts;  // boxes per epilogue warp: 2 (BN = 192) or 1
+    constexpr int kParts = S::kParts;
+    const int wcol = part * 64;                  // the warp's first column in the tile
+    const bool wide = !is_k && seg % 64 == 0;    // one 64-column store, not two of 32
+    uint8_t* stage_w = stage_out + (warp - 2) * S::kWarpStage;
     // heads whose key rows start in this tile: offsets of their positional part
     int n_heads = 0;
     if (is_k && p.d_r > 0)
       for (int ch = 0; ch < n_valid / 8; ++ch)
         if ((col0 + ch * 8) % seg == 0) {
-          if (et == 0)
+          if (warp == 2 && lane == 0)
             head_off[n_heads] =
                 static_cast<long long>((col0 + ch * 8) / seg) * p.slots * p.head_dim + p.dn;
           ++n_heads;
         }
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * S::kEpiWarps) : "memory");  // head_off is complete
     const int kr_chunks = p.d_r / 8;  // 16-byte pieces of one positional key (<= 8)
     for (int i = 0, r = g; r < p.n_row_tiles; ++i, r += G) {
       const int s = i & 1;
       const int bb = r / p.tiles_per_b;
-      const int sl0 = (r % p.tiles_per_b) * kBM;  // first slot of the tile
-      // positional keys of this tile's slots: piece u = et + 384 k is piece
-      // u % kr_chunks of row u / kr_chunks (coalesced), loaded ahead of use
-      constexpr int kKr = (kBM * 8 + kEpiThreads - 1) / kEpiThreads;
+      // first slot of the tile, and of this warp's 32 rows
+      const int sl0 = (r % p.tiles_per_b) * kBM, slw = sl0 + quarter * 32;
+      // positional keys of the warp's slots, shared with the quarter's other
+      // warps: piece u = lane + 32 (part + kParts k) is piece u % kr_chunks of row
+      // u / kr_chunks (coalesced), loaded ahead of use
+      constexpr int kKr = (8 + kParts - 1) / kParts;
       uint4 krv[kKr];
       if (n_heads > 0) {
 #pragma unroll
         for (int k = 0; k < kKr; ++k) {
-          const int u = et + kEpiThreads * k, row = u / kr_chunks;
-          if (u < kBM * kr_chunks && sl0 + row < p.slots)
+          const int u = lane + 32 * (part + kParts * k), row = u / kr_chunks;
+          if (row < 32 && slw + row < p.slots)
             krv[k] = __ldg(reinterpret_cast<const uint4*>(
-                               p.kr + (static_cast<size_t>(bb) * p.slots + sl0 + row) * p.d_r) +
+                               p.kr + (static_cast<size_t>(bb) * p.slots + slw + row) * p.d_r) +
                            u % kr_chunks);
         }
       }
-      const bool got = mbar_wait(&acc_full[s], (i >> 1) & 1, wc) && !*abort_flag;
-      if (got) tc_fence_after();
-      // row rl of box cb, 64-byte swizzle: 16-byte chunk j at j ^ ((rl >> 1) & 3)
-      const uint32_t sw = static_cast<uint32_t>((rl >> 1) & 3);
-      auto stage_box = [&](int cb) {
-        uint32_t v[32];
-        tmem_ld32(t_row + s * BN + cb * 32, v);
-        tmem_wait_ld();
-        uint8_t* brow = stage_out + cb * S::kBoxBytes + rl * 64;
+      if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[s], (i >> 1) & 1, wc)) || *abort_flag) break;
+      tc_fence_after();
+      uint32_t v[64];
+      tmem_ld32(t_row + s * BN + wcol, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+      tmem_ld32(t_row + s * BN + wcol + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
+      tmem_wait_ld();
+      tc_fence_before();
+      mbar_arrive_warp(&acc_empty[s]);  // the accumulator is in registers
+      uint32_t w[32];
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          *reinterpret_cast<uint4*>(brow + ((j ^ sw) << 4)) =
-              make_uint4(pack_bf16x2(__uint_as_float(v[8 * j]), __uint_as_float(v[8 * j + 1])),
-                         pack_bf16x2(__uint_as_float(v[8 * j + 2]), __uint_as_float(v[8 * j + 3])),
-                         pack_bf16x2(__uint_as_float(v[8 * j + 4]), __uint_as_float(v[8 * j + 5])),
-                         pack_bf16x2(__uint_as_float(v[8 * j + 6]), __uint_as_float(v[8 * j + 7])));
-      };
-      // one tensor store per box: columns col .. col + 31 are columns e .. e + 31
-      // of head h, slots sl0 .. sl0 + 127 of batch element bb
-      auto store_boxes = [&](int bx0, int bx1) {
-        for (int bx = bx0; bx < bx1 && bx < boxes; ++bx) {
-          const int col = col0 + bx * 32;
-          tma_store_3d(tm_out, stage_out + bx * S::kBoxBytes, col % seg, sl0,
-                       bb * p.heads + col / seg);
+      for (int q = 0; q < 32; ++q)
+        w[q] = pack_bf16x2(__uint_as_float(v[2 * q]), __uint_as_float(v[2 * q + 1]));
+      if (lane == 0) bulk_wait_read_all();  // the last tile's stores have read the staging
+      __syncwarp();
+      // row `lane`: 16-byte chunk j at j ^ (lane & 7) of 128 bytes (one box, 128-byte
+      // swizzle), or at j ^ ((lane >> 1) & 3) of 64 bytes (two boxes, 64-byte swizzle)
+      if (wide) {
+        uint8_t* row = stage_w + lane * 128;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          *reinterpret_cast<uint4*>(row + ((j ^ (lane & 7)) << 4)) =
+              make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+      } else {
+        uint8_t* row = stage_w + lane * 64;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          *reinterpret_cast<uint4*>(row + (j >> 2) * 2048 +
+                                    (((j & 3) ^ ((lane >> 1) & 3)) << 4)) =
+              make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+      }
+      fence_proxy_async_smem();  // the staged rows reach the TMA stores
+      __syncwarp();
+      // columns col .. are columns e .. of one head, slots slw .. slw + 31 of
+      // batch element bb (the map clips the last ones)
+      if (lane == 0 && slw < p.slots) {
+        if (wide) {
+          if (wcol < n_valid)
+            tma_store_3d(tm_out, stage_w, (col0 + wcol) % seg, slw,
+                         bb * p.heads + (col0 + wcol) / seg);
+        } else {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int col = col0 + wcol + h * 32;
+            if (wcol + h * 32 < n_valid)
+              tma_store_3d(tm_out, stage_w + h * 2048, col % seg, slw, bb * p.heads + col / seg);
+          }
         }
         bulk_commit();
-      };
-      long long* rbase = row_base + (i & 1) * kBM;  // read by this tile's key copies
-      if (part == 0)  // output offset of slot row rl (batch, head 0, slot), -1 past the last slot
-        rbase[rl] = sl0 + rl < p.slots
-                        ? (static_cast<long long>(bb) * p.heads * p.slots + sl0 + rl) * p.head_dim
-                        : -1ll;
-      if constexpr (kPhases == 1) {
-        if (got) stage_box(part);
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[s]);
-        fence_proxy_async_smem();       // the staged boxes reach the TMA stores
-        if (!epilogue_all(got)) break;  // staged tile complete, or every thread leaves
-        if (et == 0) store_boxes(0, BN / 32);
-      } else {
-        // two phases over the boxes (each part's first box, then its second),
-        // so that one phase's stores read shared memory while the other phase
-        // is staged
-        if (got) stage_box(part);
-        fence_proxy_async_smem();
-        if (et == 0) bulk_wait_read_all();  // the last tile's second-phase boxes are free
-        if (!epilogue_all(got)) break;      // first-phase boxes staged
-        if (et == 0) store_boxes(0, kParts);
-        if (got) stage_box(part + kParts);
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[s]);
-        fence_proxy_async_smem();
-        if (et == 0) bulk_wait_read_all();  // this tile's first-phase boxes are free again
-        epilogue_sync();                    // second-phase boxes staged
-        if (et == 0) store_boxes(kParts, 2 * kParts);
       }
       if (n_heads > 0) {
+        const long long base =
+            (static_cast<long long>(bb) * p.heads * p.slots + slw) * p.head_dim;
 #pragma unroll
         for (int k = 0; k < kKr; ++k) {
-          const int u = et + kEpiThreads * k, row = u / kr_chunks;
-          if (u < kBM * kr_chunks && rbase[row] >= 0)
-            for (int a = 0; a < n_heads; ++a)
-              if (debug_in_range(rbase[row] + head_off[a] + 8 * (u % kr_chunks), 0,
-                                 static_cast<long long>(p.M) * p.heads * p.head_dim - 7, p.status))
-                *reinterpret_cast<uint4*>(out + rbase[row] + head_off[a] + 8 * (u % kr_chunks)) =
-                    krv[k];
+          const int u = lane + 32 * (part + kParts * k), row = u / kr_chunks;
+          if (row < 32 && slw + row < p.slots)
+            for (int a = 0; a < n_heads; ++a) {
+              const long long at = base + static_cast<long long>(row) * p.head_dim + head_off[a] +
+                                   8 * (u % kr_chunks);
+              if (debug_in_range(at, 0, static_cast<long long>(p.M) * p.heads * p.head_dim - 7,
+                                 p.status))
+                *reinterpret_cast<uint4*>(out + at) = krv[k];
+            }
         }
       }
-      if constexpr (kPhases == 1) {
-        if (et == 0) bulk_wait_read_all();  // the stores have read the staged boxes
-        epilogue_sync();                    // staging free for the next tile
-      }
     }
-    if (et == 0) bulk_wait_read_all();
+    if (lane == 0) bulk_wait_read_all();
   }
 
   tc_fence_before();
@@ -335,7 +309,7 @@ int launch_dec(const DecompressArgs& a) {
   const unsigned long long M = static_cast<unsigned long long>(a.batch) * a.slots;
   const int cols_k = a.heads * dn, cols_v = a.heads * a.head_dim;
   CUtensorMap tm_c, tm_wk, tm_wv, tm_ko, tm_vo;
-  // outputs as [batch * heads][slots][head_dim], written in [128 x 32] boxes
+  // outputs as [batch * heads][slots][head_dim], written in [32 x 32] boxes
   const unsigned long long HD = a.head_dim, SL = a.slots;
   if (!encode_map_2d_bf16(&tm_c, a.c, DC, M, DC * 2ull, 64, kBM, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !encode_map_2d_bf16(&tm_wk, a.w_uk, DC, cols_k, DC * 2ull, 64, S::BN,
@@ -343,9 +317,11 @@ int launch_dec(const DecompressArgs& a) {
       !encode_map_2d_bf16(&tm_wv, a.w_uv, DC, cols_v, DC * 2ull, 64, S::BN,
                           CU_TENSOR_MAP_SWIZZLE_128B) ||
       !encode_map_3d_bf16(&tm_ko, a.k, HD, SL, static_cast<unsigned long long>(a.batch) * a.heads,
-                          HD * 2, SL * HD * 2, 32, kBM, CU_TENSOR_MAP_SWIZZLE_64B) ||
+                          HD * 2, SL * HD * 2, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B) ||
       !encode_map_3d_bf16(&tm_vo, a.v, HD, SL, static_cast<unsigned long long>(a.batch) * a.heads,
-                          HD * 2, SL * HD * 2, 32, kBM, CU_TENSOR_MAP_SWIZZLE_64B))
+                          HD * 2, SL * HD * 2, a.head_dim % 64 == 0 ? 64 : 32, 32,
+                          a.head_dim % 64 == 0 ? CU_TENSOR_MAP_SWIZZLE_128B
+                                               : CU_TENSOR_MAP_SWIZZLE_64B))
     return MLA_ERR_CUDA;
   auto kern = mla_decompress_tc_kernel<DC>;
   cudaError_t e =
@@ -378,7 +354,7 @@ int launch_dec(const DecompressArgs& a) {
   int groups = sms / n_col;
   if (groups < 1) groups = 1;
   if (groups > kp.n_row_tiles) groups = kp.n_row_tiles;
-  kern<<<dim3(n_col, groups), kThreads, S::kSmemBytes, a.stream>>>(tm_c, tm_wk, tm_wv, tm_ko,
+  kern<<<dim3(n_col, groups), S::kThreads, S::kSmemBytes, a.stream>>>(tm_c, tm_wk, tm_wv, tm_ko,
                                                                      tm_vo, kp);
   e = cudaGetLastError();
   if (e != cudaSuccess) {

@@ -1,0 +1,48 @@
+"""Decompression where its per-warp stores can go wrong: tiles of columns that end
+inside a warp's 64 (odd heads), heads that are not whole 64-column boxes, slots
+that end inside a warp's 32 rows, more tiles of slots than groups of CTAs."""
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2605_30351_gb300 import synth
+from paper_2605_30351_gb300 import videomla as V
+
+from test_gpu_dense import _decompress, _upload_cache
+from test_gpu_parity import assert_close, f64
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    V.load()
+    V.mla_device_status(clear=True)
+    yield
+    assert V.mla_device_status(clear=True) == V.MLA_OK
+
+
+@pytest.mark.parametrize("d_c,heads,head_dim,grid,frames,batch", [
+    (192, 5, 96, (5, 13), 3, 2),    # values in 32-column boxes; 195 slots
+    (256, 3, 128, (1, 1), 1, 3),    # one slot; the key tiles end after 32 columns
+    (64, 7, 64, (8, 12), 25, 1),    # d_nope = 32; 19 tiles of 128 slots
+    (128, 1, 160, (3, 11), 1, 1),   # 33 slots: one in the second warp's rows
+    (256, 9, 96, (8, 12), 10, 4),   # 32 tiles, each CTA several
+])
+def test_decompress_store_edges(d_c, heads, head_dim, grid, frames, batch):
+    w = synth.workload("tiny", grid_h=grid[0], grid_w=grid[1], window_frames=frames, batch=batch,
+                       d_c=d_c, heads=heads, head_dim=head_dim, rope_pairs=(6, 5, 5),
+                       rope_axis_dims=(head_dim - 2 * (head_dim // 3 // 2 * 2),
+                                       head_dim // 3 // 2 * 2, head_dim // 3 // 2 * 2))
+    wt = synth.draw_layer_weights(w, seed=71)
+    cache, c, _ = _upload_cache(w, 72)
+    k, v = _decompress(w, cache, wt)
+    dn = head_dim - w.d_r
+    assert_close(f64(k[..., :dn]), np.einsum("hec,bjc->bhje", f64(wt["w_uk"]), c), what="k_nope")
+    assert_close(f64(v), np.einsum("hvc,bjc->bhjv", f64(wt["w_uv"]), c), what="v")
+    rope_bits, src = k[..., dn:].cpu().view(torch.int16), cache.kr.cpu().view(torch.int16)
+    for h in range(heads):
+        assert torch.equal(rope_bits[:, h], src)
