@@ -54,9 +54,9 @@ struct GemmShape {
   static constexpr uint32_t kTmemCols = BN <= 128 ? 128 : (BN <= 256 ? 256 : 512);
   static constexpr int kHalves = BN > 256 ? 2 : 1;  // MMAs (and B boxes) per K step
   static constexpr int kBN1 = BN / kHalves;         // columns of one MMA
-  static constexpr int kBBox = PAIR ? BN / 2 : kBN1;  // rows of one B box
+  static constexpr int kBBox = PAIR ? kBN1 / 2 : kBN1;  // rows of one B box
   static constexpr uint32_t kIdesc = idesc_bf16_f32(PAIR ? 2 * kBM : kBM, kBN1, false, false);
-  static_assert(!PAIR || (BN <= 256 && BN % 32 == 0), "paired MMA: one N <= 256 MMA, 16-row B halves");
+  static_assert(!PAIR || kBN1 % 32 == 0, "paired MMA: 16-row B halves");
   static_assert(BN % 32 == 0 && BN <= 512 && kBN1 % 32 == 0, "tile width");
   static_assert(kStageBytes % 1024 == 0, "swizzle-atom alignment");
   static_assert(kBM * BN * 2 <= kStages * kStageBytes, "staging fits in the ring");
@@ -153,8 +153,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (q >= kn) break;
             uint8_t* a = smem + st * S::kStageBytes + q * S::kBlockBytes;
             tma_load_2d_pair(a, &tm_a, bar, (i * KS + q) * kBK, m0);
-            tma_load_2d_pair(a + S::kABytes, &tm_b, bar, (i * KS + q) * kBK,
-                             n0 + crank * S::kBBox);
+#pragma unroll
+            for (int h = 0; h < S::kHalves; ++h)
+              tma_load_2d_pair(a + S::kABytes + h * S::kBBox * 128, &tm_b, bar,
+                               (i * KS + q) * kBK, n0 + h * S::kBN1 + crank * S::kBBox);
           }
         } else {
           mbar_arrive_expect_tx(&full[st], kn * S::kTxBytes);
@@ -204,13 +206,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int k = 0; k < kBK / 16; ++k) {
               const uint32_t acc = (i | q | k) != 0 ? 1u : 0u;
-              if constexpr (PAIR) {
-                umma_pair_ss(tmem, ad + so + k * 2, bd + so + k * 2, S::kIdesc, acc);
-              } else {
 #pragma unroll
-                for (int h = 0; h < S::kHalves; ++h)
-                  umma_ss(tmem + h * S::kBN1, ad + so + k * 2,
-                          bd + so + ((h * S::kBN1 * 128) >> 4) + k * 2, S::kIdesc, acc);
+              for (int h = 0; h < S::kHalves; ++h) {
+                const uint64_t b = bd + so + ((h * S::kBBox * 128) >> 4) + k * 2;
+                if constexpr (PAIR)
+                  umma_pair_ss(tmem + h * S::kBN1, ad + so + k * 2, b, S::kIdesc, acc);
+                else
+                  umma_ss(tmem + h * S::kBN1, ad + so + k * 2, b, S::kIdesc, acc);
               }
             }
           }
@@ -868,15 +870,32 @@ int launch_output_projection(const OutProjArgs& a) {
   // (64 tokens 18.5 -> 8.4 us, 900 19.1 -> 10.2)
   const int K = a.heads * a.d_c;
   auto fits = [&](int bn) { return row_tiles * ((a.hidden + bn - 1) / bn) <= sms; };
+  // Paired-SM MMAs halve B's part of that; starting and ending together costs a
+  // pair ~0.5 us, so the K loop has to be long enough. Unpaired against paired,
+  // 12 heads, at K = 768 / 1536 / 2304 / 3072 / 6144 us: 128-wide 5.96, 6.24 / 8.21,
+  // 8.0 / 10.5, 9.75 / - / 24.4, 20.8; 192-wide 6.67, 7.16 / 9.21, 9.59 / 12.9, 12.8 /
+  // 16.2, 15.8 / 27.6, 26.1; 256-wide 7.82, 8.23 / 11.3, 11.7 / 16.0, 15.4; 384-wide
+  // 11.0, 11.3 / 18.1, 17.3 / 24.1, 22.0 (one Wan chunk) / - / 53.2, 46.8.
+  const long long pair_rows = (row_tiles + 1) / 2 * 2;
+  auto pairs = [&](int bn, int min_k) {
+    return K >= min_k && row_tiles > 1 && pair_rows * ((a.hidden + bn - 1) / bn) <= sms;
+  };
   if (fits(64))
     return launch_gemm<64, kStore, 6, false, 2>(a.o_lat, a.w_b, a.rows, a.hidden, K, k, a.stream);
+  if (pairs(128, 1536))
+    return launch_gemm<128, kStore, 6, true, 2>(a.o_lat, a.w_b, a.rows, a.hidden, K, k, a.stream);
   if (fits(128))
     return launch_gemm<128, kStore, 6, false, 2>(a.o_lat, a.w_b, a.rows, a.hidden, K, k, a.stream);
+  if (pairs(192, 3072))
+    return launch_gemm<192, kStore, 6, true>(a.o_lat, a.w_b, a.rows, a.hidden, K, k, a.stream);
   if (fits(192)) return launch_gemm<192, kStore>(a.o_lat, a.w_b, a.rows, a.hidden, K, k, a.stream);
+  if (pairs(256, 2304))
+    return launch_gemm<256, kStore, 6, true>(a.o_lat, a.w_b, a.rows, a.hidden, K, k, a.stream);
   if (fits(256)) return launch_gemm<256, kStore>(a.o_lat, a.w_b, a.rows, a.hidden, K, k, a.stream);
+  if (a.hidden % 384 == 0 && pairs(384, 1536))
+    return launch_gemm<384, kStore, 6, true>(a.o_lat, a.w_b, a.rows, a.hidden, K, k, a.stream);
   if (a.hidden % 384 == 0 && row_tiles * (a.hidden / 384) <= sms)
-    return launch_gemm<384, kStore, 3>(a.o_lat, a.w_b, a.rows, a.hidden, a.heads * a.d_c, k,
-                                       a.stream);
+    return launch_gemm<384, kStore, 3>(a.o_lat, a.w_b, a.rows, a.hidden, K, k, a.stream);
   const long long ctas256 = row_tiles * ((a.hidden + 255) / 256);
   if (ctas256 < 2ll * sms && a.hidden % 192 == 0)
     return launch_gemm<192, kStore, 2>(a.o_lat, a.w_b, a.rows, a.hidden, a.heads * a.d_c, k,

@@ -62,6 +62,10 @@ def test_query_prologue_forms(nq, d_q, d_c, d_r, hidden):
     (2400, 64, 1472),   # 192-wide, its last tile ragged; 19 row tiles
     (3000, 128, 1536),  # 256-wide, 24 row tiles
     (4000, 64, 1536),   # 384-wide
+    (1100, 192, 1472),  # 128-wide pairs: nine row tiles, the last pair's second is past the rows
+    (2300, 256, 1472),  # 192-wide pairs, the last tile ragged
+    (2500, 192, 1472),  # 256-wide pairs, the last tile ragged
+    (4700, 128, 1536),  # 384-wide pairs, 37 row tiles
 ])
 def test_output_projection_forms(nq, d_c, hidden):
     w = small(d_c=d_c, hidden=hidden)
